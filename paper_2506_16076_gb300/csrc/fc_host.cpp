@@ -10,10 +10,13 @@
 #include <cstring>
 #include <functional>
 #include <map>
+#include <memory>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "fc_internal.h"
+#include "fc_mmtab.h"
 #include "fc_tables.h"
 
 using namespace fcx;
@@ -99,12 +102,16 @@ struct fc_ctx {
   // FFT plans as uploaded and, per plan, the stage orders the autotuner may choose from
   std::vector<Plan> plans_h;
   std::vector<std::vector<Plan>> plan_cands;
+  std::vector<MmPlan> mm_h;
   double tune_report[6] = {0, 0, 0, 0, 0, 0};
   Job* d_tune_jobs = nullptr;  // the autotuner's timing batch (allocated on first use)
 
   // device tables
   std::vector<void*> allocs;
   DevTables T{};
+  MmPlan* d_mm = nullptr;
+  uint4* d_mmlo = nullptr;
+  uint2* d_mmhi = nullptr;
   Plan* d_plans = nullptr;
   double2* d_tw = nullptr;
   double* d_rp = nullptr;
@@ -125,6 +132,12 @@ struct fc_ctx {
     Job* dpp = nullptr;                          // per-patch order
     std::vector<int> pbeg, pend, plmax;
     std::vector<Job> h;                          // host copy of the batched order
+    // tensor-core contractions of the lines whose length allows them (tiles of MM_LINES
+    // lines of one patch and plan), batched by padded length and per patch; rest: the
+    // other lines, for the FFT kernels
+    std::vector<MmTiles> mm;
+    std::vector<std::vector<MmTiles>> mmpp;
+    std::unique_ptr<Queue> rest;
   };
   Queue q_cart1, q_cart2, q_gen1, q_gen2, q_filt1, q_filt2;
   int* d_fix = nullptr;
@@ -853,6 +866,9 @@ struct Builder {
   std::vector<int> ip;
   std::map<int, int> fcm_of_C;
 
+  std::vector<MmPlan> mm;  // per plan: its tensor-core contraction (H = 0: none)
+  std::vector<uint4> mmlo;
+  std::vector<uint2> mmhi;
   std::vector<std::vector<Plan>> cands;  // per plan: stage orders for the autotuner, [0] = plans[i]
 
   // slot -> mode table of an in-place transform with p's stage order, appended to the int pool:
@@ -901,14 +917,18 @@ struct Builder {
     rev_table(p);
     p.sig = (int)rp.size();
     const fc_params& prm = c->prm;
+    std::vector<long double> sig;
     for (int t = 0; t < L; ++t) {
       long double k = (2 * t <= L) ? t : t - L;
       if (2 * t == L) k = L / 2.0L;
       const long double z = 2.0L * k / (long double)L;
-      rp.push_back((double)(expl(-(long double)prm.alpha_f * powl(z, prm.p_f)) / (long double)L));
+      const long double v = expl(-(long double)prm.alpha_f * powl(z, prm.p_f));
+      rp.push_back((double)(v / (long double)L));
+      if (2 * t <= L) sig.push_back(v);
     }
     fma_tables(p);
     plans.push_back(p);
+    mm.push_back(mm_length_ok(L) ? mm_plan(L, &sig, mmlo, mmhi) : MmPlan{});
     std::vector<Plan> alt{p};
     for (size_t o = 1; o < orders.size(); ++o) {
       if ((int)orders[o].size() > MAXST) continue;
@@ -967,7 +987,88 @@ struct Builder {
 };
 
 void make_queue(fc_ctx* c, fc_ctx::Queue& q, std::vector<Job>& jobs, const std::vector<Plan>& plans, int npatch,
-                bool& ok) {
+                bool& ok, const std::vector<MmPlan>* mm);
+
+// Tiles of the contraction kernels from a queue's per-patch order pp; the lines of other
+// lengths go to q.rest. Launch classes by padded inner length: the shared memory of a CTA
+// grows with it, so a class has the lengths that let the same number of CTAs share an SM.
+void make_tiles(fc_ctx* c, fc_ctx::Queue& q, const std::vector<Job>& pp, const std::vector<Plan>& plans, int npatch,
+                bool& ok, const std::vector<MmPlan>& mm) {
+  struct Tile {
+    Job j[MM_LINES];
+    int patch, kp, two, cls;
+  };
+  static const int top[] = {48, 64, 96, 128, 176, 208, MM_KMAX};
+  std::vector<Tile> tiles;
+  std::vector<Job> rest;
+  for (const Job& J : pp) {
+    const MmPlan& m = mm[J.plan];
+    if (m.H == 0 || J.C > 128 || c->d > 8) {
+      rest.push_back(J);
+      continue;
+    }
+    if (!tiles.empty()) {
+      Tile& t = tiles.back();
+      const Job& A = t.j[0];
+      int nl = 1;
+      while (nl < MM_LINES && t.j[nl].n > 0) ++nl;
+      if (nl < MM_LINES && t.patch == J.patch && A.plan == J.plan && A.n == J.n && A.C == J.C && A.fcm == J.fcm) {
+        t.j[nl] = J;
+        continue;
+      }
+    }
+    Tile t{};
+    t.j[0] = J;
+    t.patch = J.patch;
+    t.kp = m.Kp;
+    t.two = m.S == 2;
+    while (top[t.cls] < t.kp) ++t.cls;
+    tiles.push_back(t);
+  }
+  for (Tile& t : tiles)  // absent lines share the plan (the kernel reads it from the first)
+    for (int l = 1; l < MM_LINES; ++l)
+      if (t.j[l].n == 0) t.j[l].plan = t.j[0].plan;
+  auto put = [&](const std::vector<Tile>& ts, std::vector<MmTiles>& out, std::vector<Job>& flat) {
+    for (size_t k = 0; k < ts.size();) {
+      size_t e = k;
+      MmTiles m{nullptr, 0, 0, ts[k].two};
+      while (e < ts.size() && ts[e].cls == ts[k].cls && ts[e].two == ts[k].two) {
+        m.kp = std::max(m.kp, ts[e].kp);
+        ++e;
+      }
+      m.n = (int)(e - k);
+      m.jobs = (const Job*)(uintptr_t)flat.size();  // index until the upload
+      for (size_t i = k; i < e; ++i) flat.insert(flat.end(), ts[i].j, ts[i].j + MM_LINES);
+      out.push_back(m);
+      k = e;
+    }
+  };
+  std::vector<Job> flat;
+  q.mm.clear();
+  q.mmpp.assign(npatch, {});
+  for (size_t k = 0; k < tiles.size();) {  // per patch
+    std::vector<Tile> ts;
+    const int p = tiles[k].patch;
+    while (k < tiles.size() && tiles[k].patch == p) ts.push_back(tiles[k++]);
+    std::stable_sort(ts.begin(), ts.end(), [](const Tile& a, const Tile& b) { return a.kp > b.kp; });
+    put(ts, q.mmpp[p], flat);
+  }
+  std::stable_sort(tiles.begin(), tiles.end(), [](const Tile& a, const Tile& b) {
+    return a.cls != b.cls ? a.cls > b.cls : (a.two != b.two ? a.two > b.two : a.kp > b.kp);
+  });
+  put(tiles, q.mm, flat);
+  Job* d = nullptr;
+  ok = ok && c->upload(&d, flat);
+  auto fix = [&](MmTiles& m) { m.jobs = d + (uintptr_t)m.jobs; };
+  for (MmTiles& m : q.mm) fix(m);
+  for (auto& v : q.mmpp)
+    for (MmTiles& m : v) fix(m);
+  q.rest = std::make_unique<fc_ctx::Queue>();
+  make_queue(c, *q.rest, rest, plans, npatch, ok, nullptr);
+}
+
+void make_queue(fc_ctx* c, fc_ctx::Queue& q, std::vector<Job>& jobs, const std::vector<Plan>& plans, int npatch,
+                bool& ok, const std::vector<MmPlan>* mm) {
   // per-patch order: stable by patch
   std::vector<Job> pp = jobs;
   std::stable_sort(pp.begin(), pp.end(), [](const Job& a, const Job& b) { return a.patch < b.patch; });
@@ -999,6 +1100,7 @@ void make_queue(fc_ctx* c, fc_ctx::Queue& q, std::vector<Job>& jobs, const std::
   }
   ok = ok && c->upload(&q.d, jobs) && c->upload(&q.dpp, pp);
   q.h = jobs;
+  if (mm) make_tiles(c, q, pp, plans, npatch, ok, *mm);
 }
 
 }  // namespace
@@ -1550,12 +1652,12 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
 
   // ---- upload
   bool ok = true;
-  make_queue(c, c->q_cart1, jc1, B.plans, npatch, ok);
-  make_queue(c, c->q_cart2, jc2, B.plans, npatch, ok);
-  make_queue(c, c->q_gen1, jg1, B.plans, npatch, ok);
-  make_queue(c, c->q_gen2, jg2, B.plans, npatch, ok);
-  make_queue(c, c->q_filt1, jf1, B.plans, npatch, ok);
-  make_queue(c, c->q_filt2, jf2, B.plans, npatch, ok);
+  make_queue(c, c->q_cart1, jc1, B.plans, npatch, ok, &B.mm);
+  make_queue(c, c->q_cart2, jc2, B.plans, npatch, ok, &B.mm);
+  make_queue(c, c->q_gen1, jg1, B.plans, npatch, ok, nullptr);
+  make_queue(c, c->q_gen2, jg2, B.plans, npatch, ok, nullptr);
+  make_queue(c, c->q_filt1, jf1, B.plans, npatch, ok, &B.mm);
+  make_queue(c, c->q_filt2, jf2, B.plans, npatch, ok, &B.mm);
   std::vector<PatchDev> pdev(npatch);
   bool any_pform = false;
   for (int p = 0; p < npatch; ++p) {
@@ -1575,7 +1677,8 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   std::vector<Recv> rinterp;
   std::vector<PtCopy> rcopy;
   split_exchange(recv, rinterp, rcopy);
-  ok = ok && c->upload(&c->d_plans, B.plans) && c->upload(&c->d_tw, B.tw) && c->upload(&c->d_rp, B.rp) &&
+  ok = ok && c->upload(&c->d_mm, B.mm) && c->upload(&c->d_mmlo, B.mmlo) && c->upload(&c->d_mmhi, B.mmhi) &&
+       c->upload(&c->d_plans, B.plans) && c->upload(&c->d_tw, B.tw) && c->upload(&c->d_rp, B.rp) &&
        c->upload(&c->d_ip, B.ip) &&
        c->upload(&c->d_info, info) && c->upload(&c->d_patches, pdev) && c->upload(&c->d_J, Jm) &&
        c->upload(&c->d_sdnn, c->sdnn) && c->upload(&c->d_R, Rv) && c->upload(&c->d_wtab, wtab) &&
@@ -1588,6 +1691,7 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
        c->upload(&c->d_wall, wall) && c->upload(&c->d_wallw, wallw) && c->upload(&c->d_wallc, wallc);
   c->plans_h = B.plans;
   c->plan_cands = B.cands;
+  c->mm_h = B.mm;
   c->h_recv = recv;
   c->h_bc = bcs;
   c->h_walls = walls;
@@ -1635,6 +1739,9 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   T.rp = c->d_rp;
   T.ip = c->d_ip;
   T.plans = c->d_plans;
+  T.mm = c->d_mm;
+  T.mmlo = c->d_mmlo;
+  T.mmhi = c->d_mmhi;
   T.info = c->d_info;
   T.patches = c->d_patches;
   T.npatch = npatch;
@@ -1644,6 +1751,7 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   T.d = prm->d;
   T.any_pform = any_pform ? 1 : 0;
   set_kernel_attributes();
+  set_mm_attributes();
   if (!mpts.empty()) {  // metrics of GRID patches given by their points only
     std::vector<double> xy(2 * (size_t)c->P, 0.0);
     for (const HPatch& h : c->hp)
@@ -1744,24 +1852,36 @@ struct Prof {
 // stream this pass may use (a chain already running on a side stream keeps it). While
 // the per-pass profile is on, passes run one after another so that each pass's time is
 // its own.
-template <class F>
-void run_queue(fc_ctx* c, const fc_ctx::Queue& q, bool per_patch, cudaStream_t st, const char* name, F&& launch,
-               int first_side = 1) {
-  if (q.n == 0) return;
+struct NoMm {
+  void operator()(const MmTiles&, cudaStream_t) const {}
+};
+// launch_mm: the contraction kernel for the queue's tiles (launch then takes the remaining
+// lines); NoMm: every line goes through launch
+template <class F, class G = NoMm>
+void run_queue(fc_ctx* c, const fc_ctx::Queue& q0, bool per_patch, cudaStream_t st, const char* name, F&& launch,
+               int first_side = 1, G&& launch_mm = G{}) {
+  if (q0.n == 0) return;
+  constexpr bool with_mm = !std::is_same<typename std::decay<G>::type, NoMm>::value;
+  const fc_ctx::Queue& q = with_mm ? *q0.rest : q0;
   Prof pr(c, st, name);
   if (!per_patch) {
-    const int ncls = (int)q.classes.size();
+    const int nmm = with_mm ? (int)q0.mm.size() : 0;
+    const int ncls = nmm + (int)q.classes.size();
     const int nside = fc_ctx::NSIDE - first_side;
     const bool fork = c->concurrent && !c->prof && ncls > 1 && nside > 0 && c->ensure_side();
     if (fork) cudaEventRecord(c->fork_ev[0], st);
     for (int k = 0; k < ncls; ++k) {
-      const int b = q.classes[k].first, e = q.class_end[k];
       cudaStream_t s = st;
       if (fork && k > 0) {
         s = c->side[first_side + (k - 1) % nside];
         if (k - 1 < nside) cudaStreamWaitEvent(s, c->fork_ev[0], 0);
       }
-      launch(q.d + b, e - b, q.classes[k].second, s);
+      if (k < nmm) {
+        launch_mm(q0.mm[k], s);
+      } else {
+        const int b = q.classes[k - nmm].first, e = q.class_end[k - nmm];
+        launch(q.d + b, e - b, q.classes[k - nmm].second, s);
+      }
       c->launches++;
     }
     if (fork)
@@ -1771,6 +1891,11 @@ void run_queue(fc_ctx* c, const fc_ctx::Queue& q, bool per_patch, cudaStream_t s
       }
   } else {
     for (size_t p = 0; p < q.pbeg.size(); ++p) {
+      if (with_mm)
+        for (const MmTiles& m : q0.mmpp[p]) {
+          launch_mm(m, st);
+          c->launches++;
+        }
       const int n = q.pend[p] - q.pbeg[p];
       if (n <= 0) continue;
       launch(q.dpp + q.pbeg[p], n, q.plmax[p], st);
@@ -1804,14 +1929,17 @@ void stage(fc_ctx* c, const StageCoef& sc, const double* mu, bool per_patch, cud
     launch_flux_y_points(T, c->d_fyfix, c->nfyfix, e, c->d_Fy, st);
     c->launches++;
   }
-  run_queue(c, c->q_cart1, per_patch, st, "cart_q1", [&](const Job* j, int n, int L, cudaStream_t s) {
-    launch_cart_q1(T, j, n, L, e, mu, c->d_R1, c->d_Fy, s);
-  });
+  run_queue(
+      c, c->q_cart1, per_patch, st, "cart_q1",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_cart_q1(T, j, n, L, e, mu, c->d_R1, c->d_Fy, s); }, 1,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_cart_q1(T, t, e, mu, c->d_R1, c->d_Fy, s); });
   run_queue(c, c->q_gen2, per_patch, sg, "gen_B",
             [&](const Job* j, int n, int L, cudaStream_t s) { launch_gen_B(T, j, n, L, e, mu, c->d_J, c->d_G, s); },
             gside);
-  run_queue(c, c->q_cart2, per_patch, st, "cart_q2",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_cart_q2(T, j, n, L, mu, c->d_R1, c->d_Fy, sc, s); });
+  run_queue(
+      c, c->q_cart2, per_patch, st, "cart_q2",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_cart_q2(T, j, n, L, mu, c->d_R1, c->d_Fy, sc, s); }, 1,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_cart_q2(T, t, mu, c->d_R1, c->d_Fy, sc, s); });
   run_queue(c, c->q_gen1, per_patch, sg, "gen_C",
             [&](const Job* j, int n, int L, cudaStream_t s) { launch_gen_C(T, j, n, L, c->d_J, c->d_G, sc, s); },
             gside);
@@ -1876,14 +2004,18 @@ void viscosity(fc_ctx* c, const double* e, double* mu, int32_t* tau, cudaStream_
 void filter(fc_ctx* c, double* e, bool per_patch, cudaStream_t st) {
   const DevTables& T = c->T;
   double* F = c->d_B3;
-  run_queue(c, c->q_filt1, per_patch, st, "filter_q1",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_filter_q1(T, j, n, L, e, F, s); });
+  run_queue(
+      c, c->q_filt1, per_patch, st, "filter_q1",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_filter_q1(T, j, n, L, e, F, s); }, 1,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_filter_q1(T, t, e, F, s); });
   if (c->nfcopy1) {
     launch_filter_copy_q1(T, c->d_fcopy1, c->nfcopy1, e, F, st);
     c->launches++;
   }
-  run_queue(c, c->q_filt2, per_patch, st, "filter_q2",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_filter_q2(T, j, n, L, F, e, s); });
+  run_queue(
+      c, c->q_filt2, per_patch, st, "filter_q2",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_filter_q2(T, j, n, L, F, e, s); }, 1,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_filter_q2(T, t, F, e, s); });
   if (c->nfcopy2) {
     launch_filter_copy_q2(T, c->d_fcopy2, c->nfcopy2, F, e, st);
     c->launches++;
@@ -2661,7 +2793,7 @@ fc_status fc_shard(fc_ctx* c, int nranks, int rank, const int* owner, fc_comm_fn
     std::vector<Job> jobs;
     for (const Job& J : q->h)
       if (own[J.patch] == rank) jobs.push_back(J);
-    make_queue(c, *q, jobs, c->plans_h, npatch, ok);
+    make_queue(c, *q, jobs, c->plans_h, npatch, ok, q->rest ? &c->mm_h : nullptr);
   }
   // point lists of the owned patches
   std::vector<BcPt> bc;

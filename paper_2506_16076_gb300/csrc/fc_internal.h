@@ -14,6 +14,8 @@ constexpr size_t SMEM_CAP = 200 * 1024;  // dynamic shared memory budget per CTA
 constexpr int SDNN_H = 16;      // hidden width of the stand-in classifier
 constexpr int MAX_GENERIC_RADIX = 128;  // largest prime factor of a continued length
 constexpr int CONT_TMP = 32;    // complex scratch per warp after the line buffer (detrended end data, d <= 8)
+constexpr int MM_KMAX = 256;     // largest inner length of a tensor-core line contraction (fc_mma.cu)
+constexpr int MM_LINES = 4;      // lines per tile of the contraction kernels
 constexpr int NCLASS = 24;      // length classes of the line queues: ceil(log2 Lmax)
 
 // Per-point flag word.
@@ -44,6 +46,15 @@ struct Plan {
   // st of fmod: forward stage st (odd radix, span 1) folds its inputs' factors into the
   // butterfly through per-butterfly records among the forward records
   int fmd, fmf, fmsc, psc, dmul, sigp, fmod;
+};
+
+// Tensor-core contraction of one length L = S H (fc_mmtab.h); H = 0: lines of this length
+// run on the FFT kernels.
+struct MmPlan {
+  int H, S;        // inner length and number of parts (2: even L, 1: odd L)
+  int Kp, Mp, nx;  // H padded to 16 (columns, rows), table entries per part (Mp + Kp)
+  int dtab, ftab;  // first entries of the derivative and filter tables (-1: none)
+  int dte, fte;    // their coefficients are scaled by 2^dte, 2^fte
 };
 
 // One line segment processed by one warp.
@@ -128,6 +139,9 @@ struct DevTables {
   const double* rp;         // real pool (continuation matrices, filter tables)
   const int* ip;            // int pool (slot -> mode tables)
   const Plan* plans;
+  const MmPlan* mm;         // per plan
+  const uint4* mmlo;        // digits 0..3 and 4..5 of the contraction tables
+  const uint2* mmhi;
   const uint32_t* info;     // per-point flags
   const PatchDev* patches;
   int npatch;
@@ -147,6 +161,23 @@ struct DevTables {
   // 1 when some patch uses the product-rule wall form (fc_params.wall_form)
   int any_pform;
 };
+
+// ---- launch wrappers of the contraction kernels (fc_mma.cu) ----
+// tiles: MM_LINES jobs each, of one plan (absent lines: n = 0), all of padded inner length
+// Kp <= kp; two: even lengths
+struct MmTiles {
+  const Job* jobs;
+  int n;      // tiles
+  int kp;
+  int two;
+};
+void launch_mm_cart_q1(const DevTables& T, const MmTiles& t, const double* e, const double* mu, double* R1, double* Fy,
+                       cudaStream_t st);
+void launch_mm_cart_q2(const DevTables& T, const MmTiles& t, const double* mu, const double* R1, double* Fy,
+                       const StageCoef& sc, cudaStream_t st);
+void launch_mm_filter_q1(const DevTables& T, const MmTiles& t, const double* e, double* F, cudaStream_t st);
+void launch_mm_filter_q2(const DevTables& T, const MmTiles& t, const double* F, double* e, cudaStream_t st);
+void set_mm_attributes();
 
 // ---- launch wrappers (fc_kernels.cu) ----
 // Fy (nullable): the y fluxes of the affine points, written by the q1 pass (and by

@@ -1,0 +1,133 @@
+// Host-side builder of the coefficient tables of the tensor-core line contractions
+// (fc_mma.cu): per continued length, the digits of the circulant's coefficients in the
+// order in which a warp's matrix fragments read them.
+//
+// Even L = 2H: with u_j = x_j + x_{j+H}, v_j = x_j - x_{j+H} (j < H) and
+//   U_i = sum_j (c(i-j) + c(i-j+H)) u_j,  V_i = sum_j (c(i-j) - c(i-j+H)) v_j,
+// y_i = (U_i + V_i) / 2 and y_{i+H} = (U_i - V_i) / 2: half the products of the direct
+// sum (two parts of H x H). Odd L: one part of L x L. The left operand of part s is the
+// Toeplitz matrix t_s(i - k); a table holds r(x) = t_s(off - x) at x = k - i + off, one
+// entry per x with the digits of r(x) and r(x+1) side by side (a fragment's register).
+//
+// Derivative (per index): c(m) = (pi/L) (-1)^m cot(pi m / L) for even L (the Nyquist mode
+// has no derivative), (pi/L) (-1)^m / sin(pi m / L) for odd L. Filter: c(m) =
+// (1/L) sum_k sigma(2k/L) cos(2 pi k m / L), sigma(z) = exp(-alpha z^p).
+#pragma once
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "fc_internal.h"
+#include "fc_split.cuh"
+
+namespace fcx {
+
+// whether lines of continued length L run as contractions: both parts' inner length,
+// padded to the instruction's 16, fits 256 (exact level sums, one CTA's pairs)
+inline bool mm_length_ok(int L) { return L >= 16 && ((L % 2 == 0 && L / 2 <= MM_KMAX) || (L % 2 == 1 && L <= MM_KMAX)); }
+
+// FP16 bits of an integer in [-1024, 1024]
+inline uint16_t mm_half(int v) {
+  if (v == 0) return 0;
+  const int a = v < 0 ? -v : v;
+  int e = 0;
+  while ((a >> (e + 1)) != 0) ++e;
+  return (uint16_t)((v < 0 ? 0x8000 : 0) | ((e + 15) << 10) | ((a << (10 - e)) & 0x3ff));
+}
+
+// balanced base-1024 digits, most significant first
+inline void mm_digits(long long q, int* dg) {
+  for (int k = SP_DIGITS - 1; k > 0; --k) {
+    const long long r = ((q + 512) & 1023) - 512;
+    dg[k] = (int)r;
+    q = (q - r) / 1024;
+  }
+  dg[0] = (int)q;
+}
+
+// appends the tables of coefficients c (L values, c(m) = c[m mod L]) to lo / hi (entries
+// of digits 0..3 and 4..5) and returns the first entry; *te: the coefficients were scaled
+// by 2^te
+inline int mm_table(const MmPlan& p, int L, const std::vector<long double>& c, std::vector<uint4>& lo,
+                    std::vector<uint2>& hi, int* te) {
+  const int H = p.H, S = p.S, nx = p.nx, off = p.Mp;
+  auto t = [&](int s, int m) {
+    const long double a = c[(size_t)(((m % L) + L) % L)];
+    if (S == 1) return a;
+    const long double b = c[(size_t)((((m + H) % L) + L) % L)];
+    return s ? a - b : a + b;
+  };
+  long double top = 0;
+  for (int s = 0; s < S; ++s)
+    for (int m = 0; m < H; ++m) top = std::max(top, std::fabs(t(s, m)));
+  *te = top > 0 ? SP_COEF - (int)std::lround(std::log2((double)top)) : SP_COEF;
+  const int first = (int)lo.size();
+  for (int s = 0; s < S; ++s) {
+    std::vector<uint16_t> dg((size_t)SP_DIGITS * (nx + 1));
+    for (int x = 0; x <= nx; ++x) {
+      int d[SP_DIGITS];
+      mm_digits((long long)std::llround(std::ldexp(t(s, off - x), *te)), d);
+      for (int k = 0; k < SP_DIGITS; ++k) dg[(size_t)k * (nx + 1) + x] = mm_half(d[k]);
+    }
+    auto pair = [&](int k, int x) {
+      return (uint32_t)dg[(size_t)k * (nx + 1) + x] | ((uint32_t)dg[(size_t)k * (nx + 1) + x + 1] << 16);
+    };
+    for (int x = 0; x < nx; ++x) {
+      lo.push_back(uint4{pair(0, x), pair(1, x), pair(2, x), pair(3, x)});
+      hi.push_back(uint2{pair(4, x), pair(5, x)});
+    }
+  }
+  return first;
+}
+
+// MmPlan of length L (mm_length_ok) with its derivative table and, when sig is given
+// (sigma(2k/L) for k = 0..L/2), its filter table
+inline MmPlan mm_plan(int L, const std::vector<long double>* sig, std::vector<uint4>& lo, std::vector<uint2>& hi) {
+  const long double PI_L = 3.14159265358979323846264338327950288L;
+  MmPlan p{};
+  p.S = L % 2 == 0 ? 2 : 1;
+  p.H = L / p.S;
+  p.Kp = (p.H + 15) / 16 * 16;
+  p.Mp = p.Kp;
+  p.nx = p.Mp + p.Kp;
+  // cos(pi j / (2L)), which also gives sin(pi m / L) = cos(pi (L - 2m) / (2L))
+  std::vector<long double> cs((size_t)2 * L + 1);
+  for (int j = 0; j <= L; ++j) {
+    cs[j] = cosl(PI_L * j / (2.0L * L));
+    cs[2 * L - j] = -cs[j];
+  }
+  cs[L] = 0.0L;
+  std::vector<long double> c((size_t)L, 0.0L);
+  for (int m = 1; 2 * m <= L; ++m) {
+    const long double sn = cs[L - 2 * m];  // sin(pi m / L)
+    const long double v = (PI_L / L) * (m % 2 ? -1.0L : 1.0L) * (L % 2 == 0 ? cs[2 * m] / sn : 1.0L / sn);
+    c[m] = v;
+    c[L - m] = -v;
+  }
+  if (L % 2 == 0) c[L / 2] = 0.0L;
+  p.dtab = mm_table(p, L, c, lo, hi, &p.dte);
+  p.ftab = -1;
+  if (sig) {
+    // cosine sums in 128-bit integers (sigma in 2^-58, cosines in 2^-60)
+    std::vector<long long> sq((size_t)L / 2 + 1), cq((size_t)L);
+    for (int k = 0; 2 * k <= L; ++k) sq[k] = (long long)std::llround(std::ldexp((*sig)[k], 58));
+    for (int j = 0; 2 * j <= L; ++j) {
+      cq[j] = (long long)std::llround(std::ldexp(cs[4 * j], 60));
+      if (j) cq[L - j] = cq[j];
+    }
+    for (int m = 0; 2 * m <= L; ++m) {
+      __int128 a = 0;
+      for (int k = 1; 2 * k < L; ++k) a += (__int128)sq[k] * cq[(size_t)((long long)k * m % L)];
+      a *= 2;
+      a += (__int128)sq[0] * cq[0];
+      if (L % 2 == 0) a += (__int128)sq[L / 2] * cq[(size_t)((long long)(L / 2) * m % L)];
+      const long double v = std::ldexp((long double)a, -118) / L;
+      c[m] = v;
+      if (m) c[L - m] = v;
+    }
+    p.ftab = mm_table(p, L, c, lo, hi, &p.fte);
+  }
+  return p;
+}
+
+}  // namespace fcx

@@ -1,0 +1,95 @@
+// Exact split-integer arithmetic of the tensor-core line contractions (fc_mma.cu).
+//
+// An FC line operator (derivative or filter of the continued line, eqs. fc_der and
+// filtering) is a circulant of length L: y_i = sum_j c(i - j) x_j. Data and coefficients
+// are held as fixed-point integers of 60 bits, cut into six balanced base-1024 digits in
+// [-512, 511]. A digit is exact in FP16, a product of two is at most 2^18 and a sum of up
+// to 256 of them stays below 2^24 for the operators used here (fc_mmtab.h), so the FP16
+// matrix instruction with FP32 accumulation adds them without rounding. The digit products
+// of equal weight (levels i + j = 0..5, 21 of the 36 pairs) share an accumulator; the
+// levels are joined in 64-bit integers. The dropped levels and the truncation of the data
+// leave an error of a few 2^-57 of the line's largest value times the operator's largest
+// coefficient, below the rounding of an FP64 transform of the same line.
+#pragma once
+#include <stdint.h>
+#include <string.h>
+
+#include "fc_internal.h"
+
+#ifndef FC_HD
+#define FC_HD __host__ __device__ __forceinline__
+#endif
+
+namespace fcx {
+
+constexpr int SP_DIGITS = 6;     // digits per value = accumulation levels
+constexpr int SP_BITS = 10;      // bits per digit
+constexpr int SP_DATA = 56;      // a line's data are scaled so that its largest value lies in [2^56, 2^57)
+constexpr int SP_COEF = 60;      // coefficients are scaled so that the largest lies in [2^59.5, 2^60.5]
+constexpr int SP_UNIT = 60;      // unit of the joined sums: 2^60 of data x coefficient units
+// 512 in every digit position: turns balanced digits into plain bit fields
+constexpr long long SP_BIAS = (512ll << 50) | (512ll << 40) | (512ll << 30) | (512ll << 20) | (512ll << 10) | 512ll;
+
+FC_HD uint32_t sp_hi(double x) {
+#ifdef __CUDA_ARCH__
+  return (uint32_t)__double2hiint(x);
+#else
+  uint64_t b;
+  memcpy(&b, &x, 8);
+  return (uint32_t)(b >> 32);
+#endif
+}
+FC_HD uint32_t sp_lo(double x) {
+#ifdef __CUDA_ARCH__
+  return (uint32_t)__double2loint(x);
+#else
+  uint64_t b;
+  memcpy(&b, &x, 8);
+  return (uint32_t)b;
+#endif
+}
+
+// x as a fixed-point integer in units 2^(ex - 1023 - SP_DATA), ex the biased exponent of
+// the line's largest magnitude (rounded down; zero and subnormal values are 0)
+FC_HD long long sp_fixed(double x, int ex) {
+  const uint32_t hi = sp_hi(x), lo = sp_lo(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  const int d = ex - e;
+  if (e == 0 || d > 62 || d < 0) return 0;  // d < 0 only for a non-finite line (its outputs are NaN)
+  const long long m = (long long)(((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << (SP_DATA - 52);
+  return ((hi >> 31) ? -m : m) >> d;
+}
+
+// digit pair: the base-1024 digits number k (0 = most significant) of two biased values,
+// as two FP16 integers in one word
+FC_HD uint32_t sp_field(long long biased, int k) { return (uint32_t)(biased >> (SP_BITS * (SP_DIGITS - 1 - k))) & 1023u; }
+
+// joined sum of the six level sums (exact integers below 2^24) in units 2^SP_UNIT
+FC_HD long long sp_join(const int* s) {
+  const long long hi = ((long long)s[0] << 20) + ((long long)s[1] << 10) + s[2];
+  const long long lo = ((long long)s[3] << 20) + ((long long)s[4] << 10) + s[5];
+  return (hi << (80 - SP_UNIT)) + (lo >> (SP_UNIT - 50));
+}
+
+// a 64-bit integer as a double, rounded to nearest (ties away from zero), without the FP64 pipe
+FC_HD double sp_double(long long v) {
+  const uint64_t a = v < 0 ? (uint64_t)(-v) : (uint64_t)v;
+#ifdef __CUDA_ARCH__
+  const int lz = __clzll((long long)a);
+#else
+  const int lz = a ? __builtin_clzll(a) : 64;
+#endif
+  const uint64_t m = a << (lz & 63);
+  uint64_t b = ((uint64_t)(1085 - lz) << 52) + (m >> 11) + ((m >> 10) & 1u);
+  b = a ? b : 0;
+  b |= (uint64_t)v & 0x8000000000000000ull;
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)b);
+#else
+  double r;
+  memcpy(&r, &b, 8);
+  return r;
+#endif
+}
+
+}  // namespace fcx

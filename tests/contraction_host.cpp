@@ -1,0 +1,94 @@
+// Host build of the split-integer contraction (fc_split.cuh, fc_mmtab.h): the tables and
+// the arithmetic the GPU kernels use, with the matrix products formed in plain loops.
+//
+//   contraction_host L1 L2 ...
+//     for every continued length, the derivative and the filter of a white line, a nearly
+//     constant one and one with a spike against the same circulant in long double; prints
+//     "L op kind error/max|x| largest_level_sum" (op 0: derivative, 1: filter), or "L none"
+//     when lines of this length are left to the FFT kernels.
+#include <cstdio>
+#include <cstdlib>
+#include <random>
+
+#include "../paper_2506_16076_gb300/csrc/fc_mmtab.h"
+
+using namespace fcx;
+
+static double half_value(unsigned h) {
+  const int e = (h >> 10) & 31, m = h & 1023;
+  const double v = e ? std::ldexp(1024.0 + m, e - 25) : 0.0;
+  return (h >> 15) & 1 ? -v : v;
+}
+
+int main(int argc, char** argv) {
+  std::mt19937_64 g(1);
+  std::uniform_real_distribution<double> U(-1.0, 1.0);
+  const long double PI = 3.14159265358979323846264338327950288L;
+  for (int a = 1; a < argc; ++a) {
+    const int L = std::atoi(argv[a]);
+    if (!mm_length_ok(L)) {
+      printf("%d none\n", L);
+      continue;
+    }
+    std::vector<uint4> lo;
+    std::vector<uint2> hi;
+    std::vector<long double> sig;
+    for (int k = 0; 2 * k <= L; ++k) sig.push_back(expl(-10.0L * powl(2.0L * k / L, 14)));
+    const MmPlan p = mm_plan(L, &sig, lo, hi);
+    for (int op = 0; op < 2; ++op) {
+      std::vector<long double> c(L, 0.0L);  // the circulant, by its definition
+      for (int m = 0; m < L; ++m) {
+        long double s = 0;
+        for (int k = 1; 2 * k <= L; ++k) {
+          const long double an = 2.0L * PI * ((long long)k * m % L) / L;
+          if (op == 0)
+            s += 2 * k < L ? -2.0L * (2.0L * PI * k / L) * sinl(an) : 0.0L;
+          else
+            s += (2 * k < L ? 2.0L : 1.0L) * sig[k] * cosl(an);
+        }
+        c[m] = (s + (op ? sig[0] : 0.0L)) / L;
+      }
+      for (int kind = 0; kind < 3; ++kind) {
+        std::vector<double> x(L);
+        double top = 0;
+        for (int i = 0; i < L; ++i) {
+          x[i] = kind == 0 ? U(g) : kind == 1 ? 1.4 + 0.01 * std::sin(6.283185307179586 * 3 * i / L) : 1e-3 * U(g);
+          if (kind == 2 && i == L / 3) x[i] = 1000.0;
+          top = std::max(top, std::fabs(x[i]));
+        }
+        const int ex = (int)((sp_hi(top) >> 20) & 0x7ff), te = op ? p.fte : p.dte, tab = op ? p.ftab : p.dtab;
+        std::vector<long long> W[2];
+        double level = 0;
+        for (int s = 0; s < p.S; ++s)
+          for (int i = 0; i < p.H; ++i) {
+            double lev[SP_DIGITS] = {0};
+            for (int k = 0; k < p.H; ++k) {
+              const long long x0 = sp_fixed(x[k], ex), x1 = p.S == 2 ? sp_fixed(x[k + p.H], ex) : 0;
+              const long long b = (s ? x0 - x1 : x0 + x1) + SP_BIAS;
+              const int at = tab + s * p.nx + k - i + p.Mp;
+              const unsigned w[SP_DIGITS] = {lo[at].x, lo[at].y, lo[at].z, lo[at].w, hi[at].x, hi[at].y};
+              for (int u = 0; u < SP_DIGITS; ++u)
+                for (int v = 0; u + v < SP_DIGITS; ++v)
+                  lev[u + v] += half_value(w[u] & 0xffff) * ((int)sp_field(b, v) - 512);
+            }
+            int si[SP_DIGITS];
+            for (int l = 0; l < SP_DIGITS; ++l) {
+              si[l] = (int)lev[l];
+              level = std::max(level, std::fabs(lev[l]));
+            }
+            W[s].push_back(sp_join(si));
+          }
+        const double fac = std::scalbn(1.0, ex - 1023 - SP_DATA + SP_UNIT - te - (p.S - 1));
+        double err = 0;
+        for (int i = 0; i < L; ++i) {
+          const long long v = p.S == 1 ? W[0][i] : (i < p.H ? W[0][i] + W[1][i] : W[0][i - p.H] - W[1][i - p.H]);
+          long double ref = 0;
+          for (int j = 0; j < L; ++j) ref += c[((i - j) % L + L) % L] * (long double)x[j];
+          err = std::max(err, (double)fabsl((long double)(sp_double(v) * fac) - ref));
+        }
+        printf("%d %d %d %.3e %.0f\n", L, op, kind, err / top, level);
+      }
+    }
+  }
+  return 0;
+}

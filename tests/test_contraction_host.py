@@ -1,0 +1,50 @@
+"""The exact split-integer contraction of FC lines (fc_split.cuh, fc_mmtab.h) on the CPU:
+every inner length's tables and arithmetic, with the digit products in plain loops, against
+the circulant of the spectral derivative (eq. fc_der) and of the filter (eq. filtering) in
+long double.
+
+Tolerance, relative to the line's largest value (coefficients at most about 1): the dropped
+digit products are sums of 5 H pairs of digits of standard deviation 2^8.2 in units 2^40, the
+largest value is at least 2^56 times a coefficient of 2^59.5: 2^-54 for H = 256; truncated
+data and rounded coefficients add less. Eight times that, for the largest of all rows and
+both parts, and one FP64 rounding: 2^-51 + 2^-52 < 7e-16. Level sums must stay below 2^24,
+where FP32 accumulation stops being exact."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CUDA_INC = "/usr/local/cuda/include"
+
+
+@pytest.fixture(scope="module")
+def exe(tmp_path_factory):
+    gxx = shutil.which("g++")
+    if gxx is None or not os.path.isdir(CUDA_INC):
+        pytest.skip("g++ and the CUDA headers are needed to build the host harness")
+    out = str(tmp_path_factory.mktemp("mm") / "contraction_host")
+    r = subprocess.run([gxx, "-O2", "-std=c++17", "-w", f"-I{CUDA_INC}", "-o", out,
+                        os.path.join(ROOT, "tests", "contraction_host.cpp")], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-3000:]
+    return out
+
+
+# edges of the padding to 16, both parities, the shortest and the longest inner lengths
+LENGTHS = [16, 17, 30, 31, 32, 33, 34, 37, 64, 66, 155, 192, 224, 255, 256, 258, 288, 432, 510, 512]
+
+
+def test_contraction_matches_the_circulant(exe):
+    r = subprocess.run([exe, *map(str, LENGTHS)], capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr
+    rows = [ln.split() for ln in r.stdout.splitlines()]
+    assert len(rows) == 6 * len(LENGTHS)
+    for L, op, kind, err, level in rows:
+        assert float(err) < 7e-16, (L, op, kind, err)
+        assert float(level) < 2 ** 24, (L, op, kind, level)
+
+
+def test_other_lengths_are_left_to_the_transforms(exe):
+    r = subprocess.run([exe, "15", "257", "514", "1024"], capture_output=True, text=True)
+    assert r.returncode == 0 and [ln.split()[1] for ln in r.stdout.splitlines()] == ["none"] * 4

@@ -1,0 +1,83 @@
+"""The tensor-core contraction of FC lines on the GPU at the sizes where it can go wrong:
+inner lengths around the padding to 16 and around the two CTA sizes (128 and 129), the
+longest contracted lengths and the first ones left to the transforms, odd lengths, tiles
+with absent lines; lines of zeros and non-finite values.
+
+Tolerance of the operator as in the other edge cases: 1e-11, or twice the error of an FP64
+FFT evaluation where that is larger."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import solver as S
+from paper_2506_16076_gb300 import workloads as W
+from tests.gpu_helpers import fp64_floor, from_dev, rel_err, smooth_mu, to_dev, to_dev_scalar_field
+
+pytestmark = pytest.mark.gpu
+
+
+def _box(n1, n2):
+    fs = (1.4, 1.0, 0.3, 1.0)
+    p = W.PatchDesc(W.AFFINE, n1, n2, (0.0, 1.0, 0.0, 0.7), (W.DIRICHLET,) * 4, bc=(fs,) * 4)
+    return W.Workload(f"box_{n1}x{n2}", [p], W.Params(c_policy=0), fs, "freestream", 1)
+
+
+# n + 27: 64, 66, 128, 256 / 258 (inner 128 / 129), 512 and 513 (transforms), odd 255 and 259 (transforms)
+CASES = [(37, 39), (101, 10), (229, 231), (485, 13), (486, 11), (228, 14), (232, 17)]
+
+
+@pytest.mark.parametrize("n1,n2", CASES)
+def test_rhs_and_filter_at_the_length_edges(gpu_lib, n1, n2):
+    w = _box(n1, n2)
+    ctx = gpu_lib.Context(w)
+    sv = S.Solver(w)
+    st = W.random_smooth_state(w, seed=n1 + n2, amp=0.2)
+    mu = smooth_mu(w, seed=2, scale=0.01)
+    mu[0][:, : n1 // 2] = 0.0  # inviscid and viscous column tiles
+    e = to_dev(st)
+    out = torch.empty_like(e)
+    ctx.rhs(e, out, to_dev_scalar_field(mu))
+    ref = sv.rhs(st, mu)
+    tol = max(1e-11, 2 * max(rel_err(fp64_floor(sv, lambda: sv.rhs(st, mu)), ref)))
+    errs = rel_err(from_dev(out, w), ref)
+    assert max(errs) < tol, (errs, tol)
+    ctx.filter(e)
+    ref = sv.filter(st)
+    tol = max(1e-11, 2 * max(rel_err(fp64_floor(sv, lambda: sv.filter(st)), ref)))
+    errs = rel_err(from_dev(e, w), ref)
+    assert max(errs) < tol, (errs, tol)
+
+
+def test_uniform_gas_at_rest_stays_exactly_at_rest(gpu_lib):
+    # u = v = 0: the momentum lines are zero, their derivatives exactly zero
+    w = _box(101, 37)
+    st = [W.prim_to_cons(np.full((37, 101), 1.4), np.zeros((37, 101)), np.zeros((37, 101)), np.full((37, 101), 1.0))]
+    e = to_dev(st)
+    ctx = gpu_lib.Context(w)
+    ctx.filter(e)
+    assert torch.equal(e[1:3], torch.zeros_like(e[1:3]))
+    out = torch.empty_like(e)
+    ctx.rhs(e, out, torch.zeros(e.shape[1], dtype=torch.float64, device="cuda"))
+    assert torch.equal(out[0], torch.zeros_like(out[0])) and torch.equal(out[3], torch.zeros_like(out[3]))
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_non_finite_point_spoils_its_lines_only(gpu_lib, bad):
+    w = _box(101, 39)
+    n1, n2 = 101, 39
+    st = W.random_smooth_state(w, seed=4, amp=0.2)
+    mu = torch.zeros(n1 * n2, dtype=torch.float64, device="cuda")
+    ctx = gpu_lib.Context(w)
+    e = to_dev(st)
+    good, out = torch.empty_like(e), torch.empty_like(e)
+    ctx.rhs(e, good, mu)
+    j, i = 20, 33
+    e[3, j * n1 + i] = bad
+    ctx.rhs(e, out, mu)
+    fin = torch.isfinite(out).reshape(4, n2, n1)
+    # packed pairs (0, 1) and (2, 3): the x flux has p in both, the y flux in the second only
+    assert not fin[:, j, :].any() and not fin[2:, :, i].any()
+    keep = torch.ones(n2, n1, dtype=torch.bool, device="cuda")
+    keep[j, :] = False
+    keep[:, i] = False
+    assert torch.equal(out.reshape(4, n2, n1)[:, keep], good.reshape(4, n2, n1)[:, keep])
