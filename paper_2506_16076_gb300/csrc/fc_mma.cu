@@ -17,9 +17,12 @@
 // 128 and 256 beyond keep 16 warps per SM resident.
 //
 // Measured (28M points, affine lines of 48 to 384 points, FFT kernels -> contraction, per
-// pass): q1 9.6 -> 5.4 ms, q2 10.0 -> 7.1 ms, filter q1 + q2 17.5 -> 8.5 ms; a 128 x 128
-// operator with L = 155 = 5 x 31: 464 -> 27 us. Largest error on white lines 2e-16 of the
-// largest value (FP64 FFT: 6e-16 to 9e-16).
+// pass): q1 9.6 -> 4.5 ms, q2 10.0 -> 6.3 ms, filter q1 + q2 17.5 -> 8.1 ms; a 128 x 128
+// operator with L = 155 = 5 x 31: 462 -> 25 us. Largest error on white lines 2e-16 of the
+// largest value (FP64 FFT: 6e-16 to 9e-16). Of these times, passing the values through
+// shared memory (the fluxes' lanes then follow the points, 89% of them active instead of
+// 78%) and fetching a step's table entries one step ahead took 17%; a tile keeps its
+// sub-core's matrix pipe busy for 12k of about 26k cycles, the FP64 pipe for 10k to 15k.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -41,15 +44,20 @@ struct MmShared {
   Job J[MM_LINES];
   uint32_t emax[NCOL];  // high words of the largest magnitudes
   double fac[NCOL];     // value of one unit of a joined sum
+  double tmp[NCOL * 16];  // detrended end values of the columns, 2d <= 16 each
 };
 
-// dynamic shared memory: the digits [S][SP_DIGITS][NCOL][Kp + 8] of FP16 (rows padded by
-// 16 bytes: conflict-free ldmatrix), which before the digits exist hold the lines' end
-// values, their detrended form and the continuation values
+constexpr int LB = 4;  // points of a thread whose loads are in flight together
+
+// columns of the lines' values in shared memory: a pitch of 4 (mod 16) doubles keeps the
+// four lines of a row of q2 points in different banks
+__host__ __device__ inline int mm_line_pitch(int L) { return L + ((4 - L % 16) + 16) % 16; }
+// dynamic shared memory: the digits [S][SP_DIGITS][NCOL][Kp + 8] of FP16 (columns padded by
+// 16 bytes: conflict-free ldmatrix), over the continued lines [NCOL][pitch] they come from
 size_t mm_smem(int S, int Kp) {
   const size_t dig = (size_t)S * SP_DIGITS * NCOL * (Kp + 8) * 2;
-  const size_t pre = (size_t)NCOL * (2 * 16 + 128) * sizeof(double);
-  return dig > pre ? dig : pre;
+  const size_t val = (size_t)NCOL * mm_line_pitch(S * Kp) * sizeof(double);
+  return dig > val ? dig : val;
 }
 
 __device__ __forceinline__ void mma16816(float* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
@@ -63,6 +71,25 @@ __device__ __forceinline__ void ldsm4(uint32_t* r, uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(addr));
+}
+
+// table entries stay in L1 (every warp of the SM reads them), the lines' data pass by it
+__device__ __forceinline__ uint4 ldg_keep(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::evict_last.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint2 ldg_keep(const uint2* p) {
+  uint2 v;
+  asm volatile("ld.global.nc.L1::evict_last.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_pass(const double* p) {
+  double v;
+  asm volatile("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
 }
 
 // two biased values' digit k as an FP16 pair: the 10-bit fields become 1024 + field by
@@ -87,10 +114,10 @@ __device__ __forceinline__ void mm_part(const uint4* __restrict__ lo, const uint
     for (int q = 0; q < 4; ++q) acc[l][0][q] = acc[l][1][q] = 0.f;
   const uint4* pl = lo + (p.Mp - i0 + 2 * t - g);
   const uint2* ph = hi + (p.Mp - i0 + 2 * t - g);
-  uint32_t Am[SP_DIGITS], A0[SP_DIGITS], Ap[SP_DIGITS];
+  uint32_t Am[SP_DIGITS], A0[SP_DIGITS], Ap[SP_DIGITS], N0[SP_DIGITS], Np[SP_DIGITS];
   auto entry = [&](uint32_t* A, int x) {
-    const uint4 a = __ldg(pl + x);
-    const uint2 b = __ldg(ph + x);
+    const uint4 a = ldg_keep(pl + x);
+    const uint2 b = ldg_keep(ph + x);
     A[0] = a.x;
     A[1] = a.y;
     A[2] = a.z;
@@ -99,25 +126,34 @@ __device__ __forceinline__ void mm_part(const uint4* __restrict__ lo, const uint
     A[5] = b.y;
   };
   entry(Am, -8);
+  entry(A0, 0);
+  entry(Ap, 8);
   // ldmatrix row addresses: matrices (columns 0-7, k), (columns 0-7, k+8), (8-15, k), (8-15, k+8)
   uint32_t baddr = dig + (uint32_t)(((lane & 7) + ((lane >> 4) << 3)) * pitch + ((lane >> 3) & 1) * 16);
   const uint32_t bslice = (uint32_t)NCOL * pitch;
   for (int k0 = 0; k0 < p.Kp; k0 += 16) {
-    entry(A0, k0);
-    entry(Ap, k0 + 8);
+    const int kn = k0 + 16 < p.Kp ? k0 + 16 : k0;  // the next step's entries, a whole step ahead
+    entry(N0, kn);
+    entry(Np, kn + 8);
+    uint32_t b[2][4];
+    ldsm4(b[0], baddr);
 #pragma unroll
     for (int j = 0; j < SP_DIGITS; ++j) {
-      uint32_t b[4];
-      ldsm4(b, baddr + j * bslice);
+      if (j + 1 < SP_DIGITS) ldsm4(b[(j + 1) & 1], baddr + (j + 1) * bslice);
+      const uint32_t* c = b[j & 1];
 #pragma unroll
       for (int i = 0; i + j < SP_DIGITS; ++i) {
-        mma16816(acc[i + j][0], A0[i], Am[i], Ap[i], A0[i], b[0], b[1]);
-        mma16816(acc[i + j][1], A0[i], Am[i], Ap[i], A0[i], b[2], b[3]);
+        mma16816(acc[i + j][0], A0[i], Am[i], Ap[i], A0[i], c[0], c[1]);
+        mma16816(acc[i + j][1], A0[i], Am[i], Ap[i], A0[i], c[2], c[3]);
       }
     }
     baddr += 32;
 #pragma unroll
-    for (int i = 0; i < SP_DIGITS; ++i) Am[i] = Ap[i];
+    for (int i = 0; i < SP_DIGITS; ++i) {
+      Am[i] = Ap[i];
+      A0[i] = N0[i];
+      Ap[i] = Np[i];
+    }
   }
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
@@ -137,7 +173,7 @@ __device__ __forceinline__ long long point(const MmShared& sh, int line, int t) 
 // continuation, as continue_lines), D = d when it is known at compile time
 template <int NT, int D>
 __device__ __forceinline__ void continuation(const double* __restrict__ M, int C, int dd, const double* tmp,
-                                             double* ext, uint32_t* emax) {
+                                             double* ext, int LP, uint32_t* emax) {
   const int d = D ? D : dd;
   const double* ML = M;
   const double* MR = M + C * d;
@@ -153,7 +189,7 @@ __device__ __forceinline__ void continuation(const double* __restrict__ M, int C
     x = fma(e[2 * d - 4], __ldg(u + k),
             fma(e[2 * d - 3], __ldg(u + C + k),
                 fma(e[2 * d - 2], __ldg(u + 2 * C + k), fma(e[2 * d - 1], __ldg(u + 3 * C + k), x))));
-    ext[col * C + k] = x;
+    ext[col * LP + k] = x;
     atomicMax(&emax[col], sp_hi(x) & 0x7fffffffu);
   }
 }
@@ -164,71 +200,65 @@ __device__ __forceinline__ void continuation(const double* __restrict__ M, int C
 // ep.pre(comp, point) loaded ahead for a batch of eight, or with PT ep.put(point, v[4]) a
 // point's four at once. All threads of the CTA call it; it begins with a barrier.
 template <int NT, int S, bool COL, bool FILT, bool PT, class Load, class Ep>
-__device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& p, MmShared& sh, double2* dyn, Load ld,
+__device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan, MmShared& sh, double2* dyn, Load ld,
                                          Ep ep) {
-  constexpr int NW = NT / 32;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NW = NT / 32, TS = NT / 4;  // TS: points per step of a line
+  // opaque copies: without them the compiler hoists the address arithmetic of both of a
+  // kernel's rounds out of their loop (250 registers, 280 bytes of spills; so 128 and < 150)
+  int tid = threadIdx.x;
+  MmPlan p = plan;
+  asm volatile("" : "+r"(tid), "+r"(p.H), "+r"(p.Kp), "+r"(p.nx), "+r"(p.Mp));
+  const int warp = tid >> 5, lane = tid & 31;
   const int n = sh.J[0].n, C = sh.J[0].C, fcm = sh.J[0].fcm, d = T.d, H = p.H;
-  double* ends = reinterpret_cast<double*>(dyn);  // [NCOL][2d]: first and last d values
-  double* tmp = ends + NCOL * 16;                 // [NCOL][2d]: detrended
-  double* ext = tmp + NCOL * 16;                  // [NCOL][C]
+  const int LP = mm_line_pitch(S * H);
+  double* F = reinterpret_cast<double*>(dyn);  // [NCOL][LP]: the continued lines
   if (tid < NCOL) sh.emax[tid] = 0;
   __syncthreads();
 
-  // (1) points into registers: pairs (2q, 2q+1) of each part, their end values and maxima
-  const int line = COL ? (lane & 3) : (warp & 3);
-  const int q0 = COL ? (lane >> 2) + 8 * warp : (warp >> 2) * 32 + lane;
-  constexpr int QS = COL ? 8 * NW : 8 * NW;  // pairs per r
-  const bool have = sh.J[line].n > 0;
-  double X[2][S][2][4];
-  uint32_t hm[4] = {0, 0, 0, 0};
+  // (1) the lines' values into shared memory, and their maxima. q1 lines: a warp per line
+  // (two with 256 threads), lanes along it; q2 lines: 4 neighbouring lines along the lanes
+  {
+    const int line = COL ? (tid & 3) : (warp & 3);
+    const int t0 = COL ? tid >> 2 : (warp >> 2) * 32 + lane;
+    const bool have = sh.J[line].n > 0;
+    uint32_t hm[4] = {0, 0, 0, 0};
+    for (int b = t0; b < n; b += LB * TS) {
+      double X[LB][4];
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    // all loads of the batch first (absent points read the line's first one), then the work
+      for (int r = 0; r < LB; ++r)  // the batch's loads first (absent points read the line's first one)
+        ld.raw(point(sh, line, b + r * TS < n ? b + r * TS : 0), X[r]);
 #pragma unroll
-    for (int s = 0; s < S; ++s)
-#pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const int k = 2 * (q0 + r * QS) + a, idx = k + s * H;
-        ld.raw(point(sh, line, k < H && idx < n ? idx : 0), X[r][s][a]);
-      }
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-#pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const int k = 2 * (q0 + r * QS) + a, idx = k + s * H;
-        double* v = X[r][s][a];
-        if (have && k < H && idx < n) {
-          ld.form(point(sh, line, idx), v);
+      for (int r = 0; r < LB; ++r) {
+        const int t = b + r * TS;
+        if (t < n) {
+          double* v = X[r];
+          if (have)
+            ld.form(point(sh, line, t), v);
+          else
+            v[0] = v[1] = v[2] = v[3] = 0.0;
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             const uint32_t h = sp_hi(v[c]) & 0x7fffffffu;
             hm[c] = h > hm[c] ? h : hm[c];
+            F[(c * MM_LINES + line) * LP + t] = v[c];
           }
-          if (fcm >= 0) {
-            if (idx < d)
-              for (int c = 0; c < 4; ++c) ends[(c * MM_LINES + line) * 16 + idx] = v[c];
-            if (idx >= n - d)
-              for (int c = 0; c < 4; ++c) ends[(c * MM_LINES + line) * 16 + d + idx - (n - d)] = v[c];
-          }
-        } else {
-          v[0] = v[1] = v[2] = v[3] = 0.0;
         }
       }
-  }
+    }
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    if (COL) {
-      uint32_t h = hm[c];
+    for (int c = 0; c < 4; ++c) {
+      if (COL) {
+        uint32_t h = hm[c];
 #pragma unroll
-      for (int o = 4; o < 32; o <<= 1) {
-        const uint32_t g = __shfl_xor_sync(0xffffffffu, h, o);
-        h = g > h ? g : h;
+        for (int o = 4; o < 32; o <<= 1) {
+          const uint32_t g = __shfl_xor_sync(0xffffffffu, h, o);
+          h = g > h ? g : h;
+        }
+        if (lane < MM_LINES) atomicMax(&sh.emax[c * MM_LINES + line], h);
+      } else {
+        const uint32_t h = __reduce_max_sync(0xffffffffu, hm[c]);
+        if (lane == 0) atomicMax(&sh.emax[c * MM_LINES + line], h);
       }
-      if (lane < MM_LINES) atomicMax(&sh.emax[c * MM_LINES + line], h);
-    } else {
-      const uint32_t h = __reduce_max_sync(0xffffffffu, hm[c]);
-      if (lane == 0) atomicMax(&sh.emax[c * MM_LINES + line], h);
     }
   }
   __syncthreads();
@@ -237,36 +267,26 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& p, Mm
   if (fcm >= 0) {
     for (int it = tid; it < NCOL * 2 * d; it += NT) {
       const int col = it & (NCOL - 1), q = it / NCOL;
-      const double* x = ends + col * 16;
-      const double f0 = x[0], dl = x[1] - f0, fn = x[2 * d - 1], dr = fn - x[2 * d - 2];
+      const double* x = F + col * LP;
+      const double f0 = x[0], dl = x[1] - f0, fn = x[n - 1], dr = fn - x[n - 2];
       double v;
       if (q < d - 2) {
         v = fma(-(double)(q + 2), dl, x[q + 2] - f0);
       } else if (q < 2 * d - 4) {
         const int j = q - (d - 2);
-        v = fma((double)(d - 1 - j), dr, x[d + j] - fn);
+        v = fma((double)(d - 1 - j), dr, x[n - d + j] - fn);
       } else {
         const int w = q - (2 * d - 4);
         v = w == 0 ? f0 : (w == 1 ? dl : (w == 2 ? fn : dr));
       }
-      tmp[col * 16 + q] = v;
+      sh.tmp[col * 16 + q] = v;
     }
     __syncthreads();
     if (d == 5)
-      continuation<NT, 5>(T.rp + fcm, C, 5, tmp, ext, sh.emax);
+      continuation<NT, 5>(T.rp + fcm, C, 5, sh.tmp, F + n, LP, sh.emax);
     else
-      continuation<NT, 0>(T.rp + fcm, C, d, tmp, ext, sh.emax);
+      continuation<NT, 0>(T.rp + fcm, C, d, sh.tmp, F + n, LP, sh.emax);
     __syncthreads();
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-      for (int s = 0; s < S; ++s)
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-          const int k = 2 * (q0 + r * QS) + a, idx = k + s * H;
-          if (have && k < H && idx >= n)
-            for (int c = 0; c < 4; ++c) X[r][s][a][c] = ext[(c * MM_LINES + line) * C + idx - n];
-        }
   }
   const int te = FILT ? p.fte : p.dte;
   if (tid < NCOL) {
@@ -277,37 +297,53 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& p, Mm
                       ? __longlong_as_double(0x7ff8000000000000ll)
                       : scalbn(sc, (int)(h >> 20) - 1023 - SP_DATA + SP_UNIT - te - (S - 1));
   }
-  int ex[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) ex[c] = (int)(sh.emax[c * MM_LINES + line] >> 20);
-  __syncthreads();
 
-  // (3) digits of the parts
-  const int pitchw = (p.Kp + 8) / 2;  // words per column
-  uint32_t* dig = reinterpret_cast<uint32_t*>(dyn);
+  // (3) digits of the parts, over the values: all reads come before the first write. A warp
+  // per line again, lanes along the pairs (2q, 2q + 1)
+  {
+    const int line = warp & 3, q0 = (warp >> 2) * 32 + lane;
+    double X[2][4][S][2];
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int q = q0 + r * QS;
-    if (2 * q < p.Kp) {
+    for (int r = 0; r < 2; ++r)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        long long w[S][2];
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-          const long long x0 = sp_fixed(X[r][0][a][c], ex[c]);
-          if (S == 2) {
-            const long long x1 = sp_fixed(X[r][S - 1][a][c], ex[c]);
-            w[0][a] = x0 + x1 + SP_BIAS;
-            w[S - 1][a] = x0 - x1 + SP_BIAS;
-          } else {
-            w[0][a] = x0 + SP_BIAS;
-          }
-        }
+      for (int c = 0; c < 4; ++c)
 #pragma unroll
         for (int s = 0; s < S; ++s)
 #pragma unroll
-          for (int k = 0; k < SP_DIGITS; ++k)
-            dig[((s * SP_DIGITS + k) * NCOL + c * MM_LINES + line) * pitchw + q] = digit_pair(w[s][0], w[s][1], k);
+          for (int a = 0; a < 2; ++a) {
+            const int k = 2 * (q0 + r * TS) + a;
+            X[r][c][s][a] = k < H ? F[(c * MM_LINES + line) * LP + k + s * H] : 0.0;
+          }
+    int ex[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) ex[c] = (int)(sh.emax[c * MM_LINES + line] >> 20);
+    __syncthreads();
+    const int pitchw = (p.Kp + 8) / 2;  // words per column
+    uint32_t* dig = reinterpret_cast<uint32_t*>(dyn);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int q = q0 + r * TS;
+      if (2 * q < p.Kp) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          long long w[S][2];
+#pragma unroll
+          for (int a = 0; a < 2; ++a) {
+            const long long x0 = sp_fixed(X[r][c][0][a], ex[c]);
+            if (S == 2) {
+              const long long x1 = sp_fixed(X[r][c][S - 1][a], ex[c]);
+              w[0][a] = x0 + x1 + SP_BIAS;
+              w[S - 1][a] = x0 - x1 + SP_BIAS;
+            } else {
+              w[0][a] = x0 + SP_BIAS;
+            }
+          }
+#pragma unroll
+          for (int s = 0; s < S; ++s)
+#pragma unroll
+            for (int k = 0; k < SP_DIGITS; ++k)
+              dig[((s * SP_DIGITS + k) * NCOL + c * MM_LINES + line) * pitchw + q] = digit_pair(w[s][0], w[s][1], k);
+        }
       }
     }
   }
@@ -336,20 +372,23 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& p, Mm
 #pragma unroll
     for (int half = 0; half < S; ++half) {
       if constexpr (!PT) {
-        typename Ep::Op op[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = i0 + g + 8 * (q >> 2), idx = i + half * H;
-          const int col = ((q >> 1) & 1) * 8 + 2 * t + (q & 1), ln = col & (MM_LINES - 1);
-          op[q] = ep.pre(col / MM_LINES, point(sh, ln, i < H && idx < n ? idx : 0));
-        }
+        for (int r = 0; r < 2; ++r) {  // rows g and g + 8: operands of four results in flight
+          const int i = i0 + g + 8 * r, idx = i + half * H;
+          const bool in = i < H && idx < n;
+          typename Ep::Op op[4];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = i0 + g + 8 * (q >> 2), idx = i + half * H;
-          const int col = ((q >> 1) & 1) * 8 + 2 * t + (q & 1), ln = col & (MM_LINES - 1);
-          const long long y = S == 1 ? W[0][q] : (half ? W[0][q] - W[S - 1][q] : W[0][q] + W[S - 1][q]);
-          if (i < H && idx < n && sh.J[ln].n > 0)
-            ep.put(col / MM_LINES, point(sh, ln, idx), op[q], sp_double(y) * sh.fac[col]);
+          for (int q = 0; q < 4; ++q) {
+            const int col = (q >> 1) * 8 + 2 * t + (q & 1);
+            op[q] = ep.pre(col / MM_LINES, point(sh, col & (MM_LINES - 1), in ? idx : 0));
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int col = (q >> 1) * 8 + 2 * t + (q & 1), ln = col & (MM_LINES - 1);
+            const long long w0 = W[0][4 * r + q], w1 = W[S - 1][4 * r + q];
+            const long long y = S == 1 ? w0 : (half ? w0 - w1 : w0 + w1);
+            if (in && sh.J[ln].n > 0) ep.put(col / MM_LINES, point(sh, ln, idx), op[q], sp_double(y) * sh.fac[col]);
+          }
         }
       } else {
         // lanes t and t ^ 2 hold components (0, 2) and (1, 3) of the same lines and rows:
