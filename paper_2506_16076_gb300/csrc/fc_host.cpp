@@ -93,7 +93,8 @@ struct fc_ctx {
   std::string err;
   fc_params prm{};
   std::vector<double> fctab;  // copy of the packed tables
-  std::vector<float> sdnn;
+  SdnnW sdnn{};
+  WindowW wtab{};
   int d = 5, Cmin = 0, Cmax = -1;
   std::vector<HPatch> hp;
   long long P = 0, Pg = 0, active = 0;
@@ -119,9 +120,7 @@ struct fc_ctx {
   uint32_t* d_info = nullptr;
   PatchDev* d_patches = nullptr;
   double* d_J = nullptr;
-  float* d_sdnn = nullptr;
   double* d_R = nullptr;
-  double* d_wtab = nullptr;
 
   // job queues: [pass] -> batched order (length-descending, split by length class) and per-patch ranges
   struct Queue {
@@ -1137,7 +1136,7 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
     return bad("SDNN weights missing or of the wrong size");
   if (prm->win_r < 1 || prm->win_r > 32 || prm->n_f < 1 || prm->n_v < 1 || prm->depth_cap < 2) return bad("bad params");
   if (prm->wall_form != 0 && prm->wall_form != 1) return bad("wall_form must be 0 or 1");
-  c->sdnn.assign(prm->sdnn_w, prm->sdnn_w + prm->sdnn_len);
+  std::copy(prm->sdnn_w, prm->sdnn_w + prm->sdnn_len, c->sdnn.w);
   if (prm->freestream[0] > 0.0) {  // d e_fs / d(M, alpha) at fixed rho and p (eq. mach_flow_ic)
     const double rho = prm->freestream[0], u = prm->freestream[1], v = prm->freestream[2];
     const double pr = prm->freestream[3];
@@ -1554,11 +1553,10 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   }
 
   // ---- viscosity windows, cross-patch nearest points (eqs. W, multipatch_W, zeta)
-  std::vector<double> wtab(2 * prm->win_r - 1);
   for (int a = -(prm->win_r - 1); a <= prm->win_r - 1; ++a) {
     const long double t = std::fabs((long double)a);
     const long double cc = cosl(3.14159265358979323846264338327950288L * t / (2.0L * prm->win_r));
-    wtab[a + prm->win_r - 1] = (double)(cc * cc);
+    c->wtab.w[a + prm->win_r - 1] = (double)(cc * cc);
   }
   std::vector<int> cdst, cptr{0}, csrc;
   for (int p = 0; p < npatch; ++p) {
@@ -1681,7 +1679,7 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
        c->upload(&c->d_plans, B.plans) && c->upload(&c->d_tw, B.tw) && c->upload(&c->d_rp, B.rp) &&
        c->upload(&c->d_ip, B.ip) &&
        c->upload(&c->d_info, info) && c->upload(&c->d_patches, pdev) && c->upload(&c->d_J, Jm) &&
-       c->upload(&c->d_sdnn, c->sdnn) && c->upload(&c->d_R, Rv) && c->upload(&c->d_wtab, wtab) &&
+       c->upload(&c->d_R, Rv) &&
        c->upload(&c->d_fix, fix) && c->upload(&c->d_fyfix, fyfix) && c->upload(&c->d_gfix, gfix) &&
        c->upload(&c->d_fcopy1, fc1) && c->upload(&c->d_fcopy2, fc2) &&
        c->upload(&c->d_bc, bcs) && c->upload(&c->d_walls, walls) && c->upload(&c->d_recv, rinterp) &&
@@ -1793,9 +1791,9 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
     // the generation indicator goes through mu^'s buffer, the unit divisor through phi's
     cudaMemcpy(c->d_muhat, ind.data(), ind.size() * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy(c->d_phi, ones.data(), ones.size() * sizeof(double), cudaMemcpyHostToDevice);
-    launch_window_rows(T, c->d_muhat, c->d_tmp, c->d_wtab, prm->win_r, 0);
-    launch_window_cols(T, c->d_tmp, c->d_num, c->d_wtab, prm->win_r, 0);
-    launch_mu_final(T, c->d_num, c->d_phi, c->d_cross_dst, c->d_cross_ptr, c->d_cross_src, c->ncross, c->d_den, 0);
+    launch_window_rows(T, c->d_muhat, c->d_tmp, c->wtab, prm->win_r, 0);
+    launch_window_cols(T, c->d_tmp, c->d_num, c->wtab, prm->win_r, c->d_phi, c->d_den, 0);
+    launch_mu_cross(c->d_num, c->d_phi, c->d_cross_dst, c->d_cross_ptr, c->d_cross_src, c->ncross, c->d_den, 0);
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
       fprintf(stderr, "fc_init_patches: %s\n", cudaGetErrorString(e));
@@ -1986,9 +1984,10 @@ void viscosity(fc_ctx* c, const double* e, double* mu, int32_t* tau, cudaStream_
   Prof pr(c, st, "viscosity");
   const DevTables& T = c->T;
   launch_visc_point(T, e, c->d_phi, c->d_S, st);
-  launch_visc_muhat(T, c->d_phi, c->d_S, c->d_sdnn, c->d_R, c->d_muhat, tau, st);
-  launch_window_rows(T, c->d_muhat, c->d_tmp, c->d_wtab, c->prm.win_r, st);
-  launch_window_cols(T, c->d_tmp, c->d_num, c->d_wtab, c->prm.win_r, st);
+  // (the maxima of S along q1 go through the window pass's buffer)
+  launch_visc_muhat(T, c->d_phi, c->d_S, (long long*)c->d_tmp, c->sdnn, c->d_R, c->d_muhat, tau, st);
+  launch_window_rows(T, c->d_muhat, c->d_tmp, c->wtab, c->prm.win_r, st);
+  launch_window_cols(T, c->d_tmp, c->d_num, c->wtab, c->prm.win_r, c->d_den, mu, st);
   if (c->sharded()) {  // window sums of other ranks' patches that the cross-patch sums read
     fc_ctx::XPlan& x = c->xp_visc;
     launch_gather(c->d_vsend, x.nsend, c->d_num, x.d_sbuf, st);
@@ -1997,7 +1996,7 @@ void viscosity(fc_ctx* c, const double* e, double* mu, int32_t* tau, cudaStream_
     launch_scatter(c->d_vrecv, x.nrecv, x.d_rbuf, c->d_num, st);
     c->launches += (x.nsend > 0) + (x.nrecv > 0);
   }
-  launch_mu_final(T, c->d_num, c->d_den, c->d_cross_dst, c->d_cross_ptr, c->d_cross_src, c->ncross, mu, st);
+  launch_mu_cross(c->d_num, c->d_den, c->d_cross_dst, c->d_cross_ptr, c->d_cross_src, c->ncross, mu, st);
   c->launches += 5 + (c->ncross > 0);
 }
 

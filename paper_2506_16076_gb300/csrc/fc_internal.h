@@ -164,6 +164,14 @@ struct DevTables {
 
 // ---- launch wrappers of the contraction kernels (fc_mma.cu) ----
 // tiles: MM_LINES jobs each, of one plan (absent lines: n = 0), all of padded inner length
+// kernel parameters: the classifier's FP32 weights, and the window weights (2 win_r - 1 <= 63)
+struct SdnnW {
+  float w[16 * 7 + 16 + 16 * 16 + 16 + 4 * 16 + 4];
+};
+struct WindowW {
+  double w[64];
+};
+
 // Kp <= kp; two: even lengths
 struct MmTiles {
   const Job* jobs;
@@ -227,12 +235,15 @@ void launch_filter_q2(const DevTables& T, const Job* jobs, int njobs, int Lmax, 
 void launch_filter_copy_q1(const DevTables& T, const int* idx, int n, const double* e, double* F, cudaStream_t st);
 void launch_filter_copy_q2(const DevTables& T, const int* idx, int n, const double* F, double* e, cudaStream_t st);
 void launch_visc_point(const DevTables& T, const double* e, double* phi, double* S, cudaStream_t st);
-void launch_visc_muhat(const DevTables& T, const double* phi, const double* S, const float* w, const double* R,
-                       double* muhat, int32_t* tau, cudaStream_t st);
-void launch_window_rows(const DevTables& T, const double* in, double* out, const double* wtab, int r, cudaStream_t st);
-void launch_window_cols(const DevTables& T, const double* in, double* out, const double* wtab, int r, cudaStream_t st);
-void launch_mu_final(const DevTables& T, const double* num, const double* den, const int* cross_dst,
-                     const int* cross_ptr, const int* cross_src, int ncross, double* mu, cudaStream_t st);
+// S7: scratch for the maxima of S along q1
+void launch_visc_muhat(const DevTables& T, const double* phi, const double* S, long long* S7, const SdnnW& w,
+                       const double* R, double* muhat, int32_t* tau, cudaStream_t st);
+void launch_window_rows(const DevTables& T, const double* in, double* out, const WindowW& w, int r, cudaStream_t st);
+// mu (nullable): own window sum / den as well
+void launch_window_cols(const DevTables& T, const double* in, double* out, const WindowW& w, int r, const double* den,
+                        double* mu, cudaStream_t st);
+void launch_mu_cross(const double* num, const double* den, const int* cross_dst, const int* cross_ptr,
+                     const int* cross_src, int ncross, double* mu, cudaStream_t st);
 void launch_dt(const DevTables& T, const double* e, const double* mu, unsigned long long* pmax, double cfl,
                double* dt, cudaStream_t st);
 void launch_check_state(const DevTables& T, const double* e, int* flag, cudaStream_t st);

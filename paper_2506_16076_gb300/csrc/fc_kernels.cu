@@ -14,6 +14,7 @@
 #include "fc_internal.h"
 #include "fc_line.cuh"
 #include "fc_point.cuh"
+#include "fc_split.cuh"
 
 namespace fcx {
 
@@ -880,20 +881,54 @@ __global__ void k_visc_point(DevTables T, const double* __restrict__ e, double* 
   S[p] = __dadd_rn(__dadd_rn(fabs(u), fabs(v)), __dsqrt_rn(__ddiv_rn(__dmul_rn(gam, pr), rho)));
 }
 
-__device__ __forceinline__ int classify7(const double* w, const float* __restrict__ W) {
+// position of a flat index in its patch (a patch has fewer than 2^31 points: 32-bit division)
+__device__ __forceinline__ void locate(const PatchDev& pd, long long p, int& i, int& j) {
+  const uint32_t loc = (uint32_t)(p - pd.off);
+  j = (int)(loc / (uint32_t)pd.n1);
+  i = (int)(loc - (uint32_t)j * (uint32_t)pd.n1);
+}
+
+// a window whose values may be anything: true when it is flat (class 4), else normalised into x
+__device__ __noinline__ bool flat_or_normalised(const double* w, float* x) {
   double lo = w[0], hi = w[0], am = fabs(w[0]);
-#pragma unroll
   for (int k = 1; k < 7; ++k) {
     lo = fmin(lo, w[k]);
     hi = fmax(hi, w[k]);
     am = fmax(am, fabs(w[k]));
   }
   const double rg = __dsub_rn(hi, lo);
-  if (rg < __dmul_rn(1e-6, fmax(1.0, am))) return 4;
-  float x[7];
-#pragma unroll
+  if (rg < __dmul_rn(1e-6, fmax(1.0, am))) return true;
   for (int k = 0; k < 7; ++k) x[k] = __double2float_rn(__ddiv_rn(__dsub_rn(w[k], lo), rg));
-  const float* W1 = W;
+  return false;
+}
+
+// Smoothness class of a 7-point window. The normalised values x_k = (w_k - lo) / (hi - lo)
+// are FP64 quotients rounded to FP32; FP64 operations bound this kernel (a warp's takes 64
+// clocks, a division about six of them), so one reciprocal serves all seven (quotient_f32),
+// and the extrema run on the bit patterns of the non-negative values.
+__device__ __forceinline__ int classify7(const double* w, const SdnnW& N) {
+  float x[7];
+  long long lo = __double_as_longlong(w[0]), hi = lo;
+#pragma unroll
+  for (int k = 1; k < 7; ++k) {
+    const long long b = __double_as_longlong(w[k]);
+    lo = b < lo ? b : lo;
+    hi = b > hi ? b : hi;
+  }
+  if (lo < 0 || hi >= 0x7ff0000000000000ll) {
+    if (flat_or_normalised(w, x)) return 4;
+  } else {
+    const double l = __longlong_as_double(lo), h = __longlong_as_double(hi);
+    const double rg = __dsub_rn(h, l);
+    const double tol = __dmul_rn(1e-6, hi > 0x3ff0000000000000ll ? h : 1.0);
+    if (__double_as_longlong(rg) < __double_as_longlong(tol)) return 4;
+    const double r = __drcp_rn(rg);
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+      x[k] = quotient_f32(__dsub_rn(w[k], l), rg, r);
+    }
+  }
+  const float* W1 = N.w;
   const float* b1 = W1 + SDNN_H * 7;
   const float* W2 = b1 + SDNN_H;
   const float* b2 = W2 + SDNN_H * SDNN_H;
@@ -930,10 +965,37 @@ __device__ __forceinline__ int classify7(const double* w, const float* __restric
   return best + 1;
 }
 
-// mu^ = R(tau~) max_{7x7} S h^ on generating points, 0 elsewhere (eq. V2D_unscaled)
-__global__ void k_visc_muhat(DevTables T, const double* __restrict__ phi, const double* __restrict__ S,
-                             const float* __restrict__ W, const double* __restrict__ Rw, double* __restrict__ muhat,
-                             int32_t* __restrict__ tau) {
+// 7-point maximum of S along q1 (clipped to the grid, wrapped along a periodic q1); S >= 0,
+// so the IEEE bit patterns order like the values and the maximum runs on integer compares
+__global__ void k_visc_rowmax(DevTables T, const double* __restrict__ S, long long* __restrict__ S7) {
+  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= T.P) return;
+  const PatchDev pd = T.patches[pt_patch(T.info[p])];
+  int i, j;
+  locate(pd, p, i, j);
+  long long mb = 0;
+#pragma unroll
+  for (int a = -3; a <= 3; ++a) {
+    long long q = p + a;
+    if (pd.periodic1) {
+      q += i + a < 0 ? pd.n1 : (i + a >= pd.n1 ? -pd.n1 : 0);
+      if (pd.n1 < 3) q = p - i + ((i + a) % pd.n1 + pd.n1) % pd.n1;
+    } else {
+      q = i + a < 0 || i + a >= pd.n1 ? p : q;  // the point itself is always in
+    }
+    const long long bits = __double_as_longlong(S[q]);
+    mb = bits > mb ? bits : mb;
+  }
+  S7[p] = mb;
+}
+
+// mu^ = R(tau~) max_{7x7} S h^ on generating points, 0 elsewhere (eq. V2D_unscaled); S7:
+// the maxima along q1. The classifier's weights are kernel parameters (constant bank: an
+// FMA reads them as an operand).
+__global__ void __launch_bounds__(128) k_visc_muhat(DevTables T, const double* __restrict__ phi,
+                                                    const long long* __restrict__ S7, const __grid_constant__ SdnnW W,
+                                                    const double* __restrict__ Rw, double* __restrict__ muhat,
+                                                    int32_t* __restrict__ tau) {
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= T.P) return;
   const uint32_t f = T.info[p];
@@ -943,93 +1005,99 @@ __global__ void k_visc_muhat(DevTables T, const double* __restrict__ phi, const 
     return;
   }
   const PatchDev pd = T.patches[pt_patch(f)];
-  const long long loc = p - pd.off;
-  const int j = (int)(loc / pd.n1), i = (int)(loc - (long long)j * pd.n1);
-  int t1 = 4, t2 = 4;
-  double w[7];
-  const int o1 = pt_w1(f), o2 = pt_w2(f);
-  if (o1 != 7) {
+  int i, j;
+  locate(pd, p, i, j);
+  int tc = 4;
+#pragma unroll 1
+  for (int dir = 0; dir < 2; ++dir) {
+    const int o = dir ? pt_w2(f) : pt_w1(f);
+    if (o == 7) continue;
+    double w[7];
 #pragma unroll
     for (int k = 0; k < 7; ++k) {
-      int ii = i - o1 + k;
-      if (pd.periodic1) ii = (ii + pd.n1) % pd.n1;
-      w[k] = phi[pd.off + (long long)j * pd.n1 + ii];
-    }
-    t1 = classify7(w, W);
-  }
-  if (o2 != 7) {
-#pragma unroll
-    for (int k = 0; k < 7; ++k) w[k] = phi[pd.off + (long long)(j - o2 + k) * pd.n1 + i];
-    t2 = classify7(w, W);
-  }
-  const int tc = min(t1, t2);
-  // 7x7 maximum of S (clipped to the grid, wrapped along a periodic q1); S >= 0, so the
-  // IEEE bit patterns order like the values and the maximum runs on integer compares
-  long long mb = 0;
-  for (int b = -3; b <= 3; ++b) {
-    const int jj = j + b;
-    if (jj < 0 || jj >= pd.n2) continue;
-    for (int a = -3; a <= 3; ++a) {
-      int ii = i + a;
-      if (pd.periodic1) {
-        ii = (ii + pd.n1) % pd.n1;
-      } else if (ii < 0 || ii >= pd.n1) {
-        continue;
+      long long q;
+      if (dir) {
+        q = p + (long long)(k - o) * pd.n1;
+      } else {
+        int ii = i - o + k;
+        if (pd.periodic1) ii = (ii + pd.n1) % pd.n1;
+        q = p - i + ii;
       }
-      const long long bits = __double_as_longlong(S[pd.off + (long long)jj * pd.n1 + ii]);
-      mb = bits > mb ? bits : mb;
+      w[k] = phi[q];
     }
+    tc = min(tc, classify7(w, W));
+  }
+  long long mb = 0;
+#pragma unroll
+  for (int b = -3; b <= 3; ++b) {
+    const long long bits = S7[j + b < 0 || j + b >= pd.n2 ? p : p + (long long)b * pd.n1];
+    mb = bits > mb ? bits : mb;
   }
   muhat[p] = __dmul_rn(__dmul_rn(Rw[tc - 1], __longlong_as_double(mb)), pd.hhat);
   if (tau) tau[p] = tc;
 }
 
-// separable window sums of eq. (Lambda): rows (q1) then columns (q2), zero outside, wrapped if periodic
-__global__ void k_window_rows(DevTables T, const double* __restrict__ in, double* __restrict__ out,
-                              const double* __restrict__ wtab, int r) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= T.P) return;
-  const PatchDev pd = T.patches[pt_patch(T.info[p])];
-  const long long loc = p - pd.off;
-  const int j = (int)(loc / pd.n1), i = (int)(loc - (long long)j * pd.n1);
-  const double* row = in + pd.off + (long long)j * pd.n1;
+// one point's window sum over taps at p + a step, a = -(r-1)..r-1, in that order. mu^ is
+// zero over most of the domain: a tap that is zero on the whole warp leaves the sum as it
+// is and is passed over, and so is the FP64 work of such a window.
+template <class At>
+__device__ __forceinline__ double window_sum(const WindowW& w, int r, At at) {
   double acc = 0.0;
-  for (int a = -(r - 1); a <= r - 1; ++a) {
-    int ii = i + a;
-    if (pd.periodic1) {
-      ii = (ii + pd.n1) % pd.n1;
-    } else if (ii < 0 || ii >= pd.n1) {
-      continue;
-    }
-    acc = fma(wtab[a + r - 1], row[ii], acc);
+  for (int a0 = -(r - 1); a0 <= r - 1; a0 += 8) {
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = a0 + k <= r - 1 ? at(a0 + k) : 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (__any_sync(0xffffffffu, v[k] != 0.0)) acc = fma(w.w[a0 + k + r - 1], v[k], acc);
   }
-  out[p] = acc;
+  return acc;
 }
 
-__global__ void k_window_cols(DevTables T, const double* __restrict__ in, double* __restrict__ out,
-                              const double* __restrict__ wtab, int r) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= T.P) return;
+// separable window sums of eq. (Lambda): rows (q1) then columns (q2), zero outside, wrapped if periodic
+__global__ void k_window_rows(DevTables T, const double* __restrict__ in, double* __restrict__ out,
+                              const __grid_constant__ WindowW w, int r) {
+  const long long p0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long p = p0 < T.P ? p0 : T.P - 1;
   const PatchDev pd = T.patches[pt_patch(T.info[p])];
-  const long long loc = p - pd.off;
-  const int j = (int)(loc / pd.n1), i = (int)(loc - (long long)j * pd.n1);
-  double acc = 0.0;
-  for (int b = -(r - 1); b <= r - 1; ++b) {
-    const int jj = j + b;
-    if (jj < 0 || jj >= pd.n2) continue;
-    acc = fma(wtab[b + r - 1], in[pd.off + (long long)jj * pd.n1 + i], acc);
-  }
+  int i, j;
+  locate(pd, p, i, j);
+  const double acc = window_sum(w, r, [&](int a) {
+    int ii = i + a;
+    if (pd.periodic1) {
+      if (ii < 0 || ii >= pd.n1) ii = (ii % pd.n1 + pd.n1) % pd.n1;
+    } else if (ii < 0 || ii >= pd.n1) {
+      return 0.0;
+    }
+    return in[p - i + ii];
+  });
+  if (p0 < T.P) out[p] = acc;
+}
+
+// columns; with mu, also mu = own window sum / normaliser (the points that other patches
+// contribute to are redone by k_mu_cross)
+__global__ void k_window_cols(DevTables T, const double* __restrict__ in, double* __restrict__ out,
+                              const __grid_constant__ WindowW w, int r, const double* __restrict__ den,
+                              double* __restrict__ mu) {
+  const long long p0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long p = p0 < T.P ? p0 : T.P - 1;
+  const uint32_t f = T.info[p];
+  const PatchDev pd = T.patches[pt_patch(f)];
+  int i, j;
+  locate(pd, p, i, j);
+  const double acc = window_sum(w, r, [&](int b) {
+    return j + b < 0 || j + b >= pd.n2 ? 0.0 : in[p + (long long)b * pd.n1];
+  });
+  if (p0 >= T.P) return;
   out[p] = acc;
+  if (mu) {
+    const double d = den[p];
+    mu[p] = ((f & PT_BLANK) || !(d > 0.0) || acc == 0.0) ? 0.0 : acc / d;
+  }
 }
 
 // mu = (own window sum + window sums of the other patches at their nearest points) / normaliser
-__global__ void k_mu_own(DevTables T, const double* __restrict__ num, const double* __restrict__ den,
-                         double* __restrict__ mu) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= T.P) return;
-  const double d = den[p];
-  mu[p] = ((T.info[p] & PT_BLANK) || !(d > 0.0)) ? 0.0 : num[p] / d;
-}
+// at the points with contributions of other patches
 __global__ void k_mu_cross(const double* __restrict__ num, const double* __restrict__ den, const int* __restrict__ dst,
                            const int* __restrict__ ptr, const int* __restrict__ src, int n, double* __restrict__ mu) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2077,21 +2145,20 @@ void launch_filter_copy_q2(const DevTables& T, const int* idx, int n, const doub
 void launch_visc_point(const DevTables& T, const double* e, double* phi, double* S, cudaStream_t st) {
   k_visc_point<<<grid_pts(T.P, 256), 256, 0, st>>>(T, e, phi, S);
 }
-void launch_visc_muhat(const DevTables& T, const double* phi, const double* S, const float* w, const double* R,
-                       double* muhat, int32_t* tau, cudaStream_t st) {
-  k_visc_muhat<<<grid_pts(T.P, 128), 128, 0, st>>>(T, phi, S, w, R, muhat, tau);
+void launch_visc_muhat(const DevTables& T, const double* phi, const double* S, long long* S7, const SdnnW& w,
+                       const double* R, double* muhat, int32_t* tau, cudaStream_t st) {
+  k_visc_rowmax<<<grid_pts(T.P, 256), 256, 0, st>>>(T, S, S7);
+  k_visc_muhat<<<grid_pts(T.P, 128), 128, 0, st>>>(T, phi, S7, w, R, muhat, tau);
 }
-void launch_window_rows(const DevTables& T, const double* in, double* out, const double* wtab, int r,
-                        cudaStream_t st) {
-  k_window_rows<<<grid_pts(T.P, 256), 256, 0, st>>>(T, in, out, wtab, r);
+void launch_window_rows(const DevTables& T, const double* in, double* out, const WindowW& w, int r, cudaStream_t st) {
+  k_window_rows<<<grid_pts(T.P, 256), 256, 0, st>>>(T, in, out, w, r);
 }
-void launch_window_cols(const DevTables& T, const double* in, double* out, const double* wtab, int r,
-                        cudaStream_t st) {
-  k_window_cols<<<grid_pts(T.P, 256), 256, 0, st>>>(T, in, out, wtab, r);
+void launch_window_cols(const DevTables& T, const double* in, double* out, const WindowW& w, int r, const double* den,
+                        double* mu, cudaStream_t st) {
+  k_window_cols<<<grid_pts(T.P, 256), 256, 0, st>>>(T, in, out, w, r, den, mu);
 }
-void launch_mu_final(const DevTables& T, const double* num, const double* den, const int* cross_dst,
-                     const int* cross_ptr, const int* cross_src, int ncross, double* mu, cudaStream_t st) {
-  k_mu_own<<<grid_pts(T.P, 256), 256, 0, st>>>(T, num, den, mu);
+void launch_mu_cross(const double* num, const double* den, const int* cross_dst, const int* cross_ptr,
+                     const int* cross_src, int ncross, double* mu, cudaStream_t st) {
   if (ncross > 0) k_mu_cross<<<grid_pts(ncross, 256), 256, 0, st>>>(num, den, cross_dst, cross_ptr, cross_src, ncross, mu);
 }
 void launch_dt(const DevTables& T, const double* e, const double* mu, unsigned long long* pmax, double cfl, double* dt,

@@ -92,4 +92,28 @@ FC_HD double sp_double(long long v) {
 #endif
 }
 
+// The FP64 quotient df / rg rounded to FP32 (0 <= df <= rg, both finite, r = 1 / rg rounded):
+// t = df r is within 2.5 ulp of the rounded quotient and rounds to the same FP32 number
+// unless its low 29 bits lie that close to the midpoint of two FP32 numbers, where the
+// division itself decides (as it does for quotients below 2^-100). The rounding runs on the
+// bit pattern: conversions, too, occupy the FP64 pipe.
+FC_HD float quotient_f32(double df, double rg, double r) {
+  const double t = df * r;
+  const uint32_t hi = sp_hi(t), lo = sp_lo(t);
+  const uint64_t b = ((uint64_t)hi << 32) | lo;
+  const int low = (int)(lo & 0x1fffffffu) - 0x10000000;
+  const uint32_t f = (uint32_t)((b >> 29) + ((b >> 28) & 1u)) - (896u << 23);
+  float x;
+#ifdef __CUDA_ARCH__
+  x = __uint_as_float(f);
+#else
+  memcpy(&x, &f, 4);
+#endif
+  if (b == 0)
+    x = 0.f;
+  else if ((low >= -4 && low <= 4) || (hi >> 20) < 1023u - 100u)
+    x = (float)(df / rg);
+  return x;
+}
+
 }  // namespace fcx

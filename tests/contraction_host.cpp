@@ -6,8 +6,13 @@
 //     constant one and one with a spike against the same circulant in long double; prints
 //     "L op kind error/max|x| largest_level_sum" (op 0: derivative, 1: filter), or "L none"
 //     when lines of this length are left to the FFT kernels.
+//
+//   contraction_host quotient
+//     quotient_f32 against the FP64 division rounded to FP32, on random quotients and on
+//     quotients placed around the rounding midpoints; prints "tested different".
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <random>
 
 #include "../paper_2506_16076_gb300/csrc/fc_mmtab.h"
@@ -20,7 +25,38 @@ static double half_value(unsigned h) {
   return (h >> 15) & 1 ? -v : v;
 }
 
+static int quotients() {
+  std::mt19937_64 g(7);
+  std::uniform_real_distribution<double> U(0.0, 1.0);
+  long long n = 0, bad = 0;
+  auto check = [&](double df, double rg) {
+    const volatile double q = df / rg;
+    const float a = quotient_f32(df, rg, 1.0 / rg), b = (float)q;
+    ++n;
+    bad += std::memcmp(&a, &b, 4) != 0;
+  };
+  for (int k = 0; k < 2000000; ++k) {
+    const double rg = std::ldexp(1.0 + U(g), (int)(40 * U(g)) - 20);
+    check(U(g) * rg, rg);
+    // a quotient a few ulp around the midpoint of two FP32 numbers, and around one of them
+    const float f = (float)std::ldexp(0.5 + 0.5 * U(g), -(int)(60 * U(g)));
+    const double mid = 0.5 * ((double)f + (double)std::nextafter(f, 2.f));
+    for (int u = -3; u <= 3; ++u) {
+      check(std::min(rg, std::ldexp(std::nearbyint(std::ldexp(mid, 60)), -60) * rg * (1.0 + u * 1.1e-16)), rg);
+      check(std::min(rg, (double)f * rg * (1.0 + u * 1.1e-16)), rg);
+    }
+    if (k < 1000) {
+      check(0.0, rg);
+      check(rg, rg);
+      check(std::ldexp(rg, -200 - k / 2), rg);
+    }
+  }
+  printf("%lld %lld\n", n, bad);
+  return 0;
+}
+
 int main(int argc, char** argv) {
+  if (argc == 2 && !std::strcmp(argv[1], "quotient")) return quotients();
   std::mt19937_64 g(1);
   std::uniform_real_distribution<double> U(-1.0, 1.0);
   const long double PI = 3.14159265358979323846264338327950288L;

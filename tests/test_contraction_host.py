@@ -48,3 +48,10 @@ def test_contraction_matches_the_circulant(exe):
 def test_other_lengths_are_left_to_the_transforms(exe):
     r = subprocess.run([exe, "15", "257", "514", "1024"], capture_output=True, text=True)
     assert r.returncode == 0 and [ln.split()[1] for ln in r.stdout.splitlines()] == ["none"] * 4
+
+
+def test_quotients_round_as_the_division(exe):
+    # the classifier's normalised values (bit for bit)
+    r = subprocess.run([exe, "quotient"], capture_output=True, text=True, timeout=600)
+    n, bad = map(int, r.stdout.split())
+    assert r.returncode == 0 and n > 10 ** 7 and bad == 0, (n, bad)
