@@ -889,11 +889,11 @@ struct Builder {
   }
 
   // the FMA-form records of p (fc_tables.h): inverse, then forward with the filter table
-  void fma_tables(Plan& p) {
-    fma_inverse_records(p, tw);
+  void fma_tables(Plan& p, const Trig& tg) {
+    fma_inverse_records(p, tg, tw);
     const std::vector<int> rev(ip.begin() + p.rev, ip.begin() + p.rev + p.L);
     const std::vector<double> sig(rp.begin() + p.sig, rp.begin() + p.sig + p.L);
-    fma_forward_records(p, tw, rp, rev.data(), sig.data());
+    fma_forward_records(p, tg, tw, rp, rev.data(), sig.data());
   }
 
   int plan(int L) {
@@ -906,13 +906,8 @@ struct Builder {
     p.nst = (int)f.size();
     for (int s = 0; s < p.nst; ++s) p.rad[s] = f[s];
     p.tw = (int)tw.size();
-    for (int e = 0; e < L; ++e) {
-      const long double ang = -2.0L * 3.14159265358979323846264338327950288L * (long double)e / (long double)L;
-      double2 w;
-      w.x = (double)cosl(ang);
-      w.y = (double)sinl(ang);
-      tw.push_back(w);
-    }
+    const Trig tg(L);
+    for (int e = 0; e < L; ++e) tw.push_back(table_pair(tg.c[e], -tg.s[e]));
     rev_table(p);
     p.sig = (int)rp.size();
     const fc_params& prm = c->prm;
@@ -925,7 +920,7 @@ struct Builder {
       rp.push_back((double)(v / (long double)L));
       if (2 * t <= L) sig.push_back(v);
     }
-    fma_tables(p);
+    fma_tables(p, tg);
     plans.push_back(p);
     mm.push_back(mm_length_ok(L) ? mm_plan(L, &sig, mmlo, mmhi) : MmPlan{});
     std::vector<Plan> alt{p};
@@ -935,7 +930,7 @@ struct Builder {
       q.nst = (int)orders[o].size();
       for (int s = 0; s < q.nst; ++s) q.rad[s] = orders[o][s];
       rev_table(q);
-      fma_tables(q);
+      fma_tables(q, tg);
       alt.push_back(q);
     }
     cands.push_back(alt);

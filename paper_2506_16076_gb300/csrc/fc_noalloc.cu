@@ -108,7 +108,10 @@ extern "C" fc_status fc_rhs_patch_noalloc(const double* e_dev, const double* mu_
   std::vector<double2> tw;
   std::vector<int> ip;
   std::vector<Plan> plans(2);
-  for (int k = 0; k < 2; ++k) {
+  std::vector<Trig> tg;
+  const int nplan = L[0] == L[1] ? 1 : 2;  // equal lengths share their tables
+  for (int k = 0; k < nplan; ++k) tg.emplace_back(L[k]);
+  for (int k = 0; k < nplan; ++k) {
     Plan& pl = plans[k];
     std::memset(&pl, 0, sizeof(Plan));
     pl.L = L[k];
@@ -132,14 +135,8 @@ extern "C" fc_status fc_rhs_patch_noalloc(const double* e_dev, const double* mu_
       }
       ip.push_back(mode);
     }
-    for (int e = 0; e < L[k]; ++e) {
-      const long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)e / (long double)L[k];
-      double2 w;
-      w.x = (double)cosl(a);
-      w.y = (double)sinl(a);
-      tw.push_back(w);
-    }
-    fma_inverse_records(pl, tw);
+    for (int e = 0; e < L[k]; ++e) tw.push_back(table_pair(tg[k].c[e], -tg[k].s[e]));
+    fma_inverse_records(pl, tg[k], tw);
   }
   const double* Q = table;
   const double* AL = Q + d * d;
@@ -167,10 +164,11 @@ extern "C" fc_status fc_rhs_patch_noalloc(const double* e_dev, const double* mu_
         }
         rp.push_back((double)s);
       }
-  for (int k = 0; k < 2; ++k) {  // forward records after the continuation matrices (fcm = 0)
+  for (int k = 0; k < nplan; ++k) {  // forward records after the continuation matrices (fcm = 0)
     const std::vector<int> rev(ip.begin() + plans[k].rev, ip.begin() + plans[k].rev + L[k]);
-    fma_forward_records(plans[k], tw, rp, rev.data(), nullptr);
+    fma_forward_records(plans[k], tg[k], tw, rp, rev.data(), nullptr);
   }
+  if (nplan == 1) plans[1] = plans[0];
   if (tw.size() * sizeof(double2) > NA_TW || rp.size() * sizeof(double) > NA_RP) {
     fprintf(stderr, "fc_rhs_patch_noalloc: the transform tables exceed the static scratch\n");
     return FC_ERR_INVALID;

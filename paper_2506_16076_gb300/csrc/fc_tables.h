@@ -41,9 +41,43 @@ namespace fcx {
 constexpr long double TABLE_PI = 3.14159265358979323846264338327950288L;
 constexpr long double TABLE_RSQRT2 = 0.70710678118654752440084436210484903928L;
 
-// ratio form of exp(i ang): S, t and the flag
-inline void ratio_form(long double ang, long double& S, long double& t, bool& flag) {
-  const long double c = cosl(ang), s = sinl(ang);
+// cos and sin of 2 pi e / L, e = 0..L-1. Every table of a length reads them here: the
+// long double functions cost about a microsecond each where long double has no hardware
+// (113 bits in software), and a plan's records ask for about ten times L of them. Symmetry
+// leaves L/8 + 1 evaluations (L/4 + 1, L/2 + 1 when 8 or 4 do not divide L).
+struct Trig {
+  int L;
+  std::vector<long double> c, s;
+  explicit Trig(int L_) : L(L_), c((size_t)L_), s((size_t)L_) {
+    const int top = L % 8 == 0 ? L / 8 : (L % 4 == 0 ? L / 4 : L / 2);
+    for (int e = 0; e <= top; ++e) {
+      const long double a = 2.0L * TABLE_PI * (long double)e / (long double)L;
+      c[e] = cosl(a);
+      s[e] = sinl(a);
+    }
+    if (L % 4 == 0) s[0] = 0.0L;
+    if (L % 8 == 0)  // the other half of the quadrant
+      for (int e = L / 8 + 1; e <= L / 4; ++e) {
+        c[e] = s[L / 4 - e];
+        s[e] = c[L / 4 - e];
+      }
+    if (L % 4 == 0) {
+      c[L / 4] = 0.0L;
+      s[L / 4] = 1.0L;
+      for (int e = L / 4 + 1; e <= L / 2; ++e) {
+        c[e] = -c[L / 2 - e];
+        s[e] = s[L / 2 - e];
+      }
+    }
+    for (int e = L / 2 + 1; e < L; ++e) {
+      c[e] = c[L - e];
+      s[e] = -s[L - e];
+    }
+  }
+};
+
+// ratio form of exp(i ang) from its cosine and sine: S, t and the flag
+inline void ratio_form(long double c, long double s, long double& S, long double& t, bool& flag) {
   flag = !(fabsl(c) >= fabsl(s));
   if (!flag) {
     S = c;
@@ -70,7 +104,7 @@ inline double flag_word(long long flags) {
 inline bool fma_radix(int R) { return R == 2 || R == 4 || R == 8; }
 
 // records of the inverse transform (appended to tw); sets p.fmd
-inline void fma_inverse_records(Plan& p, std::vector<double2>& tw) {
+inline void fma_inverse_records(Plan& p, const Trig& tg, std::vector<double2>& tw) {
   const int L = p.L;
   p.fmd = (int)tw.size();
   int span = 1;
@@ -84,7 +118,7 @@ inline void fma_inverse_records(Plan& p, std::vector<double2>& tw) {
         for (int q = 1; q < R; ++q) {
           const long long e = ((long long)q * j * tws) % L;
           bool f;
-          ratio_form(2.0L * TABLE_PI * (long double)e / (long double)L, S[q], t[q], f);
+          ratio_form(tg.c[e], tg.s[e], S[q], t[q], f);
           if (f) flags |= 1LL << (q - 1);
         }
         tw.push_back(table_pair(0.0L, t[1]));
@@ -113,8 +147,8 @@ inline void fma_inverse_records(Plan& p, std::vector<double2>& tw) {
 // records of the forward transform (tw) and its scale tables (rp); rev: the plan's slot ->
 // mode table; sig: the filter factor per mode (null: no filter table). Sets p.fmf, p.fmsc,
 // p.psc, p.dmul, p.sigp.
-inline void fma_forward_records(Plan& p, std::vector<double2>& tw, std::vector<double>& rp, const int* rev,
-                                const double* sig) {
+inline void fma_forward_records(Plan& p, const Trig& tg, std::vector<double2>& tw, std::vector<double>& rp,
+                                const int* rev, const double* sig) {
   const int L = p.L;
   std::vector<long double> P((size_t)L, 1.0L);
   p.fmf = (int)tw.size();
@@ -138,10 +172,10 @@ inline void fma_forward_records(Plan& p, std::vector<double2>& tw, std::vector<d
           for (int m = 1; m <= H; ++m) rec.push_back(Pr[m] / Pr[0]);
           for (int q = 1; q <= H; ++q)
             for (int m = 1; m <= H; ++m)
-              rec.push_back(cosl(2.0L * TABLE_PI * (long double)(q * m) / (long double)R) * (Pr[m] / Pr[0]));
+              rec.push_back(tg.c[(size_t)(q * m % R) * (L / R)] * (Pr[m] / Pr[0]));
           for (int q = 1; q <= H; ++q)
             for (int m = 1; m <= H; ++m)
-              rec.push_back(sinl(2.0L * TABLE_PI * (long double)(q * m) / (long double)R) * (Pr[m] / Pr[0]));
+              rec.push_back(tg.s[(size_t)(q * m % R) * (L / R)] * (Pr[m] / Pr[0]));
           if (rec.size() % 2) rec.push_back(0.0L);
           for (size_t i = 0; i < rec.size(); i += 2) tw.push_back(table_pair(rec[i], rec[i + 1]));
         }
@@ -165,7 +199,7 @@ inline void fma_forward_records(Plan& p, std::vector<double2>& tw, std::vector<d
         for (int q = 1; q < R; ++q) {
           const long long e = ((long long)q * j * tws) % L;
           bool f;
-          ratio_form(-2.0L * TABLE_PI * (long double)e / (long double)L, Sj[(size_t)j * R + q], t[q], f);
+          ratio_form(tg.c[e], -tg.s[e], Sj[(size_t)j * R + q], t[q], f);
           if (f) flags |= 1LL << (q - 1);
         }
         tw.push_back(table_pair(0.0L, t[1]));
