@@ -1043,13 +1043,13 @@ __global__ void __launch_bounds__(128) k_visc_muhat(DevTables T, const double* _
 template <class At>
 __device__ __forceinline__ double window_sum(const WindowW& w, int r, At at) {
   double acc = 0.0;
-  for (int a0 = -(r - 1); a0 <= r - 1; a0 += 8) {
-    double v[8];
+  for (int a0 = -(r - 1); a0 <= r - 1; a0 += 6) {  // 17 taps (win_r 9) in three batches of loads
+    double v[6];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = a0 + k <= r - 1 ? at(a0 + k) : 0.0;
+    for (int k = 0; k < 6; ++k) v[k] = a0 + k <= r - 1 ? at(a0 + k) : 0.0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (__any_sync(0xffffffffu, v[k] != 0.0)) acc = fma(w.w[a0 + k + r - 1], v[k], acc);
+    for (int k = 0; k < 6; ++k)  // (an integer test: FP64 compares occupy the FP64 pipe, too)
+      if (__any_sync(0xffffffffu, __double_as_longlong(v[k]) != 0)) acc = fma(w.w[a0 + k + r - 1], v[k], acc);
   }
   return acc;
 }
@@ -1092,7 +1092,7 @@ __global__ void k_window_cols(DevTables T, const double* __restrict__ in, double
   out[p] = acc;
   if (mu) {
     const double d = den[p];
-    mu[p] = ((f & PT_BLANK) || !(d > 0.0) || acc == 0.0) ? 0.0 : acc / d;
+    mu[p] = ((f & PT_BLANK) || !(d > 0.0) || __double_as_longlong(acc) == 0) ? 0.0 : acc / d;
   }
 }
 
@@ -1110,44 +1110,156 @@ __global__ void k_mu_cross(const double* __restrict__ num, const double* __restr
 }
 
 // ---------------------------------------------------------------- time step, eq. (CFL)
-__global__ void k_dt_reduce(DevTables T, const double* __restrict__ e, const double* __restrict__ mu,
-                            unsigned long long* __restrict__ pmax) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  int patch = -1;
-  unsigned long long bs = 0, bm = 0;
-  if (p < T.P) {
-    const uint32_t f = T.info[p];
-    if (!(f & PT_BLANK) && (!T.owned || T.owned[pt_patch(f)])) {
-      patch = pt_patch(f);
-      const long long cs = T.P;
-      const double gam = T.gamma;
-      const double rho = e[p];
-      const double u = __ddiv_rn(e[p + cs], rho);
-      const double v = __ddiv_rn(e[p + 2 * cs], rho);
-      const double s2 = __dadd_rn(__dmul_rn(u, u), __dmul_rn(v, v));
-      const double pr = __dmul_rn(__dsub_rn(gam, 1.0), __dsub_rn(e[p + 3 * cs], __dmul_rn(__dmul_rn(0.5, rho), s2)));
-      const double Sv = __dadd_rn(__dadd_rn(fabs(u), fabs(v)), __dsqrt_rn(__ddiv_rn(__dmul_rn(gam, pr), rho)));
-      bs = (unsigned long long)__double_as_longlong(Sv);
-      bm = (unsigned long long)__double_as_longlong(mu[p]);
-      if (!(Sv >= 0.0)) bs = 0x7FF8000000000000ull;  // NaN: poison the patch maximum
+// S = |u| + |v| + a of one state, explicitly rounded (NaN: a pattern above every number, so
+// that it poisons the patch maximum)
+__device__ __forceinline__ unsigned long long dt_speed(const double* q, double gam) {
+  const double u = __ddiv_rn(q[1], q[0]);
+  const double v = __ddiv_rn(q[2], q[0]);
+  const double s2 = __dadd_rn(__dmul_rn(u, u), __dmul_rn(v, v));
+  const double pr = __dmul_rn(__dsub_rn(gam, 1.0), __dsub_rn(q[3], __dmul_rn(__dmul_rn(0.5, q[0]), s2)));
+  const double S = __dadd_rn(__dadd_rn(fabs(u), fabs(v)), __dsqrt_rn(__ddiv_rn(__dmul_rn(gam, pr), q[0])));
+  return S >= 0.0 ? (unsigned long long)__double_as_longlong(S) : 0x7FF8000000000000ull;
+}
+// x truncated to FP32 without the FP64 pipe; outside its normal range (and for non-finite x): NaN
+__device__ __forceinline__ float dt_float(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t e = (hi >> 20) & 0x7ffu;
+  const uint32_t f = (hi & 0x80000000u) | ((((hi & 0x7fffffffu) << 3) | (lo >> 29)) - (896u << 23));
+  return e > 900 && e < 1140 ? __uint_as_float(f) : ((hi & 0x7fffffffu) | lo) == 0 ? 0.f : __int_as_float(0x7fc00000);
+}
+
+// Largest S and mu of each patch. S takes three divisions and a root, about 35 operations of
+// the FP64 pipe (2 lanes per clock and SM), which bounded this kernel (2.24 ms at 28M points,
+// bandwidth 0.17 ms). FP32 estimates with error bounds now tell which points can hold the
+// maximum: those whose upper bound reaches the block's largest lower bound, or the patch's
+// maximum so far, are evaluated exactly, and a point whose state has the bits of the block's
+// representative (uniform free stream) has its value already. The maximum is that of the
+// exact values as before.
+constexpr int DTB = 256, DTP = 4;  // threads, points per thread
+__global__ void __launch_bounds__(DTB) k_dt_reduce(DevTables T, const double* __restrict__ e,
+                                                   const double* __restrict__ mu,
+                                                   unsigned long long* __restrict__ pmax) {
+  __shared__ float slow[DTB / 32];
+  __shared__ int sidx[DTB / 32];
+  __shared__ unsigned long long rep[5], smax[2];
+  __shared__ bool have_rep;
+  const long long p0 = (long long)blockIdx.x * (DTB * DTP);
+  const long long pl = p0 + DTB * DTP - 1 < T.P ? p0 + DTB * DTP - 1 : T.P - 1;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const long long cs = T.P;
+  const double gam = T.gamma;
+  const int first = pt_patch(T.info[p0]), last = pt_patch(T.info[pl]);
+  if (T.owned && first == last && !T.owned[first]) return;
+  if (tid < 2) smax[tid] = 0;
+  double q[DTP][4];
+  float hi[DTP];
+  int patch[DTP];
+  unsigned long long bm = 0;
+  const bool whole = first == last;
+  const float g1 = (float)gam - 1.f;
+  float low = -1.f;
+  int at = -1;
+#pragma unroll
+  for (int k = 0; k < DTP; ++k) {
+    const long long p = p0 + tid + k * DTB, pc = p < T.P ? p : T.P - 1;
+    const uint32_t f = T.info[pc];
+    patch[k] = p >= T.P || (f & PT_BLANK) || (T.owned && !T.owned[pt_patch(f)]) ? -1 : pt_patch(f);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) q[k][c] = e[pc + c * cs];
+    const unsigned long long m = (unsigned long long)__double_as_longlong(mu[pc]);
+    if (patch[k] >= 0) {
+      if (whole)
+        bm = m > bm ? m : bm;
+      else
+        atomicMax(pmax + 2 * patch[k] + 1, m);
     }
   }
-  const unsigned mask = __activemask();
-  const int p0 = __shfl_sync(mask, patch, 0);
-  if (__all_sync(mask, patch == p0) && p0 >= 0) {
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long s2 = __shfl_down_sync(mask, bs, o);
-      const unsigned long long m2 = __shfl_down_sync(mask, bm, o);
-      bs = s2 > bs ? s2 : bs;
-      bm = m2 > bm ? m2 : bm;
+#pragma unroll
+  for (int k = 0; k < DTP; ++k) {
+    // relative errors: truncated inputs 2^-23, FP32 arithmetic a few 2^-24 per operation; the
+    // pressure loses what E and the kinetic energy share
+    const float r = dt_float(q[k][0]), mx = dt_float(q[k][1]), my = dt_float(q[k][2]), E = dt_float(q[k][3]);
+    const float ir = 1.f / r, u = fabsf(mx * ir), v = fabsf(my * ir);
+    const float ke = 0.5f * (fabsf(mx) * u + fabsf(my) * v), p = g1 * (E - ke);
+    const float a = sqrtf((float)gam * p * ir);
+    const float S = u + v + a, dS = 2e-6f * (u + v) + a * (2e-6f + 2e-6f * g1 * (fabsf(E) + ke) / p);
+    const bool sure = p > 0.f && r > 0.f && dS < 0.25f * S;  // false on NaN too
+    hi[k] = patch[k] < 0 ? -1.f : (sure ? S + dS : INFINITY);
+    if (patch[k] >= 0 && sure && S - dS > low) {
+      low = S - dS;
+      at = tid + k * DTB;
     }
-    if ((threadIdx.x & 31) == 0) {
-      atomicMax(pmax + 2 * p0, bs);
-      atomicMax(pmax + 2 * p0 + 1, bm);
+  }
+  if (!whole) {  // a patch boundary in the block: every point exactly
+#pragma unroll
+    for (int k = 0; k < DTP; ++k)
+      if (patch[k] >= 0) atomicMax(pmax + 2 * patch[k], dt_speed(q[k], gam));
+    return;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float l2 = __shfl_down_sync(0xffffffffu, low, o);
+    const int a2 = __shfl_down_sync(0xffffffffu, at, o);
+    const unsigned long long m2 = __shfl_down_sync(0xffffffffu, bm, o);
+    if (l2 > low) {
+      low = l2;
+      at = a2;
     }
-  } else if (patch >= 0) {
-    atomicMax(pmax + 2 * patch, bs);
-    atomicMax(pmax + 2 * patch + 1, bm);
+    bm = m2 > bm ? m2 : bm;
+  }
+  if (lane == 0) {
+    slow[tid >> 5] = low;
+    sidx[tid >> 5] = at;
+  }
+  __syncthreads();
+  if (lane == 0 && bm) atomicMax(&smax[1], bm);
+  if (tid < 32) {  // the representative: the largest lower bound
+    low = lane < DTB / 32 ? slow[lane] : -1.f;
+    at = lane < DTB / 32 ? sidx[lane] : -1;
+#pragma unroll
+    for (int o = DTB / 64; o > 0; o >>= 1) {
+      const float l2 = __shfl_down_sync(0xffffffffu, low, o);
+      const int a2 = __shfl_down_sync(0xffffffffu, at, o);
+      if (l2 > low) {
+        low = l2;
+        at = a2;
+      }
+    }
+    if (lane == 0) {
+      unsigned long long s = *(volatile unsigned long long*)(pmax + 2 * first);
+      for (int c = 0; c < 4; ++c)
+        rep[c] = at < 0 ? 0 : (unsigned long long)__double_as_longlong(e[p0 + at + c * cs]);
+      if (at >= 0) {
+        const double r4[4] = {__longlong_as_double((long long)rep[0]), __longlong_as_double((long long)rep[1]),
+                              __longlong_as_double((long long)rep[2]), __longlong_as_double((long long)rep[3])};
+        const unsigned long long x = dt_speed(r4, gam);
+        smax[0] = x;
+        s = x > s ? x : s;
+      }
+      have_rep = at >= 0;
+      rep[4] = s;  // a maximum reached already (this block's or the patch's)
+    }
+  }
+  __syncthreads();
+  const unsigned long long have = rep[4];
+  // the reached maximum as FP32, rounded down (a NaN's pattern: nothing exceeds it)
+  const float reached = have >= 0x7ff0000000000000ull ? INFINITY : dt_float(__longlong_as_double((long long)have));
+  unsigned long long bs = 0;
+#pragma unroll
+  for (int k = 0; k < DTP; ++k) {
+    bool same = have_rep;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) same = same && (unsigned long long)__double_as_longlong(q[k][c]) == rep[c];
+    if (patch[k] >= 0 && !same && !(hi[k] < reached)) {
+      const unsigned long long x = dt_speed(q[k], gam);
+      bs = x > bs ? x : bs;
+    }
+  }
+  if (bs) atomicMax(&smax[0], bs);
+  __syncthreads();
+  if (tid == 0) {
+    atomicMax(pmax + 2 * first, smax[0]);
+    atomicMax(pmax + 2 * first + 1, smax[1]);
   }
 }
 
@@ -2164,7 +2276,7 @@ void launch_mu_cross(const double* num, const double* den, const int* cross_dst,
 void launch_dt(const DevTables& T, const double* e, const double* mu, unsigned long long* pmax, double cfl, double* dt,
                cudaStream_t st) {
   cudaMemsetAsync(pmax, 0, sizeof(unsigned long long) * 2 * T.npatch, st);
-  k_dt_reduce<<<grid_pts(T.P, 256), 256, 0, st>>>(T, e, mu, pmax);
+  k_dt_reduce<<<grid_pts(T.P, DTB * DTP), DTB, 0, st>>>(T, e, mu, pmax);
   k_dt_final<<<1, 256, 0, st>>>(T, pmax, cfl, dt);
 }
 
