@@ -136,6 +136,9 @@ struct fc_ctx {
     // other lines, for the FFT kernels
     std::vector<MmTiles> mm;
     std::vector<std::vector<MmTiles>> mmpp;
+    Job* dmm = nullptr;                          // all tiles' jobs: per patch, then batched
+    uint8_t* dvisc = nullptr;                    // their viscous flags (valid while ctx::flags_on)
+    int ntiles = 0;                              // per order
     std::unique_ptr<Queue> rest;
   };
   Queue q_cart1, q_cart2, q_gen1, q_gen2, q_filt1, q_filt2;
@@ -269,6 +272,7 @@ struct fc_ctx {
   cudaEvent_t join_ev[NSIDE] = {nullptr, nullptr, nullptr};
   bool side_ready = false;
   bool concurrent = true;
+  bool flags_on = false;  // the affine queues' viscous flags belong to the current call's mu
   bool ensure_side() {
     if (side_ready) return true;
     for (int k = 0; k < NSIDE; ++k)
@@ -992,12 +996,13 @@ void make_tiles(fc_ctx* c, fc_ctx::Queue& q, const std::vector<Job>& pp, const s
     Job j[MM_LINES];
     int patch, kp, two, cls;
   };
-  static const int top[] = {48, 64, 96, 128, 176, 208, MM_KMAX};
+  static const int top[] = {64, 96, 128, 176, 256, MM_KMAX};
+  constexpr int MM_FEW = 304;
   std::vector<Tile> tiles;
   std::vector<Job> rest;
   for (const Job& J : pp) {
     const MmPlan& m = mm[J.plan];
-    if (m.H == 0 || J.C > 128 || c->d > 8) {
+    if (m.H == 0 || J.C > MM_CMAX || c->d > 8) {
       rest.push_back(J);
       continue;
     }
@@ -1019,23 +1024,41 @@ void make_tiles(fc_ctx* c, fc_ctx::Queue& q, const std::vector<Job>& pp, const s
     while (top[t.cls] < t.kp) ++t.cls;
     tiles.push_back(t);
   }
-  for (Tile& t : tiles)  // absent lines share the plan (the kernel reads it from the first)
+  for (Tile& t : tiles)  // absent lines: the first one's addresses (read, never written) and no points
     for (int l = 1; l < MM_LINES; ++l)
-      if (t.j[l].n == 0) t.j[l].plan = t.j[0].plan;
-  auto put = [&](const std::vector<Tile>& ts, std::vector<MmTiles>& out, std::vector<Job>& flat) {
-    for (size_t k = 0; k < ts.size();) {
-      size_t e = k;
-      MmTiles m{nullptr, 0, 0, ts[k].two};
-      while (e < ts.size() && ts[e].cls == ts[k].cls && ts[e].two == ts[k].two) {
-        m.kp = std::max(m.kp, ts[e].kp);
-        ++e;
+      if (t.j[l].n == 0) {
+        t.j[l] = t.j[0];
+        t.j[l].n = 0;
       }
-      m.n = (int)(e - k);
+  auto put = [&](const std::vector<Tile>& ts, std::vector<MmTiles>& out, std::vector<Job>& flat) {
+    auto shape = [](const Tile& x) { return (x.kp <= 128 ? 0 : (x.kp <= 256 ? 1 : 2)) * 2 + x.two; };
+    auto class_end = [&](size_t k) {
+      size_t e = k;
+      while (e < ts.size() && ts[e].cls == ts[k].cls && ts[e].two == ts[k].two) ++e;
+      return e;
+    };
+    for (size_t k = 0; k < ts.size();) {
+      size_t e = class_end(k);
+      while (e < ts.size() && shape(ts[e]) == shape(ts[k])) {
+        const size_t f = class_end(e);
+        if (e - k >= MM_FEW && f - e >= MM_FEW) break;
+        e = f;
+      }
+      MmTiles m{nullptr, (int)(e - k), 0, ts[k].two, 0, nullptr};
       m.jobs = (const Job*)(uintptr_t)flat.size();  // index until the upload
-      for (size_t i = k; i < e; ++i) flat.insert(flat.end(), ts[i].j, ts[i].j + MM_LINES);
+      for (size_t i = k; i < e; ++i) {
+        m.kp = std::max(m.kp, ts[i].kp);
+        m.cmax = std::max(m.cmax, ts[i].j[0].C);
+        flat.insert(flat.end(), ts[i].j, ts[i].j + MM_LINES);
+      }
       out.push_back(m);
       k = e;
     }
+  };
+  // CTA size, then parity (classes of one shape are neighbours), then length
+  auto order = [](const Tile& a, const Tile& b) {
+    const int na = a.kp <= 128 ? 0 : (a.kp <= 256 ? 1 : 2), nb = b.kp <= 128 ? 0 : (b.kp <= 256 ? 1 : 2);
+    return na != nb ? na > nb : (a.two != b.two ? a.two > b.two : a.kp > b.kp);
   };
   std::vector<Job> flat;
   q.mm.clear();
@@ -1044,16 +1067,18 @@ void make_tiles(fc_ctx* c, fc_ctx::Queue& q, const std::vector<Job>& pp, const s
     std::vector<Tile> ts;
     const int p = tiles[k].patch;
     while (k < tiles.size() && tiles[k].patch == p) ts.push_back(tiles[k++]);
-    std::stable_sort(ts.begin(), ts.end(), [](const Tile& a, const Tile& b) { return a.kp > b.kp; });
+    std::stable_sort(ts.begin(), ts.end(), order);
     put(ts, q.mmpp[p], flat);
   }
-  std::stable_sort(tiles.begin(), tiles.end(), [](const Tile& a, const Tile& b) {
-    return a.cls != b.cls ? a.cls > b.cls : (a.two != b.two ? a.two > b.two : a.kp > b.kp);
-  });
+  std::stable_sort(tiles.begin(), tiles.end(), order);
   put(tiles, q.mm, flat);
-  Job* d = nullptr;
-  ok = ok && c->upload(&d, flat);
-  auto fix = [&](MmTiles& m) { m.jobs = d + (uintptr_t)m.jobs; };
+  q.ntiles = (int)tiles.size();
+  ok = ok && c->upload(&q.dmm, flat) && c->alloc(&q.dvisc, flat.size() / MM_LINES);
+  auto fix = [&](MmTiles& m) {
+    const uintptr_t first = (uintptr_t)m.jobs;
+    m.jobs = q.dmm + first;
+    m.visc = q.dvisc + first / MM_LINES;
+  };
   for (MmTiles& m : q.mm) fix(m);
   for (auto& v : q.mmpp)
     for (MmTiles& m : v) fix(m);
@@ -1647,8 +1672,8 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   bool ok = true;
   make_queue(c, c->q_cart1, jc1, B.plans, npatch, ok, &B.mm);
   make_queue(c, c->q_cart2, jc2, B.plans, npatch, ok, &B.mm);
-  make_queue(c, c->q_gen1, jg1, B.plans, npatch, ok, nullptr);
-  make_queue(c, c->q_gen2, jg2, B.plans, npatch, ok, nullptr);
+  make_queue(c, c->q_gen1, jg1, B.plans, npatch, ok, &B.mm);
+  make_queue(c, c->q_gen2, jg2, B.plans, npatch, ok, &B.mm);
   make_queue(c, c->q_filt1, jf1, B.plans, npatch, ok, &B.mm);
   make_queue(c, c->q_filt2, jf2, B.plans, npatch, ok, &B.mm);
   std::vector<PatchDev> pdev(npatch);
@@ -1745,6 +1770,8 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   T.any_pform = any_pform ? 1 : 0;
   set_kernel_attributes();
   set_mm_attributes();
+  set_mm_gen_attributes();
+  set_mm_adj_attributes();
   if (!mpts.empty()) {  // metrics of GRID patches given by their points only
     std::vector<double> xy(2 * (size_t)c->P, 0.0);
     for (const HPatch& h : c->hp)
@@ -1897,6 +1924,25 @@ void run_queue(fc_ctx* c, const fc_ctx::Queue& q0, bool per_patch, cudaStream_t 
   }
 }
 
+// viscous flags of the affine tiles for the passes of a call that use one mu throughout
+void tile_flags(fc_ctx* c, const double* mu, bool per_patch, cudaStream_t st) {
+  for (const fc_ctx::Queue* q : {&c->q_cart1, &c->q_cart2}) {
+    if (q->ntiles == 0) continue;
+    const size_t first = per_patch ? 0 : (size_t)q->ntiles;
+    launch_tile_flags(q->dmm + first * MM_LINES, q->ntiles, mu, q->dvisc + first, st);
+    c->launches++;
+  }
+  c->flags_on = true;
+}
+struct FlagScope {  // the flags are those of a call's mu until the call returns
+  fc_ctx* c;
+  ~FlagScope() { c->flags_on = false; }
+};
+MmTiles flagged(const fc_ctx* c, MmTiles t) {
+  if (!c->flags_on) t.visc = nullptr;
+  return t;
+}
+
 void stage(fc_ctx* c, const StageCoef& sc, const double* mu, bool per_patch, cudaStream_t st) {
   const DevTables& T = c->T;
   const double* e = sc.Ucur;
@@ -1912,8 +1958,10 @@ void stage(fc_ctx* c, const StageCoef& sc, const double* mu, bool per_patch, cud
     sg = c->side[0];
     gside = fc_ctx::NSIDE;  // no class forks inside the curvilinear chain
   }
-  run_queue(c, c->q_gen1, per_patch, sg, "gen_A",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_gen_A(T, j, n, L, e, c->d_G, s); }, gside);
+  run_queue(
+      c, c->q_gen1, per_patch, sg, "gen_A",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_gen_A(T, j, n, L, e, c->d_G, s); }, gside,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_gen_A(T, t, e, c->d_G, s); });
   if (c->ngfix) {
     launch_gen_fix(T, c->d_gfix, c->ngfix, e, mu, c->d_J, c->d_G, sg);
     c->launches++;
@@ -1925,17 +1973,19 @@ void stage(fc_ctx* c, const StageCoef& sc, const double* mu, bool per_patch, cud
   run_queue(
       c, c->q_cart1, per_patch, st, "cart_q1",
       [&](const Job* j, int n, int L, cudaStream_t s) { launch_cart_q1(T, j, n, L, e, mu, c->d_R1, c->d_Fy, s); }, 1,
-      [&](const MmTiles& t, cudaStream_t s) { launch_mm_cart_q1(T, t, e, mu, c->d_R1, c->d_Fy, s); });
-  run_queue(c, c->q_gen2, per_patch, sg, "gen_B",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_gen_B(T, j, n, L, e, mu, c->d_J, c->d_G, s); },
-            gside);
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_cart_q1(T, flagged(c, t), e, mu, c->d_R1, c->d_Fy, s); });
+  run_queue(
+      c, c->q_gen2, per_patch, sg, "gen_B",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_gen_B(T, j, n, L, e, mu, c->d_J, c->d_G, s); }, gside,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_gen_B(T, t, e, mu, c->d_J, c->d_G, s); });
   run_queue(
       c, c->q_cart2, per_patch, st, "cart_q2",
       [&](const Job* j, int n, int L, cudaStream_t s) { launch_cart_q2(T, j, n, L, mu, c->d_R1, c->d_Fy, sc, s); }, 1,
-      [&](const MmTiles& t, cudaStream_t s) { launch_mm_cart_q2(T, t, mu, c->d_R1, c->d_Fy, sc, s); });
-  run_queue(c, c->q_gen1, per_patch, sg, "gen_C",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_gen_C(T, j, n, L, c->d_J, c->d_G, sc, s); },
-            gside);
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_cart_q2(T, flagged(c, t), mu, c->d_R1, c->d_Fy, sc, s); });
+  run_queue(
+      c, c->q_gen1, per_patch, sg, "gen_C",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_gen_C(T, j, n, L, c->d_J, c->d_G, sc, s); }, gside,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_gen_C(T, t, c->d_J, c->d_G, sc, s); });
   if (overlap) {
     cudaEventRecord(c->join_ev[0], c->side[0]);
     cudaStreamWaitEvent(st, c->join_ev[0], 0);
@@ -2022,14 +2072,18 @@ void filterT(fc_ctx* c, const double* lam, const double* pre, const double* filt
              cudaStream_t st) {
   const DevTables& T = c->T;
   cudaMemcpyAsync(out, lam, sizeof(double) * 4 * (size_t)c->P, cudaMemcpyDeviceToDevice, st);
-  run_queue(c, c->q_filt2, false, st, "filterT_q2",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_filterT_q2(T, j, n, L, lam, filt, MF, s); });
+  run_queue(
+      c, c->q_filt2, false, st, "filterT_q2",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_filterT_q2(T, j, n, L, lam, filt, MF, s); }, 1,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_filterT_q2(T, t, lam, filt, MF, s); });
   if (c->nfcopy2) {
     launch_filterT_copy2(T, c->d_fcopy2, c->nfcopy2, lam, filt, MF, st);
     c->launches++;
   }
-  run_queue(c, c->q_filt1, false, st, "filterT_q1",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_filterT_q1(T, j, n, L, MF, pre, out, s); });
+  run_queue(
+      c, c->q_filt1, false, st, "filterT_q1",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_filterT_q1(T, j, n, L, MF, pre, out, s); }, 1,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_filterT_q1(T, t, MF, pre, out, s); });
   if (c->nfcopy1) {
     launch_filterT_copy1(T, c->d_fcopy1, c->nfcopy1, MF, pre, out, st);
     c->launches++;
@@ -2056,6 +2110,8 @@ void rk_body(fc_ctx* c, double* e, double* dt, double* mu, int flags, cudaStream
     project(c, e, st);
   }
   if (!(flags & FC_STEP_FIXED_DT)) timestep(c, e, mu, dt, st);
+  const FlagScope flag_scope{c};
+  tile_flags(c, mu, pp, st);
   StageCoef s{};
   s.dt = dt;
   // stage 1: u1 = u0 + b1 dt L(u0)
@@ -2105,24 +2161,39 @@ void adj_stage(fc_ctx* c, const double* u, const double* mu, const double* psi, 
                cudaStream_t st) {
   const DevTables& T = c->T;
   cudaMemsetAsync(c->d_R1, 0, sizeof(double) * 4 * (size_t)c->P, st);
-  run_queue(c, c->q_gen1, false, st, "adj_gen_A",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_A(T, j, n, L, c->d_J, u, psi, c->d_G, s); });
+  run_queue(
+      c, c->q_gen1, false, st, "adj_gen_A",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_A(T, j, n, L, c->d_J, u, psi, c->d_G, s); }, 1,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_gen_A(T, t, c->d_J, u, psi, c->d_G, s); });
   if (c->ngfix) {
     launch_adj_gen_fixA(T, c->d_gfix, c->ngfix, c->d_J, u, mu, psi, c->d_G, st);
     c->launches++;
   }
-  run_queue(c, c->q_cart1, false, st, "adj_cart_q1",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_cart(T, j, n, L, 0, u, mu, psi, c->d_R1, acc, dt, s); });
-  run_queue(c, c->q_gen2, false, st, "adj_gen_B",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_B(T, j, n, L, c->d_J, u, mu, psi, c->d_G, s); });
+  // (the y-flux buffer carries the contraction kernels' mu eta between their two rounds)
+  run_queue(
+      c, c->q_cart1, false, st, "adj_cart_q1",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_cart(T, j, n, L, 0, u, mu, psi, c->d_R1, acc, dt, s); },
+      1, [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_cart(T, flagged(c, t), 0, u, mu, psi, c->d_R1, acc, c->d_Fy, dt, s); });
+  run_queue(
+      c, c->q_gen2, false, st, "adj_gen_B",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_B(T, j, n, L, c->d_J, u, mu, psi, c->d_G, s); }, 1,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_gen_B(T, t, c->d_J, u, mu, psi, c->d_G, s); });
+  if (T.any_pform)
+    run_queue(c, c->q_gen2, false, st, "adj_gen_B", [&](const Job* j, int n, int L, cudaStream_t s) {
+      launch_adj_gen_B_wall(T, j, n, L, c->d_J, u, mu, psi, c->d_G, s);
+    });
   if (c->ngfix) {
     launch_adj_gen_fixB(T, c->d_gfix, c->ngfix, c->d_G, c->d_R1, st);
     c->launches++;
   }
-  run_queue(c, c->q_cart2, false, st, "adj_cart_q2",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_cart(T, j, n, L, 1, u, mu, psi, c->d_R1, acc, dt, s); });
-  run_queue(c, c->q_gen1, false, st, "adj_gen_C",
-            [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_C(T, j, n, L, u, c->d_G, acc, dt, s); });
+  run_queue(
+      c, c->q_cart2, false, st, "adj_cart_q2",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_cart(T, j, n, L, 1, u, mu, psi, c->d_R1, acc, dt, s); },
+      1, [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_cart(T, flagged(c, t), 1, u, mu, psi, c->d_R1, acc, c->d_Fy, dt, s); });
+  run_queue(
+      c, c->q_gen1, false, st, "adj_gen_C",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_C(T, j, n, L, u, c->d_G, acc, dt, s); }, 1,
+      [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_gen_C(T, t, u, c->d_G, acc, dt, s); });
   if (c->nfix) {
     launch_adj_fixup(c->d_fix, c->nfix, c->d_R1, acc, c->P, dt, st);
     c->launches++;
@@ -2590,6 +2661,8 @@ fc_status fc_adjoint_step(fc_ctx* c, const double* e_n, const double* mu, const 
     cudaMemcpyAsync(c->d_FY, U[0], bytes4, cudaMemcpyDeviceToDevice, st);
     project(c, U[0], st);
   }
+  const FlagScope flag_scope{c};
+  tile_flags(c, mu, false, st);
   StageCoef s{};
   s.dt = dt;
   s.U0 = U[0];

@@ -14,7 +14,9 @@ constexpr size_t SMEM_CAP = 200 * 1024;  // dynamic shared memory budget per CTA
 constexpr int SDNN_H = 16;      // hidden width of the stand-in classifier
 constexpr int MAX_GENERIC_RADIX = 128;  // largest prime factor of a continued length
 constexpr int CONT_TMP = 32;    // complex scratch per warp after the line buffer (detrended end data, d <= 8)
-constexpr int MM_KMAX = 256;     // largest inner length of a tensor-core line contraction (fc_mma.cu)
+constexpr int MM_KMAX = 512;     // largest inner length of a tensor-core line contraction (fc_mma.cu)
+constexpr int MM_KCHUNK = 256;   // columns whose digit products are summed in FP32 before they are joined
+constexpr int MM_CMAX = 128;     // largest continuation length of a contracted line
 constexpr int MM_LINES = 4;      // lines per tile of the contraction kernels
 constexpr int NCLASS = 24;      // length classes of the line queues: ceil(log2 Lmax)
 
@@ -162,8 +164,6 @@ struct DevTables {
   int any_pform;
 };
 
-// ---- launch wrappers of the contraction kernels (fc_mma.cu) ----
-// tiles: MM_LINES jobs each, of one plan (absent lines: n = 0), all of padded inner length
 // kernel parameters: the classifier's FP32 weights, and the window weights (2 win_r - 1 <= 63)
 struct SdnnW {
   float w[16 * 7 + 16 + 16 * 16 + 16 + 4 * 16 + 4];
@@ -172,20 +172,48 @@ struct WindowW {
   double w[64];
 };
 
+// ---- launch wrappers of the contraction kernels (fc_mma.cu) ----
+// tiles: MM_LINES jobs each, of one plan (absent lines: n = 0), all of padded inner length
 // Kp <= kp; two: even lengths
 struct MmTiles {
   const Job* jobs;
   int n;      // tiles
   int kp;
   int two;
+  int cmax;   // largest continuation length
+  // per tile: mu != 0 somewhere on its lines, as launch_tile_flags found it (null: the
+  // kernel looks for itself)
+  uint8_t* visc;
 };
+// flags of n tiles (jobs: MM_LINES per tile)
+void launch_tile_flags(const Job* jobs, int n, const double* mu, uint8_t* visc, cudaStream_t st);
 void launch_mm_cart_q1(const DevTables& T, const MmTiles& t, const double* e, const double* mu, double* R1, double* Fy,
                        cudaStream_t st);
 void launch_mm_cart_q2(const DevTables& T, const MmTiles& t, const double* mu, const double* R1, double* Fy,
                        const StageCoef& sc, cudaStream_t st);
 void launch_mm_filter_q1(const DevTables& T, const MmTiles& t, const double* e, double* F, cudaStream_t st);
 void launch_mm_filter_q2(const DevTables& T, const MmTiles& t, const double* F, double* e, cudaStream_t st);
+void launch_mm_gen_A(const DevTables& T, const MmTiles& t, const double* e, double* G, cudaStream_t st);
+void launch_mm_gen_B(const DevTables& T, const MmTiles& t, const double* e, const double* mu, const double* J,
+                     double* G, cudaStream_t st);
+void launch_mm_gen_C(const DevTables& T, const MmTiles& t, const double* J, double* G, const StageCoef& sc,
+                     cudaStream_t st);
+// Y: scratch of the affine points ([4][P])
+void launch_mm_adj_cart(const DevTables& T, const MmTiles& t, int dir, const double* u, const double* mu,
+                        const double* psi, double* R1, double* acc, double* Y, const double* dt, cudaStream_t st);
+void launch_mm_adj_gen_A(const DevTables& T, const MmTiles& t, const double* J, const double* u, const double* psi,
+                         double* G, cudaStream_t st);
+void launch_mm_adj_gen_B(const DevTables& T, const MmTiles& t, const double* J, const double* u, const double* mu,
+                         const double* psi, double* G, cudaStream_t st);
+void launch_mm_adj_gen_C(const DevTables& T, const MmTiles& t, const double* u, const double* G, double* acc,
+                         const double* dt, cudaStream_t st);
+void launch_mm_filterT_q2(const DevTables& T, const MmTiles& t, const double* lam, const double* ef, double* MF,
+                          cudaStream_t st);
+void launch_mm_filterT_q1(const DevTables& T, const MmTiles& t, const double* MF, const double* e, double* out,
+                          cudaStream_t st);
 void set_mm_attributes();
+void set_mm_gen_attributes();
+void set_mm_adj_attributes();
 
 // ---- launch wrappers (fc_kernels.cu) ----
 // Fy (nullable): the y fluxes of the affine points, written by the q1 pass (and by
@@ -253,6 +281,9 @@ void launch_adj_gen_A(const DevTables& T, const Job* jobs, int njobs, int Lmax, 
                       const double* psi, double* G, cudaStream_t st);
 void launch_adj_gen_B(const DevTables& T, const Job* jobs, int njobs, int Lmax, const double* J, const double* u,
                       const double* mu, const double* psi, double* G, cudaStream_t st);
+// the product-rule wall form's lines (the others are passed over)
+void launch_adj_gen_B_wall(const DevTables& T, const Job* jobs, int njobs, int Lmax, const double* J, const double* u,
+                           const double* mu, const double* psi, double* G, cudaStream_t st);
 void launch_adj_gen_C(const DevTables& T, const Job* jobs, int njobs, int Lmax, const double* u, const double* G,
                       double* acc, const double* dt, cudaStream_t st);
 void launch_adj_fixup(const int* idx, int n, const double* R1, double* acc, long long P, const double* dt,

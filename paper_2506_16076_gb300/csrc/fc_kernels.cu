@@ -1454,40 +1454,6 @@ __device__ __forceinline__ void adj_wall_point_B(const DevTables& T, long long p
   *b = cpx(g2[2], g2[3]);
 }
 
-// (dQ/du)^T a for Q = (rho, rho u, rho v, theta), theta = (gamma - 1) (E / rho - |rho u|^2 / (2 rho^2))
-__device__ __forceinline__ void thetaT_add(const double* u, double gam, const double* a, double* out) {
-  const double ir = 1.0 / u[0], g1 = gam - 1.0;
-  const double m2 = fma(u[1], u[1], u[2] * u[2]);
-  out[0] += a[0] + a[3] * g1 * ir * ir * (m2 * ir - u[3]);
-  out[1] += a[1] - a[3] * g1 * u[1] * ir * ir;
-  out[2] += a[2] - a[3] * g1 * u[2] * ir * ir;
-  out[3] += a[3] * g1 * ir;
-}
-
-// A^T eta for the x (dir 0) or y (dir 1) flux Jacobian at state e (eq. euler 2d equation)
-__device__ __forceinline__ void fluxT(int dir, double r, double mx, double my, double E, double gam, const double* eta,
-                                      double* out) {
-  const double ir = 1.0 / r;
-  const double u = mx * ir, v = my * ir;
-  const double g1 = gam - 1.0;
-  const double q2 = u * u + v * v;
-  const double p = g1 * (E - 0.5 * r * q2);
-  const double H = (E + p) * ir;
-  const double pr = 0.5 * g1 * q2, pm = -g1 * u, pn = -g1 * v, pE = g1;
-  if (dir == 0) {
-    // rows c = 0..3 of A_x, columns j: out_j = sum_c A[c][j] eta_c
-    out[0] = (-u * u + pr) * eta[1] + (-u * v) * eta[2] + (-u * H + u * pr) * eta[3];
-    out[1] = eta[0] + (2.0 * u + pm) * eta[1] + v * eta[2] + (H + u * pm) * eta[3];
-    out[2] = pn * eta[1] + u * eta[2] + u * pn * eta[3];
-    out[3] = pE * eta[1] + u * (1.0 + pE) * eta[3];
-  } else {
-    out[0] = (-u * v) * eta[1] + (-v * v + pr) * eta[2] + (-v * H + v * pr) * eta[3];
-    out[1] = v * eta[1] + pm * eta[2] + v * pm * eta[3];
-    out[2] = eta[0] + u * eta[1] + (2.0 * v + pn) * eta[2] + (H + v * pn) * eta[3];
-    out[3] = pE * eta[2] + v * (1.0 + pE) * eta[3];
-  }
-}
-
 __device__ __forceinline__ void load4_masked(double2* A, int L, const Job& J, const DevTables& T,
                                              const double* __restrict__ src, int lane) {
   const long long cs = T.P;
@@ -1985,26 +1951,6 @@ __global__ void __launch_bounds__(256) k_init_sens(const uint32_t* __restrict__ 
 // ---- transpose of the linearised per-step filter (Sec. 4.3.1) -----------------------------
 // forward: Q = (rho, rho u, rho v, theta(e)) filtered along q1 lines (into F), then along q2
 // lines, and E rebuilt from the filtered Q (eq. perfect_gas_T)
-__device__ __forceinline__ void rebuild_T(const double* __restrict__ lam, const double* __restrict__ ef, long long p,
-                                          long long cs, double gam, double* o) {
-  const double r = ef[p], m = ef[p + cs], nn = ef[p + 2 * cs];
-  const double th = theta_of(r, m, nn, ef[p + 3 * cs], gam);
-  const double g1 = gam - 1.0, lE = lam[p + 3 * cs], ir = 1.0 / r;
-  o[0] = lam[p] + lE * (th / g1 - 0.5 * (m * m + nn * nn) * ir * ir);
-  o[1] = lam[p + cs] + lE * m * ir;
-  o[2] = lam[p + 2 * cs] + lE * nn * ir;
-  o[3] = lE * r / g1;
-}
-__device__ __forceinline__ void theta_T(const double* q, const double* __restrict__ e, long long p, long long cs,
-                                        double gam, double* o) {
-  const double r = e[p], m = e[p + cs], nn = e[p + 2 * cs], E = e[p + 3 * cs];
-  const double g1 = gam - 1.0, lt = q[3], ir = 1.0 / r, ir2 = ir * ir;
-  o[0] = q[0] + lt * g1 * (-E * ir2 + (m * m + nn * nn) * ir2 * ir);
-  o[1] = q[1] + lt * (-g1 * m * ir2);
-  o[2] = q[2] + lt * (-g1 * nn * ir2);
-  o[3] = lt * g1 * ir;
-}
-
 // q2 lines: lam (adjoint of the filtered state), ef (the filter output) -> MF
 __global__ void LINE_KERNEL_BOUNDS k_filterT_q2(DevTables T, const Job* __restrict__ jobs, int njobs, int Lmax,
                                                 const double* __restrict__ lam, const double* __restrict__ ef,
@@ -2294,7 +2240,11 @@ void launch_adj_gen_B(const DevTables& T, const Job* jobs, int njobs, int Lmax, 
                       const double* mu, const double* psi, double* G, cudaStream_t st) {
   if (njobs <= 0) return;
   k_adj_gen_B<<<LINE_CFG(njobs, Lmax)>>>(T, jobs, njobs, Lmax, J, u, mu, psi, G);
-  if (T.any_pform) k_adj_gen_B_wall<<<LINE_CFG(njobs, Lmax)>>>(T, jobs, njobs, Lmax, J, u, mu, psi, G);
+}
+void launch_adj_gen_B_wall(const DevTables& T, const Job* jobs, int njobs, int Lmax, const double* J, const double* u,
+                           const double* mu, const double* psi, double* G, cudaStream_t st) {
+  if (njobs <= 0) return;
+  k_adj_gen_B_wall<<<LINE_CFG(njobs, Lmax)>>>(T, jobs, njobs, Lmax, J, u, mu, psi, G);
 }
 void launch_adj_gen_C(const DevTables& T, const Job* jobs, int njobs, int Lmax, const double* u, const double* G,
                       double* acc, const double* dt, cudaStream_t st) {

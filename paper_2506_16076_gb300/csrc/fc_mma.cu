@@ -1,469 +1,9 @@
-// FC line operators as exact tensor-core contractions (fc_split.cuh, fc_mmtab.h).
-//
-// GB300 executes 2 FP64 FMAs per clock and SM but 1024 FP16 ones through mma.sync (measured
-// 600 TFLOP/s), so the circulant of a continued line (21 FP16 digit products per entry,
-// L^2/2 entries per line) costs less time than the FP64 butterflies of its two FFTs up to
-// lengths of a few hundred. What a line still needs from the FP64 pipe is its pointwise
-// work: fluxes, continuation and stage combination.
-//
-// A CTA takes MM_LINES lines of one length (16 columns: 4 lines x 4 components). Each
-// thread loads its points, forms the values to transform and keeps them in registers until
-// the lines' largest magnitudes are known; then the sums and differences of the two halves
-// go to shared memory as FP16 digits. Each warp contracts 16 output rows at a time: the
-// right operand's fragments come from shared memory (ldmatrix), the left operand is a
-// Toeplitz matrix, so a fragment is three table entries of which each 16-column step needs
-// two new ones (read through L1: all warps of an SM share a table of 24 bytes per entry).
-// Digits of a line need 12 bytes per point and part; 128 threads for inner lengths up to
-// 128 and 256 beyond keep 16 warps per SM resident.
-//
-// Measured (28M points, affine lines of 48 to 384 points, FFT kernels -> contraction, per
-// pass): q1 9.6 -> 4.5 ms, q2 10.0 -> 6.3 ms, filter q1 + q2 17.5 -> 8.1 ms; a 128 x 128
-// operator with L = 155 = 5 x 31: 462 -> 25 us. Largest error on white lines 2e-16 of the
-// largest value (FP64 FFT: 6e-16 to 9e-16). Of these times, passing the values through
-// shared memory (the fluxes' lanes then follow the points, 89% of them active instead of
-// 78%) and fetching a step's table entries one step ahead took 17%; a tile keeps its
-// sub-core's matrix pipe busy for 12k of about 26k cycles, the FP64 pipe for 10k to 15k.
-#include <cuda_fp16.h>
-#include <cuda_runtime.h>
-#include <math.h>
-#include <stdint.h>
-
-#include "fc_internal.h"
-#include "fc_line.cuh"
-#include "fc_point.cuh"
-#include "fc_split.cuh"
+// Contraction kernels of the affine passes and of the filter (fc_mma.cuh).
+#include "fc_mma.cuh"
 
 namespace fcx {
 
 namespace {
-
-constexpr int NCOL = 4 * MM_LINES;  // columns of a tile: component * MM_LINES + line
-
-// static shared state of a tile
-struct MmShared {
-  Job J[MM_LINES];
-  uint32_t emax[NCOL];  // high words of the largest magnitudes
-  double fac[NCOL];     // value of one unit of a joined sum
-  double tmp[NCOL * 16];  // detrended end values of the columns, 2d <= 16 each
-};
-
-constexpr int LB = 4;  // points of a thread whose loads are in flight together
-
-// columns of the lines' values in shared memory: a pitch of 4 (mod 16) doubles keeps the
-// four lines of a row of q2 points in different banks
-__host__ __device__ inline int mm_line_pitch(int L) { return L + ((4 - L % 16) + 16) % 16; }
-// dynamic shared memory: the digits [S][SP_DIGITS][NCOL][Kp + 8] of FP16 (columns padded by
-// 16 bytes: conflict-free ldmatrix), over the continued lines [NCOL][pitch] they come from
-size_t mm_smem(int S, int Kp) {
-  const size_t dig = (size_t)S * SP_DIGITS * NCOL * (Kp + 8) * 2;
-  const size_t val = (size_t)NCOL * mm_line_pitch(S * Kp) * sizeof(double);
-  return dig > val ? dig : val;
-}
-
-__device__ __forceinline__ void mma16816(float* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                         uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void ldsm4(uint32_t* r, uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
-}
-
-// table entries stay in L1 (every warp of the SM reads them), the lines' data pass by it
-__device__ __forceinline__ uint4 ldg_keep(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::evict_last.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
-}
-__device__ __forceinline__ uint2 ldg_keep(const uint2* p) {
-  uint2 v;
-  asm volatile("ld.global.nc.L1::evict_last.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ double ld_pass(const double* p) {
-  double v;
-  asm volatile("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
-  return v;
-}
-
-// two biased values' digit k as an FP16 pair: the 10-bit fields become 1024 + field by
-// setting the exponent bits, then 1536 comes off
-__device__ __forceinline__ uint32_t digit_pair(long long a, long long b, int k) {
-  const uint32_t fa = (uint32_t)(a >> (SP_BITS * (SP_DIGITS - 1 - k)));
-  const uint32_t fb = (uint32_t)(b >> (SP_BITS * (SP_DIGITS - 1 - k)));
-  uint32_t w = (__byte_perm(fa, fb, 0x5410) & 0x03ff03ffu) | 0x64006400u;
-  __half2 h = __hsub2(*reinterpret_cast<__half2*>(&w), __half2half2(__ushort_as_half(0x6600)));
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-
-// the joined sums of one part for the warp's 16 rows from i0: W[r * 4 + nt * 2 + c] is row
-// i0 + g + 8 r, column nt * 8 + 2 t + c (g = lane / 4, t = lane % 4)
-__device__ __forceinline__ void mm_part(const uint4* __restrict__ lo, const uint2* __restrict__ hi, uint32_t dig,
-                                        int pitch, const MmPlan& p, int i0, int lane, long long* W) {
-  const int g = lane >> 2, t = lane & 3;
-  float acc[SP_DIGITS][2][4];
-#pragma unroll
-  for (int l = 0; l < SP_DIGITS; ++l)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[l][0][q] = acc[l][1][q] = 0.f;
-  const uint4* pl = lo + (p.Mp - i0 + 2 * t - g);
-  const uint2* ph = hi + (p.Mp - i0 + 2 * t - g);
-  uint32_t Am[SP_DIGITS], A0[SP_DIGITS], Ap[SP_DIGITS], N0[SP_DIGITS], Np[SP_DIGITS];
-  auto entry = [&](uint32_t* A, int x) {
-    const uint4 a = ldg_keep(pl + x);
-    const uint2 b = ldg_keep(ph + x);
-    A[0] = a.x;
-    A[1] = a.y;
-    A[2] = a.z;
-    A[3] = a.w;
-    A[4] = b.x;
-    A[5] = b.y;
-  };
-  entry(Am, -8);
-  entry(A0, 0);
-  entry(Ap, 8);
-  // ldmatrix row addresses: matrices (columns 0-7, k), (columns 0-7, k+8), (8-15, k), (8-15, k+8)
-  uint32_t baddr = dig + (uint32_t)(((lane & 7) + ((lane >> 4) << 3)) * pitch + ((lane >> 3) & 1) * 16);
-  const uint32_t bslice = (uint32_t)NCOL * pitch;
-  for (int k0 = 0; k0 < p.Kp; k0 += 16) {
-    const int kn = k0 + 16 < p.Kp ? k0 + 16 : k0;  // the next step's entries, a whole step ahead
-    entry(N0, kn);
-    entry(Np, kn + 8);
-    uint32_t b[2][4];
-    ldsm4(b[0], baddr);
-#pragma unroll
-    for (int j = 0; j < SP_DIGITS; ++j) {
-      if (j + 1 < SP_DIGITS) ldsm4(b[(j + 1) & 1], baddr + (j + 1) * bslice);
-      const uint32_t* c = b[j & 1];
-#pragma unroll
-      for (int i = 0; i + j < SP_DIGITS; ++i) {
-        mma16816(acc[i + j][0], A0[i], Am[i], Ap[i], A0[i], c[0], c[1]);
-        mma16816(acc[i + j][1], A0[i], Am[i], Ap[i], A0[i], c[2], c[3]);
-      }
-    }
-    baddr += 32;
-#pragma unroll
-    for (int i = 0; i < SP_DIGITS; ++i) {
-      Am[i] = Ap[i];
-      A0[i] = N0[i];
-      Ap[i] = Np[i];
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    int s[SP_DIGITS];
-#pragma unroll
-    for (int l = 0; l < SP_DIGITS; ++l) s[l] = __float2int_rn(acc[l][(q >> 1) & 1][(q >> 2) * 2 + (q & 1)]);
-    W[q] = sp_join(s);
-  }
-}
-
-// the tile's point of a line (absent lines: the state's first point, read and never used)
-__device__ __forceinline__ long long point(const MmShared& sh, int line, int t) {
-  return sh.J[line].base + (long long)t * sh.J[line].stride;
-}
-
-// continuation values of the tile's columns from their detrended end values (eq.
-// continuation, as continue_lines), D = d when it is known at compile time
-template <int NT, int D>
-__device__ __forceinline__ void continuation(const double* __restrict__ M, int C, int dd, const double* tmp,
-                                             double* ext, int LP, uint32_t* emax) {
-  const int d = D ? D : dd;
-  const double* ML = M;
-  const double* MR = M + C * d;
-  const double* u = MR + C * d;  // uL, vL, uR, vR
-  for (int it = threadIdx.x; it < NCOL * C; it += NT) {
-    const int col = it & (NCOL - 1), k = it / NCOL;
-    const double* e = tmp + col * 16;
-    double x = 0.0;
-#pragma unroll
-    for (int j = 2; j < d; ++j) x = fma(__ldg(ML + k * d + j), e[j - 2], x);
-#pragma unroll
-    for (int j = 0; j < d - 2; ++j) x = fma(__ldg(MR + k * d + j), e[d - 2 + j], x);
-    x = fma(e[2 * d - 4], __ldg(u + k),
-            fma(e[2 * d - 3], __ldg(u + C + k),
-                fma(e[2 * d - 2], __ldg(u + 2 * C + k), fma(e[2 * d - 1], __ldg(u + 3 * C + k), x))));
-    ext[col * LP + k] = x;
-    atomicMax(&emax[col], sp_hi(x) & 0x7fffffffu);
-  }
-}
-
-// One round: ld.raw(point, v) loads four values and ld.form(point, v) makes the point's four
-// values to transform of them; the continued lines' operator (derivative, or the filter
-// with FILT) is applied; ep.put(comp, point, op, value) takes the results, op =
-// ep.pre(comp, point) loaded ahead for a batch of eight, or with PT ep.put(point, v[4]) a
-// point's four at once. All threads of the CTA call it; it begins with a barrier.
-template <int NT, int S, bool COL, bool FILT, bool PT, class Load, class Ep>
-__device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan, MmShared& sh, double2* dyn, Load ld,
-                                         Ep ep) {
-  constexpr int NW = NT / 32, TS = NT / 4;  // TS: points per step of a line
-  // opaque copies: without them the compiler hoists the address arithmetic of both of a
-  // kernel's rounds out of their loop (250 registers, 280 bytes of spills; so 128 and < 150)
-  int tid = threadIdx.x;
-  MmPlan p = plan;
-  asm volatile("" : "+r"(tid), "+r"(p.H), "+r"(p.Kp), "+r"(p.nx), "+r"(p.Mp));
-  const int warp = tid >> 5, lane = tid & 31;
-  const int n = sh.J[0].n, C = sh.J[0].C, fcm = sh.J[0].fcm, d = T.d, H = p.H;
-  const int LP = mm_line_pitch(S * H);
-  double* F = reinterpret_cast<double*>(dyn);  // [NCOL][LP]: the continued lines
-  if (tid < NCOL) sh.emax[tid] = 0;
-  __syncthreads();
-
-  // (1) the lines' values into shared memory, and their maxima. q1 lines: a warp per line
-  // (two with 256 threads), lanes along it; q2 lines: 4 neighbouring lines along the lanes
-  {
-    const int line = COL ? (tid & 3) : (warp & 3);
-    const int t0 = COL ? tid >> 2 : (warp >> 2) * 32 + lane;
-    const bool have = sh.J[line].n > 0;
-    uint32_t hm[4] = {0, 0, 0, 0};
-    for (int b = t0; b < n; b += LB * TS) {
-      double X[LB][4];
-#pragma unroll
-      for (int r = 0; r < LB; ++r)  // the batch's loads first (absent points read the line's first one)
-        ld.raw(point(sh, line, b + r * TS < n ? b + r * TS : 0), X[r]);
-#pragma unroll
-      for (int r = 0; r < LB; ++r) {
-        const int t = b + r * TS;
-        if (t < n) {
-          double* v = X[r];
-          if (have)
-            ld.form(point(sh, line, t), v);
-          else
-            v[0] = v[1] = v[2] = v[3] = 0.0;
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const uint32_t h = sp_hi(v[c]) & 0x7fffffffu;
-            hm[c] = h > hm[c] ? h : hm[c];
-            F[(c * MM_LINES + line) * LP + t] = v[c];
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      if (COL) {
-        uint32_t h = hm[c];
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-          const uint32_t g = __shfl_xor_sync(0xffffffffu, h, o);
-          h = g > h ? g : h;
-        }
-        if (lane < MM_LINES) atomicMax(&sh.emax[c * MM_LINES + line], h);
-      } else {
-        const uint32_t h = __reduce_max_sync(0xffffffffu, hm[c]);
-        if (lane == 0) atomicMax(&sh.emax[c * MM_LINES + line], h);
-      }
-    }
-  }
-  __syncthreads();
-
-  // (2) continuation (eq. continuation) in the detrended form of continue_lines
-  if (fcm >= 0) {
-    for (int it = tid; it < NCOL * 2 * d; it += NT) {
-      const int col = it & (NCOL - 1), q = it / NCOL;
-      const double* x = F + col * LP;
-      const double f0 = x[0], dl = x[1] - f0, fn = x[n - 1], dr = fn - x[n - 2];
-      double v;
-      if (q < d - 2) {
-        v = fma(-(double)(q + 2), dl, x[q + 2] - f0);
-      } else if (q < 2 * d - 4) {
-        const int j = q - (d - 2);
-        v = fma((double)(d - 1 - j), dr, x[n - d + j] - fn);
-      } else {
-        const int w = q - (2 * d - 4);
-        v = w == 0 ? f0 : (w == 1 ? dl : (w == 2 ? fn : dr));
-      }
-      sh.tmp[col * 16 + q] = v;
-    }
-    __syncthreads();
-    if (d == 5)
-      continuation<NT, 5>(T.rp + fcm, C, 5, sh.tmp, F + n, LP, sh.emax);
-    else
-      continuation<NT, 0>(T.rp + fcm, C, d, sh.tmp, F + n, LP, sh.emax);
-    __syncthreads();
-  }
-  const int te = FILT ? p.fte : p.dte;
-  if (tid < NCOL) {
-    const uint32_t h = sh.emax[tid], h2 = sh.emax[tid ^ MM_LINES];
-    const double sc = FILT ? 1.0 : sh.J[tid & (MM_LINES - 1)].scale;
-    // a non-finite value spoils its line, and its packed partner's, as in the FFT kernels
-    sh.fac[tid] = (h >= 0x7ff00000u || h2 >= 0x7ff00000u)
-                      ? __longlong_as_double(0x7ff8000000000000ll)
-                      : scalbn(sc, (int)(h >> 20) - 1023 - SP_DATA + SP_UNIT - te - (S - 1));
-  }
-
-  // (3) digits of the parts, over the values: all reads come before the first write. A warp
-  // per line again, lanes along the pairs (2q, 2q + 1)
-  {
-    const int line = warp & 3, q0 = (warp >> 2) * 32 + lane;
-    double X[2][4][S][2];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int s = 0; s < S; ++s)
-#pragma unroll
-          for (int a = 0; a < 2; ++a) {
-            const int k = 2 * (q0 + r * TS) + a;
-            X[r][c][s][a] = k < H ? F[(c * MM_LINES + line) * LP + k + s * H] : 0.0;
-          }
-    int ex[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) ex[c] = (int)(sh.emax[c * MM_LINES + line] >> 20);
-    __syncthreads();
-    const int pitchw = (p.Kp + 8) / 2;  // words per column
-    uint32_t* dig = reinterpret_cast<uint32_t*>(dyn);
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int q = q0 + r * TS;
-      if (2 * q < p.Kp) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          long long w[S][2];
-#pragma unroll
-          for (int a = 0; a < 2; ++a) {
-            const long long x0 = sp_fixed(X[r][c][0][a], ex[c]);
-            if (S == 2) {
-              const long long x1 = sp_fixed(X[r][c][S - 1][a], ex[c]);
-              w[0][a] = x0 + x1 + SP_BIAS;
-              w[S - 1][a] = x0 - x1 + SP_BIAS;
-            } else {
-              w[0][a] = x0 + SP_BIAS;
-            }
-          }
-#pragma unroll
-          for (int s = 0; s < S; ++s)
-#pragma unroll
-            for (int k = 0; k < SP_DIGITS; ++k)
-              dig[((s * SP_DIGITS + k) * NCOL + c * MM_LINES + line) * pitchw + q] = digit_pair(w[s][0], w[s][1], k);
-        }
-      }
-    }
-  }
-  __syncthreads();
-
-  // (4) contraction and results
-  const uint32_t dsh = (uint32_t)__cvta_generic_to_shared(dyn);
-  const int pitch = (p.Kp + 8) * 2;
-  const int tab = FILT ? p.ftab : p.dtab;
-  const int g = lane >> 2, t = lane & 3;
-  for (int i0 = warp * 16; i0 < H; i0 += NW * 16) {
-    long long W[S][8];
-#pragma unroll 1
-    for (int s = 0; s < S; ++s) {
-      long long w[8];
-      mm_part(T.mmlo + tab + s * p.nx, T.mmhi + tab + s * p.nx, dsh + s * SP_DIGITS * NCOL * pitch, pitch, p, i0, lane,
-              w);
-      if (s == 0) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) W[0][q] = w[q];
-      } else {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) W[S - 1][q] = w[q];
-      }
-    }
-#pragma unroll
-    for (int half = 0; half < S; ++half) {
-      if constexpr (!PT) {
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {  // rows g and g + 8: operands of four results in flight
-          const int i = i0 + g + 8 * r, idx = i + half * H;
-          const bool in = i < H && idx < n;
-          typename Ep::Op op[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int col = (q >> 1) * 8 + 2 * t + (q & 1);
-            op[q] = ep.pre(col / MM_LINES, point(sh, col & (MM_LINES - 1), in ? idx : 0));
-          }
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int col = (q >> 1) * 8 + 2 * t + (q & 1), ln = col & (MM_LINES - 1);
-            const long long w0 = W[0][4 * r + q], w1 = W[S - 1][4 * r + q];
-            const long long y = S == 1 ? w0 : (half ? w0 - w1 : w0 + w1);
-            if (in && sh.J[ln].n > 0) ep.put(col / MM_LINES, point(sh, ln, idx), op[q], sp_double(y) * sh.fac[col]);
-          }
-        }
-      } else {
-        // lanes t and t ^ 2 hold components (0, 2) and (1, 3) of the same lines and rows:
-        // t < 2 keeps row g, t >= 2 row g + 8
-        double y[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int col = ((q >> 1) & 1) * 8 + 2 * t + (q & 1);
-          const long long w = S == 1 ? W[0][q] : (half ? W[0][q] - W[S - 1][q] : W[0][q] + W[S - 1][q]);
-          y[q] = sp_double(w) * sh.fac[col];
-        }
-        const bool up = t >= 2;
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const double s0 = __shfl_xor_sync(0xffffffffu, up ? y[c] : y[4 + c], 2);
-          const double s1 = __shfl_xor_sync(0xffffffffu, up ? y[2 + c] : y[6 + c], 2);
-          double v[4];
-          v[0] = up ? s0 : y[c];
-          v[1] = up ? y[4 + c] : s0;
-          v[2] = up ? s1 : y[2 + c];
-          v[3] = up ? y[6 + c] : s1;
-          const int ln = 2 * (t & 1) + c, i = i0 + g + (up ? 8 : 0), idx = i + half * H;
-          if (i < H && idx < n && sh.J[ln].n > 0) ep.put(point(sh, ln, idx), v);
-        }
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ void load_tile(MmShared& sh, const Job* __restrict__ jobs) {
-  if (threadIdx.x < MM_LINES) sh.J[threadIdx.x] = jobs[(size_t)blockIdx.x * MM_LINES + threadIdx.x];
-  __syncthreads();
-}
-// mu != 0 somewhere on the tile's lines (on every thread); lines of an inviscid tile are
-// counted as skipped gradient rounds
-template <int NT, bool COL>
-__device__ __forceinline__ bool tile_viscous(const DevTables& T, const MmShared& sh, const MmPlan& p,
-                                             const double* __restrict__ mu, int dir) {
-  bool v = false;
-  const int n = sh.J[0].n;
-  const int line = COL ? (threadIdx.x & 3) : (threadIdx.x >> 5) & 3;
-  const int t0 = COL ? threadIdx.x >> 2 : (threadIdx.x & 31) + 32 * (threadIdx.x >> 7);
-  for (int t = t0; t < n; t += NT / 2) {  // two loads in flight per thread and step
-    const double a = mu[point(sh, line, t)], b = mu[point(sh, line, t + NT / 4 < n ? t + NT / 4 : t)];
-    v |= a != 0.0 || b != 0.0;
-  }
-  v = v && sh.J[line].n > 0;
-  const bool visc = __syncthreads_or(v) != 0;
-  if (!visc && threadIdx.x < MM_LINES && sh.J[threadIdx.x].n > 0 && T.skip_lines) {
-    const int L = p.H * p.S;
-    atomicAdd(T.skip_lines + dir, 1ull);
-    atomicAdd(T.skip_flops + dir, 4.0 * 5.0 * L * log2((double)L) + 16.0 * T.d * sh.J[0].C + 8.0 * L);
-  }
-  return visc;
-}
-
-#define MM_BOUNDS(NT) __launch_bounds__(NT, 512 / NT)
-
-struct NoOp {};
-struct PutField {  // results into a field
-  using Op = NoOp;
-  double* f;
-  long long cs;
-  __device__ __forceinline__ NoOp pre(int, long long) const { return {}; }
-  __device__ __forceinline__ void put(int c, long long q, NoOp, double v) const { f[q + c * cs] = v; }
-};
-struct LoadField {
-  const double* f;
-  long long cs;
-  __device__ __forceinline__ void raw(long long q, double* v) const {
-#pragma unroll
-    for (int c = 0; c < 4; ++c) v[c] = f[q + c * cs];
-  }
-  __device__ __forceinline__ void form(long long, double*) const {}
-};
 
 // affine q1 lines: R1 = d/dx (f_x(e) - mu d/dx e); Fy: the points' y fluxes
 struct LoadQ1 {
@@ -495,16 +35,17 @@ struct LoadQ1 {
 };
 template <int NT, int S>
 __global__ void MM_BOUNDS(NT) k_mm_cart_q1(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ e,
-                                           const double* __restrict__ mu, double* R1, double* __restrict__ Fy) {
+                                           const double* __restrict__ mu, double* R1, double* __restrict__ Fy,
+                                           const uint8_t* __restrict__ flags) {
   extern __shared__ double2 dyn[];
   __shared__ MmShared sh;
   load_tile(sh, jobs);
   const MmPlan p = T.mm[sh.J[0].plan];
-  const bool visc = tile_viscous<NT, false>(T, sh, p, mu, 0);
+  const bool visc = tile_viscous<NT, false>(T, sh, p, mu, flags, 0);
   // viscous tiles: the gradient goes through R1 (a round's opening barrier orders it)
 #pragma unroll 1
   for (int rd = visc ? 0 : 1; rd < 2; ++rd)
-    mm_round<NT, S, false, false, false>(T, p, sh, dyn, LoadQ1{e, mu, R1, Fy, T.P, T.gamma, rd == 0, visc},
+    mm_round<NT, S, false, false, false, false>(T, p, sh, dyn, LoadQ1{e, mu, R1, Fy, T.P, T.gamma, rd == 0, visc},
                                          PutField{R1, T.P});
 }
 
@@ -553,16 +94,17 @@ struct PutQ2 {
 };
 template <int NT, int S>
 __global__ void MM_BOUNDS(NT) k_mm_cart_q2(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ mu,
-                                           const double* __restrict__ R1, double* Fy, StageCoef sc) {
+                                           const double* __restrict__ R1, double* Fy,
+                                           const uint8_t* __restrict__ flags, StageCoef sc) {
   extern __shared__ double2 dyn[];
   __shared__ MmShared sh;
   load_tile(sh, jobs);
   const MmPlan p = T.mm[sh.J[0].plan];
-  const bool visc = tile_viscous<NT, true>(T, sh, p, mu, 1);
+  const bool visc = tile_viscous<NT, true>(T, sh, p, mu, flags, 1);
   const double dt = sc.rhs_only ? 0.0 : *sc.dt;
 #pragma unroll 1
   for (int rd = visc ? 0 : 1; rd < 2; ++rd)
-    mm_round<NT, S, true, false, false>(T, p, sh, dyn, LoadField{rd == 0 ? sc.Ucur : Fy, T.P},
+    mm_round<NT, S, true, false, false, false>(T, p, sh, dyn, LoadField{rd == 0 ? sc.Ucur : Fy, T.P},
                                         PutQ2{mu, R1, Fy, T.info, sc, dt, T.P, rd == 0});
 }
 
@@ -584,15 +126,17 @@ __global__ void MM_BOUNDS(NT) k_mm_filter_q1(DevTables T, const Job* __restrict_
   __shared__ MmShared sh;
   load_tile(sh, jobs);
   const MmPlan p = T.mm[sh.J[0].plan];
-  mm_round<NT, S, false, true, false>(T, p, sh, dyn, LoadTheta{e, T.P, T.gamma}, PutField{F, T.P});
+  mm_round<NT, S, false, true, false, false>(T, p, sh, dyn, LoadTheta{e, T.P, T.gamma}, PutField{F, T.P});
 }
 
 // filter, q2 lines, and E rebuilt
 struct PutEnergy {
+  using Op = NoOp;
   double* __restrict__ e;
   long long cs;
   double gamma;
-  __device__ __forceinline__ void put(long long q, const double* v) const {
+  __device__ __forceinline__ NoOp pre(long long) const { return {}; }
+  __device__ __forceinline__ void put(long long q, NoOp, const double* v) const {
     e[q] = v[0];
     e[q + cs] = v[1];
     e[q + 2 * cs] = v[2];
@@ -606,49 +150,45 @@ __global__ void MM_BOUNDS(NT) k_mm_filter_q2(DevTables T, const Job* __restrict_
   __shared__ MmShared sh;
   load_tile(sh, jobs);
   const MmPlan p = T.mm[sh.J[0].plan];
-  mm_round<NT, S, true, true, true>(T, p, sh, dyn, LoadField{F, T.P}, PutEnergy{e, T.P, T.gamma});
+  mm_round<NT, S, true, true, true, false>(T, p, sh, dyn, LoadField{F, T.P}, PutEnergy{e, T.P, T.gamma});
+}
+
+// one warp per tile: mu != 0 on one of its lines
+__global__ void k_tile_flags(const Job* __restrict__ jobs, int n, const double* __restrict__ mu,
+                             uint8_t* __restrict__ flags) {
+  const int tile = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+  if (tile >= n) return;
+  const Job* J = jobs + (size_t)tile * MM_LINES;
+  const bool col = J[0].stride != 1;
+  bool v = false;
+  for (int l = 0; l < (col ? 1 : MM_LINES); ++l) {  // columns: the four lines side by side
+    const Job& K = J[col ? (lane & 3) : l];
+    for (int t = col ? lane >> 2 : lane; t < K.n; t += col ? 8 : 32) v |= mu[K.base + (long long)t * K.stride] != 0.0;
+  }
+  v = __any_sync(0xffffffffu, v);
+  if (lane == 0) flags[tile] = v;
 }
 
 }  // namespace
 
-// 128 threads where the pairs of an inner length up to 128 fit them, 256 beyond
-#define MM_LAUNCH(KERNEL, ...)                                             \
-  do {                                                                     \
-    if (t.n <= 0) return;                                                  \
-    const size_t sm = mm_smem(t.two ? 2 : 1, t.kp);                        \
-    if (t.kp <= 128 && t.two)                                              \
-      KERNEL<128, 2><<<t.n, 128, sm, st>>>(T, t.jobs, __VA_ARGS__);        \
-    else if (t.kp <= 128)                                                  \
-      KERNEL<128, 1><<<t.n, 128, sm, st>>>(T, t.jobs, __VA_ARGS__);        \
-    else if (t.two)                                                        \
-      KERNEL<256, 2><<<t.n, 256, sm, st>>>(T, t.jobs, __VA_ARGS__);        \
-    else                                                                   \
-      KERNEL<256, 1><<<t.n, 256, sm, st>>>(T, t.jobs, __VA_ARGS__);        \
-  } while (0)
-
+void launch_tile_flags(const Job* jobs, int n, const double* mu, uint8_t* visc, cudaStream_t st) {
+  if (n > 0) k_tile_flags<<<(n + 7) / 8, 256, 0, st>>>(jobs, n, mu, visc);
+}
 void launch_mm_cart_q1(const DevTables& T, const MmTiles& t, const double* e, const double* mu, double* R1, double* Fy,
                        cudaStream_t st) {
-  MM_LAUNCH(k_mm_cart_q1, e, mu, R1, Fy);
+  MM_LAUNCH(k_mm_cart_q1, 0, e, mu, R1, Fy, t.visc);
 }
 void launch_mm_cart_q2(const DevTables& T, const MmTiles& t, const double* mu, const double* R1, double* Fy,
                        const StageCoef& sc, cudaStream_t st) {
-  MM_LAUNCH(k_mm_cart_q2, mu, R1, Fy, sc);
+  MM_LAUNCH(k_mm_cart_q2, 0, mu, R1, Fy, t.visc, sc);
 }
 void launch_mm_filter_q1(const DevTables& T, const MmTiles& t, const double* e, double* F, cudaStream_t st) {
-  MM_LAUNCH(k_mm_filter_q1, e, F);
+  MM_LAUNCH(k_mm_filter_q1, 0, e, F);
 }
 void launch_mm_filter_q2(const DevTables& T, const MmTiles& t, const double* F, double* e, cudaStream_t st) {
-  MM_LAUNCH(k_mm_filter_q2, F, e);
+  MM_LAUNCH(k_mm_filter_q2, 0, F, e);
 }
 
-namespace {
-template <class K>
-void opt_in(K k) {
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mm_smem(2, MM_KMAX));
-}
-}  // namespace
-#define MM_OPT_IN(KERNEL) \
-  opt_in(KERNEL<128, 1>), opt_in(KERNEL<128, 2>), opt_in(KERNEL<256, 1>), opt_in(KERNEL<256, 2>)
 void set_mm_attributes() {
   MM_OPT_IN(k_mm_cart_q1);
   MM_OPT_IN(k_mm_cart_q2);

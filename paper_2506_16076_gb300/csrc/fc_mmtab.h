@@ -108,11 +108,11 @@ inline MmPlan mm_plan(int L, const std::vector<long double>* sig, std::vector<ui
   p.dtab = mm_table(p, L, c, lo, hi, &p.dte);
   p.ftab = -1;
   if (sig) {
-    // cosine sums in 128-bit integers (sigma in 2^-58, cosines in 2^-60)
+    // cosine sums in 128-bit integers (sigma and cosines in 2^-58)
     std::vector<long long> sq((size_t)L / 2 + 1), cq((size_t)L);
     for (int k = 0; 2 * k <= L; ++k) sq[k] = (long long)std::llround(std::ldexp((*sig)[k], 58));
     for (int j = 0; 2 * j <= L; ++j) {
-      cq[j] = (long long)std::llround(std::ldexp(cs[4 * j], 60));
+      cq[j] = (long long)std::llround(std::ldexp(cs[4 * j], 58));
       if (j) cq[L - j] = cq[j];
     }
     for (int m = 0; 2 * m <= L; ++m) {
@@ -121,7 +121,7 @@ inline MmPlan mm_plan(int L, const std::vector<long double>* sig, std::vector<ui
       a *= 2;
       a += (__int128)sq[0] * cq[0];
       if (L % 2 == 0) a += (__int128)sq[L / 2] * cq[(size_t)((long long)(L / 2) * m % L)];
-      const long double v = std::ldexp((long double)a, -118) / L;
+      const long double v = std::ldexp((long double)a, -116) / L;
       c[m] = v;
       if (m) c[L - m] = v;
     }

@@ -106,4 +106,69 @@ __device__ __forceinline__ double energy_of(double r, double mx, double my, doub
   return r * th / (gam - 1.0) + 0.5 * (mx * mx + my * my) / r;
 }
 
+// A^T eta for the x (dir 0) or y (dir 1) flux Jacobian at state e (eq. euler 2d equation)
+__device__ __forceinline__ void fluxT(int dir, double r, double mx, double my, double E, double gam, const double* eta,
+                                      double* out) {
+  const double ir = 1.0 / r;
+  const double u = mx * ir, v = my * ir;
+  const double g1 = gam - 1.0;
+  const double q2 = u * u + v * v;
+  const double p = g1 * (E - 0.5 * r * q2);
+  const double H = (E + p) * ir;
+  const double pr = 0.5 * g1 * q2, pm = -g1 * u, pn = -g1 * v, pE = g1;
+  if (dir == 0) {
+    // rows c = 0..3 of A_x, columns j: out_j = sum_c A[c][j] eta_c
+    out[0] = (-u * u + pr) * eta[1] + (-u * v) * eta[2] + (-u * H + u * pr) * eta[3];
+    out[1] = eta[0] + (2.0 * u + pm) * eta[1] + v * eta[2] + (H + u * pm) * eta[3];
+    out[2] = pn * eta[1] + u * eta[2] + u * pn * eta[3];
+    out[3] = pE * eta[1] + u * (1.0 + pE) * eta[3];
+  } else {
+    out[0] = (-u * v) * eta[1] + (-v * v + pr) * eta[2] + (-v * H + v * pr) * eta[3];
+    out[1] = v * eta[1] + pm * eta[2] + v * pm * eta[3];
+    out[2] = eta[0] + u * eta[1] + (2.0 * v + pn) * eta[2] + (H + v * pn) * eta[3];
+    out[3] = pE * eta[2] + v * (1.0 + pE) * eta[3];
+  }
+}
+
+// Jacobian transposes of the filter's pointwise maps: of E rebuilt from the filtered
+// (rho, rho u, rho v, theta) at the filtered state ef, and of theta(e)
+__device__ __forceinline__ void rebuild_T(const double* lam, const double* ef, double gam, double* o) {
+  const double r = ef[0], m = ef[1], nn = ef[2];
+  const double th = theta_of(r, m, nn, ef[3], gam);
+  const double g1 = gam - 1.0, lE = lam[3], ir = 1.0 / r;
+  o[0] = lam[0] + lE * (th / g1 - 0.5 * (m * m + nn * nn) * ir * ir);
+  o[1] = lam[1] + lE * m * ir;
+  o[2] = lam[2] + lE * nn * ir;
+  o[3] = lE * r / g1;
+}
+__device__ __forceinline__ void rebuild_T(const double* __restrict__ lam, const double* __restrict__ ef, long long p,
+                                          long long cs, double gam, double* o) {
+  const double l[4] = {lam[p], lam[p + cs], lam[p + 2 * cs], lam[p + 3 * cs]};
+  const double f[4] = {ef[p], ef[p + cs], ef[p + 2 * cs], ef[p + 3 * cs]};
+  rebuild_T(l, f, gam, o);
+}
+__device__ __forceinline__ void theta_T(const double* q, const double* e, double gam, double* o) {
+  const double r = e[0], m = e[1], nn = e[2], E = e[3];
+  const double g1 = gam - 1.0, lt = q[3], ir = 1.0 / r, ir2 = ir * ir;
+  o[0] = q[0] + lt * g1 * (-E * ir2 + (m * m + nn * nn) * ir2 * ir);
+  o[1] = q[1] + lt * (-g1 * m * ir2);
+  o[2] = q[2] + lt * (-g1 * nn * ir2);
+  o[3] = lt * g1 * ir;
+}
+__device__ __forceinline__ void theta_T(const double* q, const double* __restrict__ e, long long p, long long cs,
+                                        double gam, double* o) {
+  const double f[4] = {e[p], e[p + cs], e[p + 2 * cs], e[p + 3 * cs]};
+  theta_T(q, f, gam, o);
+}
+
+// (dQ/du)^T a for Q = (rho, rho u, rho v, theta), theta = (gamma - 1) (E / rho - |rho u|^2 / (2 rho^2))
+__device__ __forceinline__ void thetaT_add(const double* u, double gam, const double* a, double* out) {
+  const double ir = 1.0 / u[0], g1 = gam - 1.0;
+  const double m2 = fma(u[1], u[1], u[2] * u[2]);
+  out[0] += a[0] + a[3] * g1 * ir * ir * (m2 * ir - u[3]);
+  out[1] += a[1] - a[3] * g1 * u[1] * ir * ir;
+  out[2] += a[2] - a[3] * g1 * u[2] * ir * ir;
+  out[3] += a[3] * g1 * ir;
+}
+
 }  // namespace fcx

@@ -97,8 +97,10 @@ int main(int argc, char** argv) {
         double level = 0;
         for (int s = 0; s < p.S; ++s)
           for (int i = 0; i < p.H; ++i) {
+            long long joined = 0;
+            for (int kb = 0; kb < p.H; kb += MM_KCHUNK) {
             double lev[SP_DIGITS] = {0};
-            for (int k = 0; k < p.H; ++k) {
+            for (int k = kb; k < std::min(p.H, kb + MM_KCHUNK); ++k) {
               const long long x0 = sp_fixed(x[k], ex), x1 = p.S == 2 ? sp_fixed(x[k + p.H], ex) : 0;
               const long long b = (s ? x0 - x1 : x0 + x1) + SP_BIAS;
               const int at = tab + s * p.nx + k - i + p.Mp;
@@ -112,7 +114,9 @@ int main(int argc, char** argv) {
               si[l] = (int)lev[l];
               level = std::max(level, std::fabs(lev[l]));
             }
-            W[s].push_back(sp_join(si));
+            joined += sp_join(si);
+            }
+            W[s].push_back(joined);
           }
         const double fac = std::scalbn(1.0, ex - 1023 - SP_DATA + SP_UNIT - te - (p.S - 1));
         double err = 0;

@@ -5,9 +5,9 @@ long double.
 
 Tolerance, relative to the line's largest value (coefficients at most about 1): the dropped
 digit products are sums of 5 H pairs of digits of standard deviation 2^8.2 in units 2^40, the
-largest value is at least 2^56 times a coefficient of 2^59.5: 2^-54 for H = 256; truncated
+largest value is at least 2^56 times a coefficient of 2^59.5: 2^-53.5 for H = 512; truncated
 data and rounded coefficients add less. Eight times that, for the largest of all rows and
-both parts, and one FP64 rounding: 2^-51 + 2^-52 < 7e-16. Level sums must stay below 2^24,
+both parts, and one FP64 rounding: 2^-50.5 + 2^-52 < 9e-16. Level sums must stay below 2^24,
 where FP32 accumulation stops being exact."""
 import os
 import shutil
@@ -32,7 +32,7 @@ def exe(tmp_path_factory):
 
 
 # edges of the padding to 16, both parities, the shortest and the longest inner lengths
-LENGTHS = [16, 17, 30, 31, 32, 33, 34, 37, 64, 66, 155, 192, 224, 255, 256, 258, 288, 432, 510, 512]
+LENGTHS = [16, 17, 30, 31, 32, 33, 34, 37, 64, 66, 155, 192, 224, 255, 256, 258, 288, 432, 510, 512, 514, 509, 800, 1024]
 
 
 def test_contraction_matches_the_circulant(exe):
@@ -41,12 +41,12 @@ def test_contraction_matches_the_circulant(exe):
     rows = [ln.split() for ln in r.stdout.splitlines()]
     assert len(rows) == 6 * len(LENGTHS)
     for L, op, kind, err, level in rows:
-        assert float(err) < 7e-16, (L, op, kind, err)
+        assert float(err) < 9e-16, (L, op, kind, err)
         assert float(level) < 2 ** 24, (L, op, kind, level)
 
 
 def test_other_lengths_are_left_to_the_transforms(exe):
-    r = subprocess.run([exe, "15", "257", "514", "1024"], capture_output=True, text=True)
+    r = subprocess.run([exe, "15", "513", "1026", "2048"], capture_output=True, text=True)
     assert r.returncode == 0 and [ln.split()[1] for ln in r.stdout.splitlines()] == ["none"] * 4
 
 

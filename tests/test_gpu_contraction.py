@@ -1,10 +1,12 @@
 """The tensor-core contraction of FC lines on the GPU at the sizes where it can go wrong:
-inner lengths around the padding to 16 and around the two CTA sizes (128 and 129), the
+inner lengths around the padding to 16 and around the CTA sizes (128 / 129, 256 / 258), the
 longest contracted lengths and the first ones left to the transforms, odd lengths, tiles
 with absent lines; lines of zeros and non-finite values.
 
 Tolerance of the operator as in the other edge cases: 1e-11, or twice the error of an FP64
 FFT evaluation where that is larger."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -22,8 +24,9 @@ def _box(n1, n2):
     return W.Workload(f"box_{n1}x{n2}", [p], W.Params(c_policy=0), fs, "freestream", 1)
 
 
-# n + 27: 64, 66, 128, 256 / 258 (inner 128 / 129), 512 and 513 (transforms), odd 255 and 259 (transforms)
-CASES = [(37, 39), (101, 10), (229, 231), (485, 13), (486, 11), (228, 14), (232, 17)]
+# n + 27: 64, 66, 128, 256 / 258 (inner 128 / 129), 512 / 516 (256 / 258), odd 255, 259 and 513, 1024 and
+# 1026 (transforms)
+CASES = [(37, 39), (101, 10), (229, 231), (485, 13), (489, 11), (228, 14), (232, 17), (486, 10), (997, 12), (999, 10)]
 
 
 @pytest.mark.parametrize("n1,n2", CASES)
@@ -81,3 +84,21 @@ def test_non_finite_point_spoils_its_lines_only(gpu_lib, bad):
     keep[j, :] = False
     keep[:, i] = False
     assert torch.equal(out.reshape(4, n2, n1)[:, keep], good.reshape(4, n2, n1)[:, keep])
+
+
+@pytest.mark.parametrize("wall_form", [0, 1])
+def test_curvilinear_patch_after_affine_ones(gpu_lib, wall_form):
+    # the scratch of a curvilinear patch starts at another index than its points; 126 radial
+    # lines leave a tile with absent lines
+    w = W.small_multipatch(W.ADIABATIC)
+    og = dataclasses.replace(w.patches[0], n1=126)
+    w = dataclasses.replace(w, patches=w.patches[1:] + [og], params=dataclasses.replace(w.params, wall_form=wall_form))
+    ctx = gpu_lib.Context(w)
+    sv = S.Solver(w)
+    st = W.random_smooth_state(w, seed=6, amp=0.2)
+    mu = smooth_mu(w, seed=2, scale=0.01)
+    e = to_dev(st)
+    out = torch.empty_like(e)
+    ctx.rhs(e, out, to_dev_scalar_field(mu))
+    errs = rel_err(from_dev(out, w), sv.rhs(st, mu))
+    assert max(errs) < 1e-11, errs
