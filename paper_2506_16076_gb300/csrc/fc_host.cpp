@@ -1073,7 +1073,9 @@ void make_tiles(fc_ctx* c, fc_ctx::Queue& q, const std::vector<Job>& pp, const s
   std::stable_sort(tiles.begin(), tiles.end(), order);
   put(tiles, q.mm, flat);
   q.ntiles = (int)tiles.size();
-  ok = ok && c->upload(&q.dmm, flat) && c->alloc(&q.dvisc, flat.size() / MM_LINES);
+  q.dmm = nullptr;
+  q.dvisc = nullptr;
+  ok = ok && (flat.empty() || (c->upload(&q.dmm, flat) && c->alloc(&q.dvisc, flat.size() / MM_LINES)));
   auto fix = [&](MmTiles& m) {
     const uintptr_t first = (uintptr_t)m.jobs;
     m.jobs = q.dmm + first;
@@ -1117,7 +1119,8 @@ void make_queue(fc_ctx* c, fc_ctx::Queue& q, std::vector<Job>& jobs, const std::
     q.class_end.push_back(e);
     k = e;
   }
-  ok = ok && c->upload(&q.d, jobs) && c->upload(&q.dpp, pp);
+  q.d = q.dpp = nullptr;  // (an empty queue uploads nothing: device allocations cost more than the rest)
+  ok = ok && (jobs.empty() || (c->upload(&q.d, jobs) && c->upload(&q.dpp, pp)));
   q.h = jobs;
   if (mm) make_tiles(c, q, pp, plans, npatch, ok, *mm);
 }
@@ -1772,6 +1775,7 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   set_mm_attributes();
   set_mm_gen_attributes();
   set_mm_adj_attributes();
+  set_mm_adj_gen_attributes();
   if (!mpts.empty()) {  // metrics of GRID patches given by their points only
     std::vector<double> xy(2 * (size_t)c->P, 0.0);
     for (const HPatch& h : c->hp)
@@ -2161,12 +2165,23 @@ void adj_stage(fc_ctx* c, const double* u, const double* mu, const double* psi, 
                cudaStream_t st) {
   const DevTables& T = c->T;
   cudaMemsetAsync(c->d_R1, 0, sizeof(double) * 4 * (size_t)c->P, st);
+  // as in stage(): the curvilinear chain has patches of its own and runs on a side stream (an
+  // O-grid's few long lines leave most of the chip to the affine chain)
+  const bool overlap = c->concurrent && !c->prof && c->q_gen1.n > 0 && c->q_cart1.n > 0 && c->ensure_side();
+  cudaStream_t sg = st;
+  int gside = 1;
+  if (overlap) {
+    cudaEventRecord(c->fork_ev[1], st);
+    cudaStreamWaitEvent(c->side[0], c->fork_ev[1], 0);
+    sg = c->side[0];
+    gside = fc_ctx::NSIDE;
+  }
   run_queue(
-      c, c->q_gen1, false, st, "adj_gen_A",
-      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_A(T, j, n, L, c->d_J, u, psi, c->d_G, s); }, 1,
+      c, c->q_gen1, false, sg, "adj_gen_A",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_A(T, j, n, L, c->d_J, u, psi, c->d_G, s); }, gside,
       [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_gen_A(T, t, c->d_J, u, psi, c->d_G, s); });
   if (c->ngfix) {
-    launch_adj_gen_fixA(T, c->d_gfix, c->ngfix, c->d_J, u, mu, psi, c->d_G, st);
+    launch_adj_gen_fixA(T, c->d_gfix, c->ngfix, c->d_J, u, mu, psi, c->d_G, sg);
     c->launches++;
   }
   // (the y-flux buffer carries the contraction kernels' mu eta between their two rounds)
@@ -2175,15 +2190,15 @@ void adj_stage(fc_ctx* c, const double* u, const double* mu, const double* psi, 
       [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_cart(T, j, n, L, 0, u, mu, psi, c->d_R1, acc, dt, s); },
       1, [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_cart(T, flagged(c, t), 0, u, mu, psi, c->d_R1, acc, c->d_Fy, dt, s); });
   run_queue(
-      c, c->q_gen2, false, st, "adj_gen_B",
-      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_B(T, j, n, L, c->d_J, u, mu, psi, c->d_G, s); }, 1,
+      c, c->q_gen2, false, sg, "adj_gen_B",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_B(T, j, n, L, c->d_J, u, mu, psi, c->d_G, s); }, gside,
       [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_gen_B(T, t, c->d_J, u, mu, psi, c->d_G, s); });
   if (T.any_pform)
-    run_queue(c, c->q_gen2, false, st, "adj_gen_B", [&](const Job* j, int n, int L, cudaStream_t s) {
+    run_queue(c, c->q_gen2, false, sg, "adj_gen_B", [&](const Job* j, int n, int L, cudaStream_t s) {
       launch_adj_gen_B_wall(T, j, n, L, c->d_J, u, mu, psi, c->d_G, s);
-    });
+    }, gside);
   if (c->ngfix) {
-    launch_adj_gen_fixB(T, c->d_gfix, c->ngfix, c->d_G, c->d_R1, st);
+    launch_adj_gen_fixB(T, c->d_gfix, c->ngfix, c->d_G, c->d_R1, sg);
     c->launches++;
   }
   run_queue(
@@ -2191,9 +2206,13 @@ void adj_stage(fc_ctx* c, const double* u, const double* mu, const double* psi, 
       [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_cart(T, j, n, L, 1, u, mu, psi, c->d_R1, acc, dt, s); },
       1, [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_cart(T, flagged(c, t), 1, u, mu, psi, c->d_R1, acc, c->d_Fy, dt, s); });
   run_queue(
-      c, c->q_gen1, false, st, "adj_gen_C",
-      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_C(T, j, n, L, u, c->d_G, acc, dt, s); }, 1,
+      c, c->q_gen1, false, sg, "adj_gen_C",
+      [&](const Job* j, int n, int L, cudaStream_t s) { launch_adj_gen_C(T, j, n, L, u, c->d_G, acc, dt, s); }, gside,
       [&](const MmTiles& t, cudaStream_t s) { launch_mm_adj_gen_C(T, t, u, c->d_G, acc, dt, s); });
+  if (overlap) {
+    cudaEventRecord(c->join_ev[0], c->side[0]);
+    cudaStreamWaitEvent(st, c->join_ev[0], 0);
+  }
   if (c->nfix) {
     launch_adj_fixup(c->d_fix, c->nfix, c->d_R1, acc, c->P, dt, st);
     c->launches++;
@@ -2202,6 +2221,11 @@ void adj_stage(fc_ctx* c, const double* u, const double* mu, const double* psi, 
 
 void axpby(fc_ctx* c, double a, const double* x, double b, double* y, cudaStream_t st) {
   launch_axpby(4 * c->P, a, x, b, y, st);
+  c->launches++;
+}
+
+void axpby_many(fc_ctx* c, const double* x, const AxpbyMany& m, cudaStream_t st) {
+  launch_axpby_many(4 * c->P, x, m, st);
   c->launches++;
 }
 
@@ -2701,30 +2725,20 @@ fc_status fc_adjoint_step(fc_ctx* c, const double* e_n, const double* mu, const 
   // reverse sweep (Shu-Osher coefficients, see the forward stages)
   axpby(c, 1.0, lam_np1, 0.0, A14, st);
   projectT(c, A14, gbc, A3, st);  // lam_v5
-  axpby(c, A53, A14, 0.0, A3, st);
-  axpby(c, B53, A14, 0.0, PSb, st);
-  axpby(c, A52, A14, 0.0, A2, st);
-  axpby(c, B54, A14, 0.0, PSa, st);
-  axpby(c, A54, A14, 0.0, A14, st);  // lam_u4 (without its L' term)
+  axpby_many(c, A14, {5, {A3, PSb, A2, PSa, A14}, {A53, B53, A52, B54, A54}, {0.0, 0.0, 0.0, 0.0, 0.0}},
+             st);  // A14: lam_u4 (without its L' term)
   adj_stage(c, U[4], mu, PSa, A14, dt, st);
   projectT(c, A14, gbc, U[4], st);  // lam_v4
-  axpby(c, A40, A14, 0.0, A0, st);
-  axpby(c, A43, A14, 1.0, A3, st);
-  axpby(c, B4, A14, 1.0, PSb, st);
+  axpby_many(c, A14, {3, {A0, A3, PSb}, {A40, A43, B4}, {0.0, 1.0, 1.0}}, st);
   adj_stage(c, U[3], mu, PSb, A3, dt, st);
   projectT(c, A3, gbc, U[3], st);  // lam_v3
-  axpby(c, A30, A3, 1.0, A0, st);
-  axpby(c, A32, A3, 1.0, A2, st);
-  axpby(c, B3, A3, 0.0, PSa, st);
+  axpby_many(c, A3, {3, {A0, A2, PSa}, {A30, A32, B3}, {1.0, 1.0, 0.0}}, st);
   adj_stage(c, U[2], mu, PSa, A2, dt, st);
   projectT(c, A2, gbc, U[2], st);  // lam_v2
-  axpby(c, A20, A2, 1.0, A0, st);
-  axpby(c, A21, A2, 0.0, A14, st);
-  axpby(c, B2, A2, 0.0, PSb, st);
+  axpby_many(c, A2, {3, {A0, A14, PSb}, {A20, A21, B2}, {1.0, 0.0, 0.0}}, st);
   adj_stage(c, U[1], mu, PSb, A14, dt, st);
   projectT(c, A14, gbc, U[1], st);  // lam_v1
-  axpby(c, 1.0, A14, 1.0, A0, st);
-  axpby(c, B1, A14, 0.0, PSa, st);
+  axpby_many(c, A14, {2, {A0, PSa}, {1.0, B1}, {1.0, 0.0}}, st);
   adj_stage(c, U[0], mu, PSa, A0, dt, st);
   projectT(c, A0, gbc, U[0], st);
   if (filt) {  // transposes of F and of the projection before it

@@ -214,6 +214,7 @@ void launch_mm_filterT_q1(const DevTables& T, const MmTiles& t, const double* MF
 void set_mm_attributes();
 void set_mm_gen_attributes();
 void set_mm_adj_attributes();
+void set_mm_adj_gen_attributes();
 
 // ---- launch wrappers (fc_kernels.cu) ----
 // Fy (nullable): the y fluxes of the affine points, written by the q1 pass (and by
@@ -307,6 +308,14 @@ void launch_init_sens(const uint32_t* info, const uint8_t* owned, long long P, c
 void launch_drag(const int* wall, const double* w, const double* nx, int n, const double* e, long long P, double gam,
                  double* J, double* dJde, cudaStream_t st);
 void launch_axpby(long long n, double a, const double* x, double b, double* y, cudaStream_t st);
+// y[k] = a[k] x + b[k] y[k], k < n (b[k] == 0: y[k] is not read); only the last y may be x
+struct AxpbyMany {
+  static constexpr int MOST = 5;
+  int n;
+  double* y[MOST];
+  double a[MOST], b[MOST];
+};
+void launch_axpby_many(long long n, const double* x, const AxpbyMany& m, cudaStream_t st);
 int length_class(int Lmax);
 size_t line_smem_bytes(const DevTables& T, int Lmax);
 int line_warps(const DevTables& T, int Lmax);

@@ -2068,6 +2068,21 @@ __global__ void k_axpby(long long n, double a, const double* __restrict__ x, dou
   y[i] = (b == 0.0) ? a * x[i] : fma(a, x[i], b * y[i]);
 }
 
+// the same for up to five y of one x, which is read once (the reverse sweep's weights of a
+// stage's adjoint); x may be the last y
+__global__ void k_axpby_many(long long n, const double* x, AxpbyMany m) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double v = x[i];
+  double y[AxpbyMany::MOST];
+#pragma unroll
+  for (int k = 0; k < AxpbyMany::MOST; ++k)
+    if (k < m.n && m.b[k] != 0.0) y[k] = m.y[k][i];
+#pragma unroll
+  for (int k = 0; k < AxpbyMany::MOST; ++k)
+    if (k < m.n) m.y[k][i] = m.b[k] == 0.0 ? m.a[k] * v : fma(m.a[k], v, m.b[k] * y[k]);
+}
+
 // ---------------------------------------------------------------- wall drag functional
 // J = sum_i w_i n_x,i p_i over the wall ring (periodic trapezoid of the wall-pressure integral);
 // dJde (optional): its gradient at the wall points, zero elsewhere (caller zeroes it)
@@ -2328,6 +2343,10 @@ void launch_fill_wave(double* p, long long n, double a, double b, double w, cuda
 }
 void launch_axpby(long long n, double a, const double* x, double b, double* y, cudaStream_t st) {
   k_axpby<<<grid_pts(n, 256), 256, 0, st>>>(n, a, x, b, y);
+}
+
+void launch_axpby_many(long long n, const double* x, const AxpbyMany& m, cudaStream_t st) {
+  k_axpby_many<<<grid_pts(n, 256), 256, 0, st>>>(n, x, m);
 }
 
 void launch_drag(const int* wall, const double* w, const double* nx, int n, const double* e, long long P, double gam,

@@ -33,19 +33,19 @@ struct LoadQ1 {
     for (int c = 0; c < 4; ++c) v[c] = f[c];
   }
 };
-template <int NT, int S>
-__global__ void MM_BOUNDS(NT) k_mm_cart_q1(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ e,
+template <class Cfg>
+__global__ void MM_BOUNDS k_mm_cart_q1(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ e,
                                            const double* __restrict__ mu, double* R1, double* __restrict__ Fy,
                                            const uint8_t* __restrict__ flags) {
   extern __shared__ double2 dyn[];
   __shared__ MmShared sh;
   load_tile(sh, jobs);
   const MmPlan p = T.mm[sh.J[0].plan];
-  const bool visc = tile_viscous<NT, false>(T, sh, p, mu, flags, 0);
+  const bool visc = tile_viscous<Cfg::NT, false>(T, sh, p, mu, flags, 0);
   // viscous tiles: the gradient goes through R1 (a round's opening barrier orders it)
 #pragma unroll 1
   for (int rd = visc ? 0 : 1; rd < 2; ++rd)
-    mm_round<NT, S, false, false, false, false>(T, p, sh, dyn, LoadQ1{e, mu, R1, Fy, T.P, T.gamma, rd == 0, visc},
+    mm_round<Cfg, false, false, false, false>(T, p, sh, dyn, LoadQ1{e, mu, R1, Fy, T.P, T.gamma, rd == 0, visc},
                                          PutField{R1, T.P});
 }
 
@@ -92,19 +92,19 @@ struct PutQ2 {
       stage_put(sc, dt, qc, (o.info & PT_NODIFF) ? 0.0 : -(o.a + v), o.cur, o.u0, o.aux);
   }
 };
-template <int NT, int S>
-__global__ void MM_BOUNDS(NT) k_mm_cart_q2(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ mu,
+template <class Cfg>
+__global__ void MM_BOUNDS k_mm_cart_q2(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ mu,
                                            const double* __restrict__ R1, double* Fy,
                                            const uint8_t* __restrict__ flags, StageCoef sc) {
   extern __shared__ double2 dyn[];
   __shared__ MmShared sh;
   load_tile(sh, jobs);
   const MmPlan p = T.mm[sh.J[0].plan];
-  const bool visc = tile_viscous<NT, true>(T, sh, p, mu, flags, 1);
+  const bool visc = tile_viscous<Cfg::NT, true>(T, sh, p, mu, flags, 1);
   const double dt = sc.rhs_only ? 0.0 : *sc.dt;
 #pragma unroll 1
   for (int rd = visc ? 0 : 1; rd < 2; ++rd)
-    mm_round<NT, S, true, false, false, false>(T, p, sh, dyn, LoadField{rd == 0 ? sc.Ucur : Fy, T.P},
+    mm_round<Cfg, true, false, false, false>(T, p, sh, dyn, LoadField{rd == 0 ? sc.Ucur : Fy, T.P},
                                         PutQ2{mu, R1, Fy, T.info, sc, dt, T.P, rd == 0});
 }
 
@@ -119,14 +119,14 @@ struct LoadTheta {
   }
   __device__ __forceinline__ void form(long long, double* v) const { v[3] = theta_of(v[0], v[1], v[2], v[3], gamma); }
 };
-template <int NT, int S>
-__global__ void MM_BOUNDS(NT) k_mm_filter_q1(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ e,
+template <class Cfg>
+__global__ void MM_BOUNDS k_mm_filter_q1(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ e,
                                              double* __restrict__ F) {
   extern __shared__ double2 dyn[];
   __shared__ MmShared sh;
   load_tile(sh, jobs);
   const MmPlan p = T.mm[sh.J[0].plan];
-  mm_round<NT, S, false, true, false, false>(T, p, sh, dyn, LoadTheta{e, T.P, T.gamma}, PutField{F, T.P});
+  mm_round<Cfg, false, true, false, false>(T, p, sh, dyn, LoadTheta{e, T.P, T.gamma}, PutField{F, T.P});
 }
 
 // filter, q2 lines, and E rebuilt
@@ -143,14 +143,14 @@ struct PutEnergy {
     e[q + 3 * cs] = energy_of(v[0], v[1], v[2], v[3], gamma);
   }
 };
-template <int NT, int S>
-__global__ void MM_BOUNDS(NT) k_mm_filter_q2(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ F,
+template <class Cfg>
+__global__ void MM_BOUNDS k_mm_filter_q2(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ F,
                                              double* __restrict__ e) {
   extern __shared__ double2 dyn[];
   __shared__ MmShared sh;
   load_tile(sh, jobs);
   const MmPlan p = T.mm[sh.J[0].plan];
-  mm_round<NT, S, true, true, true, false>(T, p, sh, dyn, LoadField{F, T.P}, PutEnergy{e, T.P, T.gamma});
+  mm_round<Cfg, true, true, true, false>(T, p, sh, dyn, LoadField{F, T.P}, PutEnergy{e, T.P, T.gamma});
 }
 
 // one warp per tile: mu != 0 on one of its lines

@@ -50,16 +50,9 @@ struct MmShared {
 
 constexpr int LB = 4;  // points of a thread whose loads are in flight together
 
-// columns of the lines' values in shared memory: a pitch of 4 (mod 16) doubles keeps the
-// four lines of a row of q2 points in different banks
+// pitch of a column's values in shared memory: 4 (mod 16) doubles keep the four lines of a
+// row of q2 points in different banks
 __host__ __device__ inline int mm_line_pitch(int L) { return L + ((4 - L % 16) + 16) % 16; }
-// dynamic shared memory: the digits [S][SP_DIGITS][NCOL][Kp + 8] of FP16 (columns padded by
-// 16 bytes: conflict-free ldmatrix), over the continued lines [NCOL][pitch] they come from
-inline size_t mm_smem(int S, int Kp) {
-  const size_t dig = (size_t)S * SP_DIGITS * NCOL * (Kp + 8) * 2;
-  const size_t val = (size_t)NCOL * mm_line_pitch(S * Kp) * sizeof(double);
-  return dig > val ? dig : val;
-}
 
 __device__ __forceinline__ void mma16816(float* c, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                          uint32_t b1) {
@@ -103,19 +96,20 @@ __device__ __forceinline__ uint32_t digit_pair(long long a, long long b, int k) 
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// adds the joined sums of one part over columns kb..ke-1 for the warp's 16 rows from i0:
-// W[r * 4 + nt * 2 + c] is row i0 + g + 8 r, column nt * 8 + 2 t + c (g = lane / 4, t = lane % 4)
-__device__ __forceinline__ void mm_part(const uint4* __restrict__ lo, const uint2* __restrict__ hi, uint32_t dig,
-                                        int pitch, const MmPlan& p, int i0, int kb, int ke, int lane, long long* W) {
+// adds the joined sums of one part over columns kb..ke-1 for the warp's 16 rows from i0 and
+// its 8 columns: W[r * 2 + c] is row i0 + g + 8 r, column 2 t + c (g = lane / 4, t = lane % 4)
+// (x0: table entry of row i0, column 0)
+__device__ __forceinline__ void mm_part(const uint4* __restrict__ lo, const uint2* __restrict__ hi, int x0,
+                                        uint32_t dig, int pitch, int kb, int ke, int lane, long long* W) {
   const int g = lane >> 2, t = lane & 3;
-  float acc[SP_DIGITS][2][4];
+  float acc[SP_DIGITS][4];
 #pragma unroll
   for (int l = 0; l < SP_DIGITS; ++l)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[l][0][q] = acc[l][1][q] = 0.f;
-  const uint4* pl = lo + (p.Mp - i0 + kb + 2 * t - g);
-  const uint2* ph = hi + (p.Mp - i0 + kb + 2 * t - g);
-  uint32_t Am[SP_DIGITS], A0[SP_DIGITS], Ap[SP_DIGITS], N0[SP_DIGITS], Np[SP_DIGITS];
+    for (int q = 0; q < 4; ++q) acc[l][q] = 0.f;
+  const uint4* pl = lo + (x0 + kb + 2 * t - g);
+  const uint2* ph = hi + (x0 + kb + 2 * t - g);
+  uint32_t Am[SP_DIGITS], A0[SP_DIGITS], Ap[SP_DIGITS];
   auto entry = [&](uint32_t* A, int x) {
     const uint4 a = ldg_keep(pl + x);
     const uint2 b = ldg_keep(ph + x);
@@ -127,40 +121,32 @@ __device__ __forceinline__ void mm_part(const uint4* __restrict__ lo, const uint
     A[5] = b.y;
   };
   entry(Am, -8);
-  entry(A0, 0);
-  entry(Ap, 8);
-  // ldmatrix row addresses: matrices (columns 0-7, k), (columns 0-7, k+8), (8-15, k), (8-15, k+8)
-  uint32_t baddr = dig + (uint32_t)(((lane & 7) + ((lane >> 4) << 3)) * pitch + ((lane >> 3) & 1) * 16 + kb * 2);
-  const uint32_t bslice = (uint32_t)NCOL * pitch;
+  // ldmatrix: the 8 columns of two digits, at k and k + 8 each
+  const uint32_t slice = (uint32_t)NCOL * pitch;
+  uint32_t baddr = dig + (uint32_t)((lane & 7) * pitch + ((lane >> 3) & 1) * 16 + kb * 2) + (lane >> 4) * slice;
+#pragma unroll 1
   for (int k0 = 0; k0 < ke - kb; k0 += 16) {
-    const int kn = k0 + 16 < ke - kb ? k0 + 16 : k0;  // the next step's entries, a whole step ahead
-    entry(N0, kn);
-    entry(Np, kn + 8);
-    uint32_t b[2][4];
-    ldsm4(b[0], baddr);
+    entry(A0, k0);
+    entry(Ap, k0 + 8);
 #pragma unroll
-    for (int j = 0; j < SP_DIGITS; ++j) {
-      if (j + 1 < SP_DIGITS) ldsm4(b[(j + 1) & 1], baddr + (j + 1) * bslice);
-      const uint32_t* c = b[j & 1];
+    for (int j2 = 0; j2 < SP_DIGITS; j2 += 2) {
+      uint32_t b[4];
+      ldsm4(b, baddr + j2 * slice);
 #pragma unroll
-      for (int i = 0; i + j < SP_DIGITS; ++i) {
-        mma16816(acc[i + j][0], A0[i], Am[i], Ap[i], A0[i], c[0], c[1]);
-        mma16816(acc[i + j][1], A0[i], Am[i], Ap[i], A0[i], c[2], c[3]);
+      for (int i = 0; i + j2 < SP_DIGITS; ++i) {
+        mma16816(acc[i + j2], A0[i], Am[i], Ap[i], A0[i], b[0], b[1]);
+        if (i + j2 + 1 < SP_DIGITS) mma16816(acc[i + j2 + 1], A0[i], Am[i], Ap[i], A0[i], b[2], b[3]);
       }
     }
     baddr += 32;
 #pragma unroll
-    for (int i = 0; i < SP_DIGITS; ++i) {
-      Am[i] = Ap[i];
-      A0[i] = N0[i];
-      Ap[i] = Np[i];
-    }
+    for (int i = 0; i < SP_DIGITS; ++i) Am[i] = Ap[i];
   }
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
+  for (int q = 0; q < 4; ++q) {
     int s[SP_DIGITS];
 #pragma unroll
-    for (int l = 0; l < SP_DIGITS; ++l) s[l] = __float2int_rn(acc[l][(q >> 1) & 1][(q >> 2) * 2 + (q & 1)]);
+    for (int l = 0; l < SP_DIGITS; ++l) s[l] = __float2int_rn(acc[l][q]);
     W[q] += sp_join(s);
   }
 }
@@ -203,10 +189,10 @@ __device__ __forceinline__ void continuation(const double* __restrict__ M, int C
 // with a barrier. TR (with PT): the transposed operator (eqs. fc_der and filtering of a line
 // extended by zeros; the derivative's circulant is odd, its transpose the negative; the
 // results at the continuation points are folded back onto the first and last d points).
-template <int NT, int S, bool COL, bool FILT, bool PT, bool TR, class Load, class Ep>
+template <class Cfg, bool COL, bool FILT, bool PT, bool TR, class Load, class Ep>
 __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan, MmShared& sh, double2* dyn, Load ld,
                                          Ep ep) {
-  constexpr int NW = NT / 32, TS = NT / 4;  // TS: points per step of a line
+  constexpr int NT = Cfg::NT, S = Cfg::S, NW = NT / 32, TS = NT / 4;  // TS: points per step of a line
   // opaque copies: without them the compiler hoists the address arithmetic of both of a
   // kernel's rounds out of their loop (250 registers, 280 bytes of spills; so 128 and < 100)
   int tid = threadIdx.x;
@@ -303,12 +289,16 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
   }
 
   // (3) digits of the parts, over the values: all reads come before the first write. A warp
-  // per line again, lanes along the pairs (2q, 2q + 1)
+  // per line again, lanes along the pairs (2q, 2q + 1). Digit column of (component, line):
+  // 8 (line / 2) + 2 component + line % 2, so that a warp's 8 columns are two lines whole
+  const int pitch = (p.Kp + 8) * 2;                         // bytes per column
+  const uint32_t part1 = (uint32_t)(SP_DIGITS * NCOL) * pitch;  // bytes per part
   {
+    constexpr int R = Cfg::R;  // pairs per thread
     const int line = warp & 3, q0 = (warp >> 2) * 32 + lane;
-    double X[2][4][S][2];
+    double X[R][4][S][2];
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
       for (int c = 0; c < 4; ++c)
 #pragma unroll
@@ -322,10 +312,9 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
 #pragma unroll
     for (int c = 0; c < 4; ++c) ex[c] = (int)(sh.emax[c * MM_LINES + line] >> 20);
     __syncthreads();
-    const int pitchw = (p.Kp + 8) / 2;  // words per column
-    uint32_t* dig = reinterpret_cast<uint32_t*>(dyn);
+    char* dig = reinterpret_cast<char*>(dyn) + (8 * (line >> 1) + (line & 1)) * pitch;
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+    for (int r = 0; r < R; ++r) {
       const int q = q0 + r * TS;
       if (2 * q < p.Kp) {
 #pragma unroll
@@ -346,103 +335,101 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
           for (int s = 0; s < S; ++s)
 #pragma unroll
             for (int k = 0; k < SP_DIGITS; ++k)
-              dig[((s * SP_DIGITS + k) * NCOL + c * MM_LINES + line) * pitchw + q] = digit_pair(w[s][0], w[s][1], k);
+              *(uint32_t*)(dig + s * part1 + (k * NCOL + 2 * c) * pitch + 4 * q) = digit_pair(w[s][0], w[s][1], k);
         }
       }
     }
   }
   __syncthreads();
 
-  // (4) contraction and results
+  // (4) contraction and results: a warp takes 16 rows of two lines at a time
   const uint32_t dsh = (uint32_t)__cvta_generic_to_shared(dyn);
-  const int pitch = (p.Kp + 8) * 2;
   const int tab = FILT ? p.ftab : p.dtab;
   const int g = lane >> 2, t = lane & 3;
   // TR: results at the end points and at the continuation points, past the digits
-  double* endv = reinterpret_cast<double*>(dyn) + (size_t)S * SP_DIGITS * NCOL * pitch / sizeof(double);
+  double* endv = reinterpret_cast<double*>(reinterpret_cast<char*>(dyn) + S * part1);
   double* extv = endv + NCOL * 16;
-  for (int i0 = warp * 16; i0 < H; i0 += NW * 16) {
-    long long W[S][8];
-#pragma unroll 1
-    for (int s = 0; s < S; ++s) {
-      long long w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      // FP32 sums are exact over MM_KCHUNK columns: longer ones (512 threads) in two pieces
-#pragma unroll 1
-      for (int kb = 0; kb < (NT == 512 ? p.Kp : 1); kb += MM_KCHUNK)
-        mm_part(T.mmlo + tab + s * p.nx, T.mmhi + tab + s * p.nx, dsh + s * SP_DIGITS * NCOL * pitch, pitch, p, i0, kb,
-                NT == 512 && kb + MM_KCHUNK < p.Kp ? kb + MM_KCHUNK : p.Kp, lane, w);
-      if (s == 0) {
+  // joined sums y of rows i0 + g (+ 8) of lines l0, l0 + 1, component t: y[r * 2 + c]; the
+  // results are at index row + off
+  auto emit = [&](int i0, int l0, int off, const long long* y) {
+    const double fac[2] = {sh.fac[t * MM_LINES + l0], sh.fac[t * MM_LINES + l0 + 1]};
+    if constexpr (!PT) {
+      const int stride = sh.J[0].stride;
+      const long long base[2] = {sh.J[l0].base, sh.J[l0 + 1].base};
+      const bool have[2] = {sh.J[l0].n > 0, sh.J[l0 + 1].n > 0};
+      typename Ep::Op op[4];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) W[0][q] = w[q];
-      } else {
+      for (int q = 0; q < 4; ++q) {  // the operands of the four results in flight
+        const int i = i0 + g + 8 * (q >> 1), idx = i + off;
+        op[q] = ep.pre(t, base[q & 1] + (long long)(i < H && idx < n ? idx : 0) * stride);
+      }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) W[S - 1][q] = w[q];
+      for (int q = 0; q < 4; ++q) {
+        const int i = i0 + g + 8 * (q >> 1), idx = i + off;
+        if (i < H && idx < n && have[q & 1])
+          ep.put(t, base[q & 1] + (long long)idx * stride, op[q], sp_double(y[q]) * fac[q & 1]);
+      }
+    } else {
+      // the four lanes of a row hold its four components: a 4 x 4 transpose gives each lane
+      // one point, row g + 8 (t / 2) of line l0 + t % 2
+      const int i = i0 + g + 8 * (t >> 1), idx = i + off, ln = l0 + (t & 1);
+      const bool in = i < H && sh.J[ln].n > 0;
+      const typename Ep::Op op = ep.pre(point(sh, ln, i < H && idx < n ? idx : 0));
+      double z[4], x[4], v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) z[q] = sp_double(y[q]) * fac[q & 1];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {  // x[s]: component t ^ s of this lane's point
+        const int d = t ^ s;
+        const double snd = d & 2 ? (d & 1 ? z[3] : z[2]) : (d & 1 ? z[1] : z[0]);
+        x[s] = s ? __shfl_xor_sync(0xffffffffu, snd, s) : snd;
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int s = c ^ t;
+        v[c] = s & 2 ? (s & 1 ? x[3] : x[2]) : (s & 1 ? x[1] : x[0]);
+      }
+      if (TR && fcm >= 0 && in && (idx < d || idx >= n - d)) {  // completed after the fold
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int col = m * MM_LINES + ln;
+          if (idx >= n)
+            extv[col * C + idx - n] = v[m];
+          else
+            endv[col * 16 + (idx < d ? idx : d + idx - (n - d))] = v[m];
+        }
+      } else if (in && idx < n) {
+        ep.put(point(sh, ln, idx), op, v);
       }
     }
+  };
+  // joined sums of part s for 16 rows from i0 and the two lines from l0. FP32 sums are exact
+  // over MM_KCHUNK columns: longer ones (768 threads) in two pieces
+  auto part = [&](int s, int i0, int l0, long long* w) {
 #pragma unroll
-    for (int half = 0; half < S; ++half) {
-      if constexpr (!PT) {
-        // a thread's columns: lines 2 (t & 1) + c, components t / 2 and t / 2 + 2
-        const int stride = sh.J[0].stride, l0 = 2 * (t & 1), c0 = t >> 1;
-        const long long base[2] = {sh.J[l0].base, sh.J[l0 + 1].base};
-        const bool have[2] = {sh.J[l0].n > 0, sh.J[l0 + 1].n > 0};
+    for (int q = 0; q < 4; ++q) w[q] = 0;
+#pragma unroll 1
+    for (int kb = 0; kb < (NT == 768 ? p.Kp : 1); kb += MM_KCHUNK)
+      mm_part(T.mmlo + tab + s * p.nx, T.mmhi + tab + s * p.nx, p.Mp - i0, dsh + s * part1 + 4 * l0 * pitch, pitch, kb,
+              NT == 768 && kb + MM_KCHUNK < p.Kp ? kb + MM_KCHUNK : p.Kp, lane, w);
+  };
+  for (int u = warp; 16 * (u >> 1) < H; u += NW) {
+    const int i0 = 16 * (u >> 1), l0 = 2 * (u & 1);
+    long long y[4];
+    part(0, i0, l0, y);
+    if constexpr (S == 2) {
+      long long w[4];
+      part(1, i0, l0, w);
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {  // rows g and g + 8: operands of four results in flight
-          const int i = i0 + g + 8 * r, idx = i + half * H;
-          const bool in = i < H && idx < n;
-          const long long at = (long long)(in ? idx : 0) * stride;
-          typename Ep::Op op[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) op[q] = ep.pre(c0 + (q & 2), base[q & 1] + at);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const long long w0 = W[0][4 * r + q], w1 = W[S - 1][4 * r + q];
-            const long long y = S == 1 ? w0 : (half ? w0 - w1 : w0 + w1);
-            if (in && have[q & 1])
-              ep.put(c0 + (q & 2), base[q & 1] + at, op[q], sp_double(y) * sh.fac[(q >> 1) * 8 + 2 * t + (q & 1)]);
-          }
-        }
-      } else {
-        // lanes t and t ^ 2 hold components (0, 2) and (1, 3) of the same lines and rows:
-        // t < 2 keeps row g, t >= 2 row g + 8
-        double y[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int col = ((q >> 1) & 1) * 8 + 2 * t + (q & 1);
-          const long long w = S == 1 ? W[0][q] : (half ? W[0][q] - W[S - 1][q] : W[0][q] + W[S - 1][q]);
-          y[q] = sp_double(w) * sh.fac[col];
-        }
-        const bool up = t >= 2;
-        const int i = i0 + g + (up ? 8 : 0), idx = i + half * H;
-        typename Ep::Op op[2];
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-          op[c] = ep.pre(point(sh, 2 * (t & 1) + c, i < H && idx < n ? idx : 0));
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const double s0 = __shfl_xor_sync(0xffffffffu, up ? y[c] : y[4 + c], 2);
-          const double s1 = __shfl_xor_sync(0xffffffffu, up ? y[2 + c] : y[6 + c], 2);
-          double v[4];
-          v[0] = up ? s0 : y[c];
-          v[1] = up ? y[4 + c] : s0;
-          v[2] = up ? s1 : y[2 + c];
-          v[3] = up ? y[6 + c] : s1;
-          const int ln = 2 * (t & 1) + c;
-          const bool in = i < H && sh.J[ln].n > 0;
-          if (TR && fcm >= 0 && in && (idx < d || idx >= n - d)) {  // completed after the fold
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-              const int col = m * MM_LINES + ln;
-              if (idx >= n)
-                extv[col * C + idx - n] = v[m];
-              else
-                endv[col * 16 + (idx < d ? idx : d + idx - (n - d))] = v[m];
-            }
-          } else if (in && idx < n) {
-            ep.put(point(sh, ln, idx), op[c], v);
-          }
-        }
+      for (int q = 0; q < 4; ++q) {
+        const long long a = y[q];
+        y[q] = a + w[q];
+        w[q] = a - w[q];
       }
+      emit(i0, l0, 0, y);
+      emit(i0, l0, H, w);
+    } else {
+      emit(i0, l0, 0, y);
     }
   }
   if constexpr (TR) {
@@ -506,7 +493,13 @@ __device__ __forceinline__ bool tile_viscous(const DevTables& T, const MmShared&
   return visc;
 }
 
-#define MM_BOUNDS(NT) __launch_bounds__(NT, 512 / NT)
+// CTA configurations: NT threads (24 warps per SM resident, 80 registers a thread), S parts,
+// R pairs of columns per thread in the digits phase
+template <int NT_, int S_, int R_>
+struct MmCfg {
+  static constexpr int NT = NT_, S = S_, R = R_;
+};
+#define MM_BOUNDS __launch_bounds__(Cfg::NT, 768 / Cfg::NT)
 
 struct NoOp {};
 struct PutField {  // results into a field
@@ -515,6 +508,16 @@ struct PutField {  // results into a field
   long long cs;
   __device__ __forceinline__ NoOp pre(int, long long) const { return {}; }
   __device__ __forceinline__ void put(int c, long long q, NoOp, double v) const { f[q + c * cs] = v; }
+};
+struct PutField4 {
+  using Op = NoOp;
+  double* f;
+  long long cs;
+  __device__ __forceinline__ NoOp pre(long long) const { return {}; }
+  __device__ __forceinline__ void put(long long q, NoOp, const double* v) const {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) f[q + c * cs] = v[c];
+  }
 };
 struct LoadField {
   const double* f;
@@ -528,33 +531,41 @@ struct LoadField {
 
 }  // namespace
 
-// Threads per CTA: 128 hold the pairs of an inner length up to 128, 256 and 512 those of 256
-// and 512. A launch of at most one CTA per SM takes the next size up: nothing shares its SM,
-// and twice the warps shorten the tile's chain of loads, digits and row blocks (the results
-// do not depend on it).
+// Threads per CTA by padded inner length: 256 to 128 (three CTAs per SM), 384 to 256 (two),
+// 768 beyond. A launch of at most one CTA per SM takes more: nothing shares its SM, and more
+// warps shorten the tile's chain of loads, digits and row blocks (the results do not depend
+// on it).
 inline int mm_threads(int kp, int tiles) {
-  const int nt = kp <= 128 ? 128 : (kp <= 256 ? 256 : 512);
-  return tiles <= 152 && nt < 512 ? 2 * nt : nt;
+  if (tiles <= 152) return kp <= 64 ? 384 : 768;
+  return kp <= 128 ? 256 : (kp <= 256 ? 384 : 768);
+}
+// dynamic shared memory: the digits [S][SP_DIGITS][NCOL][Kp + 8] of FP16 (columns padded by
+// 16 bytes: conflict-free ldmatrix), over the continued lines [NCOL][pitch] they come from
+inline size_t mm_smem(int S, int Kp) {
+  const size_t dig = (size_t)S * SP_DIGITS * NCOL * (Kp + 8) * 2;
+  const size_t val = (size_t)NCOL * mm_line_pitch(S * Kp) * sizeof(double);
+  return dig > val ? dig : val;
 }
 // TAIL: the transposed operators' end and continuation results
 inline size_t mm_tail(int cmax) { return (size_t)NCOL * (16 + cmax) * sizeof(double); }
-#define MM_LAUNCH(KERNEL, TAIL, ...)                                       \
-  do {                                                                     \
-    if (t.n <= 0) return;                                                  \
-    const size_t sm = mm_smem(t.two ? 2 : 1, t.kp) + (TAIL);               \
-    const int nt = mm_threads(t.kp, t.n);                                  \
-    if (nt == 128 && t.two)                                                \
-      KERNEL<128, 2><<<t.n, nt, sm, st>>>(T, t.jobs, __VA_ARGS__);         \
-    else if (nt == 128)                                                    \
-      KERNEL<128, 1><<<t.n, nt, sm, st>>>(T, t.jobs, __VA_ARGS__);         \
-    else if (nt == 256 && t.two)                                           \
-      KERNEL<256, 2><<<t.n, nt, sm, st>>>(T, t.jobs, __VA_ARGS__);         \
-    else if (nt == 256)                                                    \
-      KERNEL<256, 1><<<t.n, nt, sm, st>>>(T, t.jobs, __VA_ARGS__);         \
-    else if (t.two)                                                        \
-      KERNEL<512, 2><<<t.n, nt, sm, st>>>(T, t.jobs, __VA_ARGS__);         \
-    else                                                                   \
-      KERNEL<512, 1><<<t.n, nt, sm, st>>>(T, t.jobs, __VA_ARGS__);         \
+#define MM_LAUNCH_CFG(KERNEL, NT, R, ...)                                                \
+  (t.two ? (void)(KERNEL<MmCfg<NT, 2, R>><<<t.n, NT, sm, st>>>(T, t.jobs, __VA_ARGS__))  \
+         : (void)(KERNEL<MmCfg<NT, 1, R>><<<t.n, NT, sm, st>>>(T, t.jobs, __VA_ARGS__)))
+#define MM_LAUNCH(KERNEL, TAIL, ...)                                 \
+  do {                                                               \
+    if (t.n <= 0) return;                                            \
+    const size_t sm = mm_smem(t.two ? 2 : 1, t.kp) + (TAIL);         \
+    const int nt = mm_threads(t.kp, t.n);                            \
+    if (nt == 256)                                                   \
+      MM_LAUNCH_CFG(KERNEL, 256, 1, __VA_ARGS__);                    \
+    else if (nt == 384 && t.kp <= 192)                               \
+      MM_LAUNCH_CFG(KERNEL, 384, 1, __VA_ARGS__);                    \
+    else if (nt == 384)                                              \
+      MM_LAUNCH_CFG(KERNEL, 384, 2, __VA_ARGS__);                    \
+    else if (t.kp <= 384)                                            \
+      MM_LAUNCH_CFG(KERNEL, 768, 1, __VA_ARGS__);                    \
+    else                                                             \
+      MM_LAUNCH_CFG(KERNEL, 768, 2, __VA_ARGS__);                    \
   } while (0)
 
 namespace {
@@ -563,8 +574,10 @@ void opt_in(K k) {
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(mm_smem(2, MM_KMAX) + mm_tail(MM_CMAX)));
 }
 }  // namespace
-#define MM_OPT_IN(KERNEL) \
-  opt_in(KERNEL<128, 1>), opt_in(KERNEL<128, 2>), opt_in(KERNEL<256, 1>), opt_in(KERNEL<256, 2>), \
-      opt_in(KERNEL<512, 1>), opt_in(KERNEL<512, 2>)
+#define MM_OPT_IN(KERNEL)                                                                                      \
+  opt_in(KERNEL<MmCfg<256, 1, 1>>), opt_in(KERNEL<MmCfg<256, 2, 1>>), opt_in(KERNEL<MmCfg<384, 1, 1>>),        \
+      opt_in(KERNEL<MmCfg<384, 2, 1>>), opt_in(KERNEL<MmCfg<384, 1, 2>>), opt_in(KERNEL<MmCfg<384, 2, 2>>),    \
+      opt_in(KERNEL<MmCfg<768, 1, 1>>), opt_in(KERNEL<MmCfg<768, 2, 1>>), opt_in(KERNEL<MmCfg<768, 1, 2>>),    \
+      opt_in(KERNEL<MmCfg<768, 2, 2>>)
 
 }  // namespace fcx

@@ -30,15 +30,15 @@ struct PutSlot {
   __device__ __forceinline__ NoOp pre(int, long long) const { return {}; }
   __device__ __forceinline__ void put(int c, long long q, NoOp, double v) const { G[(4 * s + c) * Pg + q] = v; }
 };
-template <int NT, int S>
-__global__ void MM_BOUNDS(NT) k_mm_gen_A(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ e,
+template <class Cfg>
+__global__ void MM_BOUNDS k_mm_gen_A(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ e,
                                          double* __restrict__ G) {
   extern __shared__ double2 dyn[];
   __shared__ MmShared sh;
   load_tile(sh, jobs);
   const MmPlan p = T.mm[sh.J[0].plan];
   const bool pf = T.patches[sh.J[0].patch].pform != 0;
-  mm_round<NT, S, false, false, false, false>(T, p, sh, dyn, LoadState{e, T.P, T.gamma, pf},
+  mm_round<Cfg, false, false, false, false>(T, p, sh, dyn, LoadState{e, T.P, T.gamma, pf},
                                               PutSlot{G + (sh.J[0].gbase - sh.J[0].base), T.Pg, 0});
 }
 
@@ -136,8 +136,8 @@ struct PutB {
     }
   }
 };
-template <int NT, int S>
-__global__ void MM_BOUNDS(NT) k_mm_gen_B(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ e,
+template <class Cfg>
+__global__ void MM_BOUNDS k_mm_gen_B(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ e,
                                          const double* __restrict__ mu, const double* __restrict__ Jm, double* G) {
   extern __shared__ double2 dyn[];
   __shared__ MmShared sh;
@@ -147,7 +147,7 @@ __global__ void MM_BOUNDS(NT) k_mm_gen_B(DevTables T, const Job* __restrict__ jo
   const long long off = sh.J[0].gbase - sh.J[0].base;
 #pragma unroll 1
   for (int rd = 0; rd < 3; ++rd)
-    mm_round<NT, S, true, false, true, false>(T, p, sh, dyn, LoadB{e, G + off, T.P, T.Pg, T.gamma, rd, pf},
+    mm_round<Cfg, true, false, true, false>(T, p, sh, dyn, LoadB{e, G + off, T.P, T.Pg, T.gamma, rd, pf},
                                               PutB{e, mu, Jm + off, G + off, T.P, T.Pg, T.gamma, rd, pf});
 }
 
@@ -199,8 +199,8 @@ struct PutC {
       stage_put(sc, dt, q + c * cs, (o.info & PT_NODIFF) ? 0.0 : -(fma(o.j, v, o.r1) + o.r2), o.cur, o.u0, o.aux);
   }
 };
-template <int NT, int S>
-__global__ void MM_BOUNDS(NT) k_mm_gen_C(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ Jm,
+template <class Cfg>
+__global__ void MM_BOUNDS k_mm_gen_C(DevTables T, const Job* __restrict__ jobs, const double* __restrict__ Jm,
                                          double* G, StageCoef sc) {
   extern __shared__ double2 dyn[];
   __shared__ MmShared sh;
@@ -210,7 +210,7 @@ __global__ void MM_BOUNDS(NT) k_mm_gen_C(DevTables T, const Job* __restrict__ jo
   const double dt = sc.rhs_only ? 0.0 : *sc.dt;
 #pragma unroll 1
   for (int rd = 0; rd < 2; ++rd)
-    mm_round<NT, S, false, false, false, false>(T, p, sh, dyn, LoadC{G + off, T.Pg, rd},
+    mm_round<Cfg, false, false, false, false>(T, p, sh, dyn, LoadC{G + off, T.Pg, rd},
                                                 PutC{Jm + off, G + off, T.info, sc, dt, T.P, T.Pg, rd});
 }
 

@@ -19,6 +19,7 @@
 
 #include "fc_internal.h"
 #include "fc_split.cuh"
+#include "fc_tables.h"
 
 namespace fcx {
 
@@ -90,13 +91,9 @@ inline MmPlan mm_plan(int L, const std::vector<long double>* sig, std::vector<ui
   p.Kp = (p.H + 15) / 16 * 16;
   p.Mp = p.Kp;
   p.nx = p.Mp + p.Kp;
-  // cos(pi j / (2L)), which also gives sin(pi m / L) = cos(pi (L - 2m) / (2L))
-  std::vector<long double> cs((size_t)2 * L + 1);
-  for (int j = 0; j <= L; ++j) {
-    cs[j] = cosl(PI_L * j / (2.0L * L));
-    cs[2 * L - j] = -cs[j];
-  }
-  cs[L] = 0.0L;
+  // cos(pi j / (2L)), j = 0..2L, which also gives sin(pi m / L) = cos(pi (L - 2m) / (2L))
+  const Trig tg(4 * L);
+  const std::vector<long double>& cs = tg.c;
   std::vector<long double> c((size_t)L, 0.0L);
   for (int m = 1; 2 * m <= L; ++m) {
     const long double sn = cs[L - 2 * m];  // sin(pi m / L)
