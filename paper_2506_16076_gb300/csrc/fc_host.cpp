@@ -113,6 +113,8 @@ struct fc_ctx {
   MmPlan* d_mm = nullptr;
   uint4* d_mmlo = nullptr;
   uint2* d_mmhi = nullptr;
+  MmCont* d_mmc = nullptr;
+  uint4* d_mmcf = nullptr;
   Plan* d_plans = nullptr;
   double2* d_tw = nullptr;
   double* d_rp = nullptr;
@@ -872,6 +874,8 @@ struct Builder {
   std::vector<MmPlan> mm;  // per plan: its tensor-core contraction (H = 0: none)
   std::vector<uint4> mmlo;
   std::vector<uint2> mmhi;
+  std::vector<uint4> mmcf;
+  std::vector<MmCont> mmc = std::vector<MmCont>(MM_CMAX + 1, MmCont{-1, {0}});  // per C
   std::vector<std::vector<Plan>> cands;  // per plan: stage orders for the autotuner, [0] = plans[i]
 
   // slot -> mode table of an in-place transform with p's stage order, appended to the int pool:
@@ -967,6 +971,13 @@ struct Builder {
         }
       for (long double v : M[which]) rp.push_back((double)v);
     }
+    // the same columns for the contraction kernels, in the order of their detrended end values
+    std::vector<long double> X((size_t)C * 2 * d, 0.0L);
+    for (int k = 0; k < C; ++k)
+      for (int j = 0; j < d - 2; ++j) {
+        X[(size_t)k * 2 * d + j] = M[0][(size_t)k * d + j + 2];
+        X[(size_t)k * 2 * d + d - 2 + j] = M[1][(size_t)k * d + j];
+      }
     for (int which = 0; which < 2; ++which)
       for (int pass = 0; pass < 2; ++pass)
         for (int k = 0; k < C; ++k) {
@@ -976,7 +987,9 @@ struct Builder {
             s += M[which][(size_t)k * d + i] * (pass == 0 ? 1.0L : tau);
           }
           rp.push_back((double)s);
+          X[(size_t)k * 2 * d + 2 * d - 4 + 2 * which + pass] = s;
         }
+    if (C <= MM_CMAX && d <= 8) mmc[C] = mm_continuation(C, 2 * d, X, mmcf);
     fcm_of_C[C] = off;
     return off;
   }
@@ -1698,7 +1711,7 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   std::vector<Recv> rinterp;
   std::vector<PtCopy> rcopy;
   split_exchange(recv, rinterp, rcopy);
-  ok = ok && c->upload(&c->d_mm, B.mm) && c->upload(&c->d_mmlo, B.mmlo) && c->upload(&c->d_mmhi, B.mmhi) &&
+  ok = ok && c->upload(&c->d_mm, B.mm) && c->upload(&c->d_mmlo, B.mmlo) && c->upload(&c->d_mmhi, B.mmhi) && c->upload(&c->d_mmc, B.mmc) && c->upload(&c->d_mmcf, B.mmcf) &&
        c->upload(&c->d_plans, B.plans) && c->upload(&c->d_tw, B.tw) && c->upload(&c->d_rp, B.rp) &&
        c->upload(&c->d_ip, B.ip) &&
        c->upload(&c->d_info, info) && c->upload(&c->d_patches, pdev) && c->upload(&c->d_J, Jm) &&
@@ -1763,6 +1776,8 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   T.mm = c->d_mm;
   T.mmlo = c->d_mmlo;
   T.mmhi = c->d_mmhi;
+  T.mmc = c->d_mmc;
+  T.mmcf = c->d_mmcf;
   T.info = c->d_info;
   T.patches = c->d_patches;
   T.npatch = npatch;

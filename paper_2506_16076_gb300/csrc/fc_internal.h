@@ -59,6 +59,13 @@ struct MmPlan {
   int dte, fte;    // their coefficients are scaled by 2^dte, 2^fte
 };
 
+// Continuation matrix of C points for the matrix instruction (fc_mmtab.h): coefficient column
+// q of the detrended end values is scaled by 2^-sq[q]
+struct MmCont {
+  int first;   // first uint4 of its fragments [C / 16][digit][lane] (-1: none)
+  int sq[16];
+};
+
 // One line segment processed by one warp.
 struct Job {
   long long base;   // flat index of the first point
@@ -144,6 +151,8 @@ struct DevTables {
   const MmPlan* mm;         // per plan
   const uint4* mmlo;        // digits 0..3 and 4..5 of the contraction tables
   const uint2* mmhi;
+  const MmCont* mmc;        // per continuation length C <= MM_CMAX
+  const uint4* mmcf;        // their fragments
   const uint32_t* info;     // per-point flags
   const PatchDev* patches;
   int npatch;

@@ -40,12 +40,18 @@ namespace {
 
 constexpr int NCOL = 4 * MM_LINES;  // columns of a tile: component * MM_LINES + line
 
+constexpr int CONT_PITCH = 24;  // FP16 per column of the end values' digits: 16 and a conflict-free pad
+
 // static shared state of a tile
 struct MmShared {
   Job J[MM_LINES];
   uint32_t emax[NCOL];  // high words of the largest magnitudes
   double fac[NCOL];     // value of one unit of a joined sum
+  int fexp[NCOL];       // without the lines' scale: 2^fexp
   double tmp[NCOL * 16];  // detrended end values of the columns, 2d <= 16 each
+  int cexp[NCOL];         // largest exponent of a column's weighted end values
+  int sq[16];             // their weights (MmCont)
+  __align__(16) uint16_t cdig[SP_DIGITS * NCOL * CONT_PITCH];  // their digits (FP16)
 };
 
 constexpr int LB = 4;  // points of a thread whose loads are in flight together
@@ -156,28 +162,51 @@ __device__ __forceinline__ long long point(const MmShared& sh, int line, int t) 
   return sh.J[line].base + (long long)t * sh.J[line].stride;
 }
 
-// continuation values of the tile's columns from their detrended end values (eq.
-// continuation, as continue_lines), D = d when it is known at compile time
-template <int NT, int D>
-__device__ __forceinline__ void continuation(const double* __restrict__ M, int C, int dd, const double* tmp,
-                                             double* ext, int LP, uint32_t* emax) {
-  const int d = D ? D : dd;
-  const double* ML = M;
-  const double* MR = M + C * d;
-  const double* u = MR + C * d;  // uL, vL, uR, vR
-  for (int it = threadIdx.x; it < NCOL * C; it += NT) {
-    const int col = it & (NCOL - 1), k = it / NCOL;
-    const double* e = tmp + col * 16;
-    double x = 0.0;
+// Continuation values of the tile's columns from their detrended end values (eq.
+// continuation, as continue_lines): 2d FP64 operations per value, a quarter of a pass's FP64
+// work, are one 16-column step of digit products instead (mm_continuation in fc_mmtab.h). A
+// column's end values are scaled by the largest of their weighted magnitudes, not by the
+// line's, so small second differences keep their bits.
+template <int NT>
+__device__ __forceinline__ void continuation(const uint4* __restrict__ frag, int C, MmShared& sh, double* ext, int LP) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  constexpr uint32_t pitch = CONT_PITCH * 2, slice = NCOL * pitch;
+  for (int u = warp; 16 * (u >> 1) < C; u += NT / 32) {
+    const int mb = u >> 1, n0 = 8 * (u & 1);
+    const uint4* f = frag + (size_t)mb * SP_DIGITS * 32 + lane;
+    uint4 A[SP_DIGITS];
 #pragma unroll
-    for (int j = 2; j < d; ++j) x = fma(__ldg(ML + k * d + j), e[j - 2], x);
+    for (int j = 0; j < SP_DIGITS; ++j) A[j] = ldg_keep(f + 32 * j);
+    float acc[SP_DIGITS][4];
 #pragma unroll
-    for (int j = 0; j < d - 2; ++j) x = fma(__ldg(MR + k * d + j), e[d - 2 + j], x);
-    x = fma(e[2 * d - 4], __ldg(u + k),
-            fma(e[2 * d - 3], __ldg(u + C + k),
-                fma(e[2 * d - 2], __ldg(u + 2 * C + k), fma(e[2 * d - 1], __ldg(u + 3 * C + k), x))));
-    ext[col * LP + k] = x;
-    atomicMax(&emax[col], sp_hi(x) & 0x7fffffffu);
+    for (int l = 0; l < SP_DIGITS; ++l)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[l][q] = 0.f;
+    const uint32_t addr = (uint32_t)__cvta_generic_to_shared(sh.cdig) +
+                          (uint32_t)((n0 + (lane & 7)) * pitch + ((lane >> 3) & 1) * 16) + (lane >> 4) * slice;
+#pragma unroll
+    for (int j2 = 0; j2 < SP_DIGITS; j2 += 2) {
+      uint32_t b[4];
+      ldsm4(b, addr + j2 * slice);
+#pragma unroll
+      for (int i = 0; i + j2 < SP_DIGITS; ++i) {
+        mma16816(acc[i + j2], A[i].x, A[i].y, A[i].z, A[i].w, b[0], b[1]);
+        if (i + j2 + 1 < SP_DIGITS) mma16816(acc[i + j2 + 1], A[i].x, A[i].y, A[i].z, A[i].w, b[2], b[3]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = 16 * mb + g + 8 * (q >> 1), col = n0 + 2 * t + (q & 1);
+      int s[SP_DIGITS];
+#pragma unroll
+      for (int l = 0; l < SP_DIGITS; ++l) s[l] = __float2int_rn(acc[l][q]);
+      const int e = sh.cexp[col] - 1023 - SP_DATA + SP_UNIT - SP_COEF;
+      if (k < C) {
+        const double x = sp_double_exp(sp_join(s), e, scalbn(1.0, e));
+        ext[col * LP + k] = x;
+        atomicMax(&sh.emax[col], sp_hi(x) & 0x7fffffffu);
+      }
+    }
   }
 }
 
@@ -202,7 +231,11 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
   const int n = sh.J[0].n, C = sh.J[0].C, fcm = sh.J[0].fcm, d = T.d, H = p.H;
   const int LP = mm_line_pitch(S * H);
   double* F = reinterpret_cast<double*>(dyn);  // [NCOL][LP]: the continued lines
-  if (tid < NCOL) sh.emax[tid] = 0;
+  if (tid < NCOL) {
+    sh.emax[tid] = 0;
+    sh.cexp[tid] = 0;
+    if (!TR && fcm >= 0) sh.sq[tid] = T.mmc[C].sq[tid];
+  }
   __syncthreads();
 
   // (1) the lines' values into shared memory, and their maxima. q1 lines: a warp per line
@@ -270,12 +303,20 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
         v = w == 0 ? f0 : (w == 1 ? dl : (w == 2 ? fn : dr));
       }
       sh.tmp[col * 16 + q] = v;
+      const int e = (int)((sp_hi(v) >> 20) & 0x7ffu);
+      if (e > 0) atomicMax(&sh.cexp[col], e + sh.sq[q]);
+      if (e == 0x7ff) atomicMax(&sh.emax[col], 0x7ff00000u);
     }
     __syncthreads();
-    if (d == 5)
-      continuation<NT, 5>(T.rp + fcm, C, 5, sh.tmp, F + n, LP, sh.emax);
-    else
-      continuation<NT, 0>(T.rp + fcm, C, d, sh.tmp, F + n, LP, sh.emax);
+    for (int it = tid; it < NCOL * 16; it += NT) {
+      const int col = it & (NCOL - 1), q = it / NCOL;
+      const long long x = q < 2 * d ? sp_fixed(sh.tmp[col * 16 + q], sh.cexp[col] - sh.sq[q]) : 0;
+#pragma unroll
+      for (int k = 0; k < SP_DIGITS; ++k)
+        sh.cdig[(k * NCOL + col) * CONT_PITCH + q] = (uint16_t)digit_pair(x + SP_BIAS, 0, k);
+    }
+    __syncthreads();
+    continuation<NT>(T.mmcf + T.mmc[C].first, C, sh, F + n, LP);
     __syncthreads();
   }
   const int te = FILT ? p.fte : p.dte;
@@ -283,9 +324,10 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
     const uint32_t h = sh.emax[tid], h2 = sh.emax[tid ^ MM_LINES];
     const double sc = FILT ? 1.0 : (TR ? -1.0 : 1.0) * sh.J[tid & (MM_LINES - 1)].scale;
     // a non-finite value spoils its line, and its packed partner's, as in the FFT kernels
-    sh.fac[tid] = (h >= 0x7ff00000u || h2 >= 0x7ff00000u)
-                      ? __longlong_as_double(0x7ff8000000000000ll)
-                      : scalbn(sc, (int)(h >> 20) - 1023 - SP_DATA + SP_UNIT - te - (S - 1));
+    const int e = (int)(h >> 20) - 1023 - SP_DATA + SP_UNIT - te - (S - 1);
+    const bool bad = h >= 0x7ff00000u || h2 >= 0x7ff00000u;
+    sh.fac[tid] = bad ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(sc, e);
+    sh.fexp[tid] = bad ? 1 << 20 : e;  // the filter's factor is a power of two
   }
 
   // (3) digits of the parts, over the values: all reads come before the first write. A warp
@@ -353,6 +395,9 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
   // results are at index row + off
   auto emit = [&](int i0, int l0, int off, const long long* y) {
     const double fac[2] = {sh.fac[t * MM_LINES + l0], sh.fac[t * MM_LINES + l0 + 1]};
+    auto value = [&](long long w, int c) {
+      return FILT ? sp_double_exp(w, sh.fexp[t * MM_LINES + l0 + c], fac[c]) : sp_double(w) * fac[c];
+    };
     if constexpr (!PT) {
       const int stride = sh.J[0].stride;
       const long long base[2] = {sh.J[l0].base, sh.J[l0 + 1].base};
@@ -367,7 +412,7 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
       for (int q = 0; q < 4; ++q) {
         const int i = i0 + g + 8 * (q >> 1), idx = i + off;
         if (i < H && idx < n && have[q & 1])
-          ep.put(t, base[q & 1] + (long long)idx * stride, op[q], sp_double(y[q]) * fac[q & 1]);
+          ep.put(t, base[q & 1] + (long long)idx * stride, op[q], value(y[q], q & 1));
       }
     } else {
       // the four lanes of a row hold its four components: a 4 x 4 transpose gives each lane
@@ -377,7 +422,7 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
       const typename Ep::Op op = ep.pre(point(sh, ln, i < H && idx < n ? idx : 0));
       double z[4], x[4], v[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) z[q] = sp_double(y[q]) * fac[q & 1];
+      for (int q = 0; q < 4; ++q) z[q] = value(y[q], q & 1);
 #pragma unroll
       for (int s = 0; s < 4; ++s) {  // x[s]: component t ^ s of this lane's point
         const int d = t ^ s;

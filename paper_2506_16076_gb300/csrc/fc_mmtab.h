@@ -127,4 +127,39 @@ inline MmPlan mm_plan(int L, const std::vector<long double>* sig, std::vector<ui
   return p;
 }
 
+// The continuation's contraction: ext_k = sum_q M[k][q] e_q over the Q <= 16 detrended end
+// values of a line, as digit products of one 16-column step. The columns' coefficients differ
+// by four orders of magnitude (second differences 1e4, values 1), so column q carries 2^-sq
+// and its value 2^sq. Fragments of the matrix instruction, 16 rows (continuation points) each:
+// [block][digit][lane], a lane's four registers side by side.
+inline MmCont mm_continuation(int C, int Q, const std::vector<long double>& M, std::vector<uint4>& lo) {
+  MmCont r{};
+  r.first = (int)lo.size();
+  for (int q = 0; q < Q; ++q) {
+    long double top = 0;
+    for (int k = 0; k < C; ++k) top = std::max(top, std::fabs(M[(size_t)k * Q + q]));
+    int e = 0;
+    if (top > 0) std::frexp(top, &e);
+    r.sq[q] = e;
+  }
+  auto digit = [&](int k, int q, int j) -> uint32_t {
+    if (k >= C || q >= Q) return 0;
+    int d[SP_DIGITS];
+    mm_digits((long long)std::llround(std::ldexp(M[(size_t)k * Q + q], SP_COEF - r.sq[q])), d);
+    return mm_half(d[j]);
+  };
+  for (int b = 0; b < (C + 15) / 16; ++b)
+    for (int j = 0; j < SP_DIGITS; ++j)
+      for (int lane = 0; lane < 32; ++lane) {
+        const int g = lane >> 2, t = lane & 3;
+        uint32_t a[4];
+        for (int i = 0; i < 4; ++i) {
+          const int k = 16 * b + g + 8 * (i & 1), q = 2 * t + 8 * (i >> 1);
+          a[i] = digit(k, q, j) | (digit(k, q + 1, j) << 16);
+        }
+        lo.push_back(uint4{a[0], a[1], a[2], a[3]});
+      }
+  return r;
+}
+
 }  // namespace fcx

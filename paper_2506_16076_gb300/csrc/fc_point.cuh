@@ -69,10 +69,18 @@ __device__ __forceinline__ void conv_div_product(const double* e, double th, con
   out[3] = fma(e[3] + p, ux + vy, fma(u, ex[3] + px, v * (ey[3] + py)));
 }
 
+// a / b from ib = 1 / b: the quotient estimate and one correction with its exact remainder
+// (Markstein's scheme: a correctly rounded ib gives a correctly rounded quotient up to rare
+// cases within an ulp), three FP64 operations where a division takes about six
+__device__ __forceinline__ double div_by(double a, double b, double ib) {
+  const double q = a * ib;
+  return fma(fma(-q, b, a), ib, q);
+}
 // theta = p / rho (eq. p_T)
 __device__ __forceinline__ double theta_of(double r, double mx, double my, double E, double gam) {
-  const Prim q = primitives(r, mx, my, E, gam);
-  return q.p / r;
+  const double ir = 1.0 / r;
+  const double p = (gam - 1.0) * (E - 0.5 * (mx * (mx * ir) + my * (my * ir)));
+  return div_by(p, r, ir);
 }
 
 // Runge-Kutta stage combination of one component (q: flat index of the component's point)
@@ -103,7 +111,8 @@ __device__ __forceinline__ void stage_write(const StageCoef& sc, long long p, lo
 }
 
 __device__ __forceinline__ double energy_of(double r, double mx, double my, double th, double gam) {
-  return r * th / (gam - 1.0) + 0.5 * (mx * mx + my * my) / r;
+  const double g1 = gam - 1.0;
+  return div_by(r * th, g1, 1.0 / g1) + div_by(0.5 * (mx * mx + my * my), r, 1.0 / r);
 }
 
 // A^T eta for the x (dir 0) or y (dir 1) flux Jacobian at state e (eq. euler 2d equation)

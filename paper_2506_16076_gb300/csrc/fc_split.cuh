@@ -92,6 +92,30 @@ FC_HD double sp_double(long long v) {
 #endif
 }
 
+// v 2^e as a double, without the FP64 pipe while the result is a normal number; else by the
+// multiplication with fac = 2^e (NaN for a non-finite line, with e out of every range)
+FC_HD double sp_double_exp(long long v, int e, double fac) {
+  const uint64_t a = v < 0 ? (uint64_t)(-v) : (uint64_t)v;
+#ifdef __CUDA_ARCH__
+  const int lz = __clzll((long long)a);
+#else
+  const int lz = a ? __builtin_clzll(a) : 64;
+#endif
+  const int x = 1085 - lz + e;  // biased exponent - 1
+  if ((unsigned)(x - 1) >= 2040u) return sp_double(v) * fac;
+  const uint64_t m = a << (lz & 63);
+  uint64_t b = ((uint64_t)x << 52) + (m >> 11) + ((m >> 10) & 1u);
+  b = a ? b : 0;
+  b |= (uint64_t)v & 0x8000000000000000ull;
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)b);
+#else
+  double r;
+  memcpy(&r, &b, 8);
+  return r;
+#endif
+}
+
 // The FP64 quotient df / rg rounded to FP32 (0 <= df <= rg, both finite, r = 1 / rg rounded):
 // t = df r is within 2.5 ulp of the rounded quotient and rounds to the same FP32 number
 // unless its low 29 bits lie that close to the midpoint of two FP32 numbers, where the

@@ -7,6 +7,11 @@
 //     "L op kind error/max|x| largest_level_sum" (op 0: derivative, 1: filter), or "L none"
 //     when lines of this length are left to the FFT kernels.
 //
+//   contraction_host continuation C Q
+//     the continuation's digit products (mm_continuation, fragments read back as the matrix
+//     instruction does) for a matrix whose columns differ in size, on end values that differ,
+//     against long double; prints the error over the largest |coefficient x value|.
+//
 //   contraction_host quotient
 //     quotient_f32 against the FP64 division rounded to FP32, on random quotients and on
 //     quotients placed around the rounding midpoints; prints "tested different".
@@ -55,7 +60,55 @@ static int quotients() {
   return 0;
 }
 
+static int continuation(int C, int Q) {
+  std::mt19937_64 g(3);
+  std::uniform_real_distribution<double> U(-1.0, 1.0);
+  std::vector<long double> M((size_t)C * Q);
+  std::vector<uint4> lo(5);  // (a table does not start at 0)
+  for (int k = 0; k < C; ++k)
+    for (int q = 0; q < Q; ++q) M[(size_t)k * Q + q] = std::ldexp((long double)U(g), (int)(14.0 * q / Q));
+  const MmCont r = mm_continuation(C, Q, M, lo);
+  double worst = 0;
+  for (int trial = 0; trial < 200; ++trial) {
+    std::vector<double> e(Q);
+    int ce = 0;
+    for (int q = 0; q < Q; ++q) {
+      e[q] = trial == 0 ? 0.0 : std::ldexp(U(g), -(int)(30 * (U(g) + 1.0)) * (trial % 3) - 14 * q / Q);
+      const int x = (int)((sp_hi(e[q]) >> 20) & 0x7ffu);
+      if (x > 0) ce = std::max(ce, x + r.sq[q]);
+    }
+    std::vector<long long> f(16, SP_BIAS);
+    for (int q = 0; q < Q; ++q) f[q] += sp_fixed(e[q], ce - r.sq[q]);
+    for (int k = 0; k < C; ++k) {
+      double lev[SP_DIGITS] = {0};
+      for (int q = 0; q < 16; ++q) {
+        const int i = ((k & 15) >> 3) + 2 * (q >> 3), lane = (k & 7) * 4 + (q & 7) / 2;
+        for (int u = 0; u < SP_DIGITS; ++u) {
+          const uint4 a = lo[(size_t)r.first + ((k / 16) * SP_DIGITS + u) * 32 + lane];
+          const unsigned w = i == 0 ? a.x : i == 1 ? a.y : i == 2 ? a.z : a.w;
+          for (int v = 0; u + v < SP_DIGITS; ++v)
+            lev[u + v] += half_value(q & 1 ? w >> 16 : w & 0xffff) * ((int)sp_field(f[q], v) - 512);
+        }
+      }
+      int si[SP_DIGITS];
+      for (int l = 0; l < SP_DIGITS; ++l) si[l] = (int)lev[l];
+      const int x = ce - 1023 - SP_DATA + SP_UNIT - SP_COEF;
+      const double got = sp_double_exp(sp_join(si), x, std::scalbn(1.0, x));
+      long double ref = 0, top = 0;
+      for (int q = 0; q < Q; ++q) {
+        ref += M[(size_t)k * Q + q] * e[q];
+        top = std::max(top, std::ldexp(std::fabs((long double)e[q]), r.sq[q]));
+      }
+      if (top > 0) worst = std::max(worst, (double)(std::fabs(got - ref) / top));
+      if (trial == 0 && got != 0.0) worst = 1.0;
+    }
+  }
+  printf("%.3e\n", worst);
+  return 0;
+}
+
 int main(int argc, char** argv) {
+  if (argc == 4 && !std::strcmp(argv[1], "continuation")) return continuation(std::atoi(argv[2]), std::atoi(argv[3]));
   if (argc == 2 && !std::strcmp(argv[1], "quotient")) return quotients();
   std::mt19937_64 g(1);
   std::uniform_real_distribution<double> U(-1.0, 1.0);

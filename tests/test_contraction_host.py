@@ -55,3 +55,12 @@ def test_quotients_round_as_the_division(exe):
     r = subprocess.run([exe, "quotient"], capture_output=True, text=True, timeout=600)
     n, bad = map(int, r.stdout.split())
     assert r.returncode == 0 and n > 10 ** 7 and bad == 0, (n, bad)
+
+
+@pytest.mark.parametrize("C,Q", [(27, 10), (32, 10), (71, 10), (33, 4), (128, 16)])
+def test_continuation_products(exe, C, Q):
+    # relative to the largest weighted end value: at most 16 values of 57 bits truncated (2^-57 each,
+    # coefficients below 1), five levels of dropped products (2^-54.8 at eight deviations of 80 pairs):
+    # below 2^-52.5 in all; and one FP64 rounding of a sum of up to Q such values, Q 2^-53
+    r = subprocess.run([exe, "continuation", str(C), str(Q)], capture_output=True, text=True)
+    assert r.returncode == 0 and float(r.stdout) < 2.0 ** -52.5 + Q * 2.0 ** -53, r.stdout
