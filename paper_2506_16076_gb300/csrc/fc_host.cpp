@@ -1138,6 +1138,26 @@ void make_queue(fc_ctx* c, fc_ctx::Queue& q, std::vector<Job>& jobs, const std::
   if (mm) make_tiles(c, q, pp, plans, npatch, ok, *mm);
 }
 
+// launch configurations of a queue's tiles, batched and per patch
+unsigned mm_configs(const fc_ctx::Queue& q) {
+  unsigned m = 0;
+  for (const MmTiles& t : q.mm) m |= 1u << mm_config(t);
+  for (const auto& v : q.mmpp)
+    for (const MmTiles& t : v) m |= 1u << mm_config(t);
+  return m;
+}
+// shared-memory limits of the contraction kernels in the configurations this context launches
+// (a call costs a microsecond and more; the adjoint's kernels wait for its first step)
+void contraction_attributes(const fc_ctx* c) {
+  set_mm_attributes(mm_configs(c->q_cart1) | mm_configs(c->q_cart2) | mm_configs(c->q_filt1) | mm_configs(c->q_filt2));
+  set_mm_gen_attributes(mm_configs(c->q_gen1) | mm_configs(c->q_gen2));
+  if (c->adj_ready) {
+    set_mm_adj_attributes(mm_configs(c->q_cart1) | mm_configs(c->q_cart2) | mm_configs(c->q_filt1) |
+                          mm_configs(c->q_filt2));
+    set_mm_adj_gen_attributes(mm_configs(c->q_gen1) | mm_configs(c->q_gen2));
+  }
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------- API
@@ -1787,10 +1807,7 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
   T.d = prm->d;
   T.any_pform = any_pform ? 1 : 0;
   set_kernel_attributes();
-  set_mm_attributes();
-  set_mm_gen_attributes();
-  set_mm_adj_attributes();
-  set_mm_adj_gen_attributes();
+  contraction_attributes(c);
   if (!mpts.empty()) {  // metrics of GRID patches given by their points only
     std::vector<double> xy(2 * (size_t)c->P, 0.0);
     for (const HPatch& h : c->hp)
@@ -2683,6 +2700,7 @@ fc_status fc_adjoint_step(fc_ctx* c, const double* e_n, const double* mu, const 
          c->alloc(&c->d_A3, n4) && c->alloc(&c->d_PSa, n4) && c->alloc(&c->d_PSb, n4);
     if (!ok) return FC_ERR_OOM;
     c->adj_ready = true;
+    contraction_attributes(c);
   }
   const bool filt = (flags & FC_STEP_FILTER) != 0;
   const size_t bytes4 = sizeof(double) * 4 * (size_t)c->P;
@@ -2891,6 +2909,7 @@ fc_status fc_shard(fc_ctx* c, int nranks, int rank, const int* owner, fc_comm_fn
       if (own[J.patch] == rank) jobs.push_back(J);
     make_queue(c, *q, jobs, c->plans_h, npatch, ok, q->rest ? &c->mm_h : nullptr);
   }
+  if (ok) contraction_attributes(c);
   // point lists of the owned patches
   std::vector<BcPt> bc;
   for (const BcPt& b : c->h_bc)

@@ -194,6 +194,19 @@ struct MmTiles {
   // kernel looks for itself)
   uint8_t* visc;
 };
+// Threads per CTA by padded inner length: 256 to 128 (three CTAs per SM), 384 to 256 (two),
+// 768 beyond. A launch of at most one CTA per SM takes more: nothing shares its SM, and more
+// warps shorten the tile's chain of loads, digits and row blocks (the results do not depend
+// on it).
+inline int mm_threads(int kp, int tiles) {
+  if (tiles <= 152) return kp <= 64 ? 384 : 768;
+  return kp <= 128 ? 256 : (kp <= 256 ? 384 : 768);
+}
+// the kernel configuration of a launch: threads (256, 384, 768), pairs per thread (1, 2), parity
+inline int mm_config(const MmTiles& t) {
+  const int nt = mm_threads(t.kp, t.n);
+  return (nt == 256 ? 0 : nt == 384 ? (t.kp <= 192 ? 1 : 2) : (t.kp <= 384 ? 3 : 4)) * 2 + t.two;
+}
 // flags of n tiles (jobs: MM_LINES per tile)
 void launch_tile_flags(const Job* jobs, int n, const double* mu, uint8_t* visc, cudaStream_t st);
 void launch_mm_cart_q1(const DevTables& T, const MmTiles& t, const double* e, const double* mu, double* R1, double* Fy,
@@ -220,10 +233,11 @@ void launch_mm_filterT_q2(const DevTables& T, const MmTiles& t, const double* la
                           cudaStream_t st);
 void launch_mm_filterT_q1(const DevTables& T, const MmTiles& t, const double* MF, const double* e, double* out,
                           cudaStream_t st);
-void set_mm_attributes();
-void set_mm_gen_attributes();
-void set_mm_adj_attributes();
-void set_mm_adj_gen_attributes();
+// shared-memory limits of the kernels in the configurations of a bit mask (1 << mm_config)
+void set_mm_attributes(unsigned configs);
+void set_mm_gen_attributes(unsigned configs);
+void set_mm_adj_attributes(unsigned configs);
+void set_mm_adj_gen_attributes(unsigned configs);
 
 // ---- launch wrappers (fc_kernels.cu) ----
 // Fy (nullable): the y fluxes of the affine points, written by the q1 pass (and by

@@ -189,7 +189,7 @@ void launch_mm_filter_q2(const DevTables& T, const MmTiles& t, const double* F, 
   MM_LAUNCH(k_mm_filter_q2, 0, F, e);
 }
 
-void set_mm_attributes() {
+void set_mm_attributes(unsigned configs) {
   MM_OPT_IN(k_mm_cart_q1);
   MM_OPT_IN(k_mm_cart_q2);
   MM_OPT_IN(k_mm_filter_q1);

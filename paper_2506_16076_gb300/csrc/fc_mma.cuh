@@ -576,14 +576,6 @@ struct LoadField {
 
 }  // namespace
 
-// Threads per CTA by padded inner length: 256 to 128 (three CTAs per SM), 384 to 256 (two),
-// 768 beyond. A launch of at most one CTA per SM takes more: nothing shares its SM, and more
-// warps shorten the tile's chain of loads, digits and row blocks (the results do not depend
-// on it).
-inline int mm_threads(int kp, int tiles) {
-  if (tiles <= 152) return kp <= 64 ? 384 : 768;
-  return kp <= 128 ? 256 : (kp <= 256 ? 384 : 768);
-}
 // dynamic shared memory: the digits [S][SP_DIGITS][NCOL][Kp + 8] of FP16 (columns padded by
 // 16 bytes: conflict-free ldmatrix), over the continued lines [NCOL][pitch] they come from
 inline size_t mm_smem(int S, int Kp) {
@@ -593,36 +585,40 @@ inline size_t mm_smem(int S, int Kp) {
 }
 // TAIL: the transposed operators' end and continuation results
 inline size_t mm_tail(int cmax) { return (size_t)NCOL * (16 + cmax) * sizeof(double); }
-#define MM_LAUNCH_CFG(KERNEL, NT, R, ...)                                                \
-  (t.two ? (void)(KERNEL<MmCfg<NT, 2, R>><<<t.n, NT, sm, st>>>(T, t.jobs, __VA_ARGS__))  \
-         : (void)(KERNEL<MmCfg<NT, 1, R>><<<t.n, NT, sm, st>>>(T, t.jobs, __VA_ARGS__)))
-#define MM_LAUNCH(KERNEL, TAIL, ...)                                 \
-  do {                                                               \
-    if (t.n <= 0) return;                                            \
-    const size_t sm = mm_smem(t.two ? 2 : 1, t.kp) + (TAIL);         \
-    const int nt = mm_threads(t.kp, t.n);                            \
-    if (nt == 256)                                                   \
-      MM_LAUNCH_CFG(KERNEL, 256, 1, __VA_ARGS__);                    \
-    else if (nt == 384 && t.kp <= 192)                               \
-      MM_LAUNCH_CFG(KERNEL, 384, 1, __VA_ARGS__);                    \
-    else if (nt == 384)                                              \
-      MM_LAUNCH_CFG(KERNEL, 384, 2, __VA_ARGS__);                    \
-    else if (t.kp <= 384)                                            \
-      MM_LAUNCH_CFG(KERNEL, 768, 1, __VA_ARGS__);                    \
-    else                                                             \
-      MM_LAUNCH_CFG(KERNEL, 768, 2, __VA_ARGS__);                    \
+#define MM_CASE(I, KERNEL, NT, S, R, ...)                                   \
+  case I:                                                                   \
+    KERNEL<MmCfg<NT, S, R>><<<t.n, NT, sm, st>>>(T, t.jobs, __VA_ARGS__);   \
+    break;
+#define MM_LAUNCH(KERNEL, TAIL, ...)                          \
+  do {                                                        \
+    if (t.n <= 0) return;                                     \
+    const size_t sm = mm_smem(t.two ? 2 : 1, t.kp) + (TAIL);  \
+    switch (mm_config(t)) {                                   \
+      MM_CASE(0, KERNEL, 256, 1, 1, __VA_ARGS__)              \
+      MM_CASE(1, KERNEL, 256, 2, 1, __VA_ARGS__)              \
+      MM_CASE(2, KERNEL, 384, 1, 1, __VA_ARGS__)              \
+      MM_CASE(3, KERNEL, 384, 2, 1, __VA_ARGS__)              \
+      MM_CASE(4, KERNEL, 384, 1, 2, __VA_ARGS__)              \
+      MM_CASE(5, KERNEL, 384, 2, 2, __VA_ARGS__)              \
+      MM_CASE(6, KERNEL, 768, 1, 1, __VA_ARGS__)              \
+      MM_CASE(7, KERNEL, 768, 2, 1, __VA_ARGS__)              \
+      MM_CASE(8, KERNEL, 768, 1, 2, __VA_ARGS__)              \
+      MM_CASE(9, KERNEL, 768, 2, 2, __VA_ARGS__)              \
+    }                                                         \
   } while (0)
 
 namespace {
 template <class K>
-void opt_in(K k) {
-  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(mm_smem(2, MM_KMAX) + mm_tail(MM_CMAX)));
+void opt_in(unsigned configs, int i, K k) {
+  if (configs >> i & 1)
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(mm_smem(2, MM_KMAX) + mm_tail(MM_CMAX)));
 }
 }  // namespace
-#define MM_OPT_IN(KERNEL)                                                                                      \
-  opt_in(KERNEL<MmCfg<256, 1, 1>>), opt_in(KERNEL<MmCfg<256, 2, 1>>), opt_in(KERNEL<MmCfg<384, 1, 1>>),        \
-      opt_in(KERNEL<MmCfg<384, 2, 1>>), opt_in(KERNEL<MmCfg<384, 1, 2>>), opt_in(KERNEL<MmCfg<384, 2, 2>>),    \
-      opt_in(KERNEL<MmCfg<768, 1, 1>>), opt_in(KERNEL<MmCfg<768, 2, 1>>), opt_in(KERNEL<MmCfg<768, 1, 2>>),    \
-      opt_in(KERNEL<MmCfg<768, 2, 2>>)
+#define MM_OPT_IN(KERNEL)                                                                                     \
+  opt_in(configs, 0, KERNEL<MmCfg<256, 1, 1>>), opt_in(configs, 1, KERNEL<MmCfg<256, 2, 1>>),                 \
+      opt_in(configs, 2, KERNEL<MmCfg<384, 1, 1>>), opt_in(configs, 3, KERNEL<MmCfg<384, 2, 1>>),             \
+      opt_in(configs, 4, KERNEL<MmCfg<384, 1, 2>>), opt_in(configs, 5, KERNEL<MmCfg<384, 2, 2>>),             \
+      opt_in(configs, 6, KERNEL<MmCfg<768, 1, 1>>), opt_in(configs, 7, KERNEL<MmCfg<768, 2, 1>>),             \
+      opt_in(configs, 8, KERNEL<MmCfg<768, 1, 2>>), opt_in(configs, 9, KERNEL<MmCfg<768, 2, 2>>)
 
 }  // namespace fcx

@@ -178,7 +178,7 @@ void launch_mm_filterT_q1(const DevTables& T, const MmTiles& t, const double* MF
   MM_LAUNCH(k_mm_filterT_q1, mm_tail(t.cmax), MF, e, out);
 }
 
-void set_mm_adj_attributes() {
+void set_mm_adj_attributes(unsigned configs) {
   MM_OPT_IN(k_mm_adj_q1);
   MM_OPT_IN(k_mm_adj_q2);
   MM_OPT_IN(k_mm_filterT_q1);

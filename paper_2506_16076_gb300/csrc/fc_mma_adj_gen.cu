@@ -180,7 +180,7 @@ void launch_mm_adj_gen_C(const DevTables& T, const MmTiles& t, const double* u, 
   MM_LAUNCH(k_mm_adj_gen_C, mm_tail(t.cmax), u, G, acc, dt);
 }
 
-void set_mm_adj_gen_attributes() {
+void set_mm_adj_gen_attributes(unsigned configs) {
   MM_OPT_IN(k_mm_adj_gen_A);
   MM_OPT_IN(k_mm_adj_gen_B);
   MM_OPT_IN(k_mm_adj_gen_C);

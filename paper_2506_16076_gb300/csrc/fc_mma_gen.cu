@@ -228,7 +228,7 @@ void launch_mm_gen_C(const DevTables& T, const MmTiles& t, const double* J, doub
   MM_LAUNCH(k_mm_gen_C, 0, J, G, sc);
 }
 
-void set_mm_gen_attributes() {
+void set_mm_gen_attributes(unsigned configs) {
   MM_OPT_IN(k_mm_gen_A);
   MM_OPT_IN(k_mm_gen_B);
   MM_OPT_IN(k_mm_gen_C);
