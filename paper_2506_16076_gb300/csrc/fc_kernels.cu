@@ -2,10 +2,11 @@
 //
 // Line kernels: one warp per grid-line segment, shared-memory mixed-radix Stockham
 // FFTs of the FC-Gram continued line (Sec. 2.2), fused with the Euler flux, the
-// artificial-viscosity flux and the SSPRK stage combination (Sec. 2.1, 2.3, 4.1).
-// The path is bound by the FP64 pipe (2 FP64 lanes/clk/SM on GB300), so the kernels
-// minimise FP64 instructions: packed real pairs per complex FFT, radix 2/3/4/5/7/8
-// butterflies with table twiddles, continuation as a 2d-term matvec.
+// artificial-viscosity flux and the SSPRK stage combination (Sec. 2.1, 2.3, 4.1). They
+// take the lines whose continued length the contraction kernels (fc_mma.cuh) do not: these
+// are twice as fast up to 1024 points. The FFT form is bound by the FP64 pipe (2 FP64
+// lanes/clk/SM on GB300), so it minimises FP64 instructions: packed real pairs per complex
+// FFT, radix 2/3/4/5/7/8 butterflies with table twiddles, continuation as a 2d-term matvec.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -1134,7 +1135,8 @@ __device__ __forceinline__ float dt_float(double x) {
 // maximum: those whose upper bound reaches the block's largest lower bound, or the patch's
 // maximum so far, are evaluated exactly, and a point whose state has the bits of the block's
 // representative (uniform free stream) has its value already: 0.78 ms (1.06 with bounds of
-// 2e-6 throughout). The maximum is that of the exact values.
+// 2e-6 throughout; 1.8 where most of the flow is the free stream up to rounding, and holds
+// the maximum). The maximum is that of the exact values.
 constexpr int DTB = 256, DTP = 4;  // threads, points per thread
 __global__ void __launch_bounds__(DTB) k_dt_reduce(DevTables T, const double* __restrict__ e,
                                                    const double* __restrict__ mu,

@@ -4,25 +4,25 @@
 // 600 TFLOP/s), so the circulant of a continued line (21 FP16 digit products per entry,
 // L^2/2 entries per line) costs less time than the FP64 butterflies of its two FFTs up to
 // lengths of a few hundred. What a line still needs from the FP64 pipe is its pointwise
-// work: fluxes, continuation and stage combination.
+// work: fluxes and stage combination.
 //
-// A CTA takes MM_LINES lines of one length (16 columns: 4 lines x 4 components). Each
-// thread loads its points, forms the values to transform and keeps them in registers until
-// the lines' largest magnitudes are known; then the sums and differences of the two halves
-// go to shared memory as FP16 digits. Each warp contracts 16 output rows at a time: the
-// right operand's fragments come from shared memory (ldmatrix), the left operand is a
-// Toeplitz matrix, so a fragment is three table entries of which each 16-column step needs
-// two new ones (read through L1: all warps of an SM share a table of 24 bytes per entry).
-// Digits of a line need 12 bytes per point and part; 128 threads for inner lengths up to
-// 128 and 256 beyond keep 16 warps per SM resident.
+// A CTA takes MM_LINES lines of one length (16 columns: 4 lines x 4 components): their values
+// go to shared memory with lanes along the points, are continued there, and are replaced by
+// the FP16 digits of the sums and differences of the two halves. A warp then contracts 16
+// output rows of two lines at a time: the right operand's fragments come from shared memory
+// (ldmatrix), the left operand is a Toeplitz matrix, so a fragment is three table entries of
+// which each 16-column step needs two new ones (read through L1: all warps of an SM share a
+// table of 24 bytes per entry). Digits need 12 bytes per point, component and part; 24
+// accumulators per lane leave room for 24 warps per SM at 80 registers.
 //
-// Measured (28M points, affine lines of 48 to 384 points, FFT kernels -> contraction, per
-// pass): q1 9.6 -> 4.5 ms, q2 10.0 -> 6.3 ms, filter q1 + q2 17.5 -> 8.1 ms; a 128 x 128
-// operator with L = 155 = 5 x 31: 462 -> 25 us. Largest error on white lines 2e-16 of the
-// largest value (FP64 FFT: 6e-16 to 9e-16). Of these times, passing the values through
-// shared memory (the fluxes' lanes then follow the points, 89% of them active instead of
-// 78%) and fetching a step's table entries one step ahead took 17%; a tile keeps its
-// sub-core's matrix pipe busy for 12k of about 26k cycles, the FP64 pipe for 10k to 15k.
+// Measured (28M points, affine lines of 48 to 384 points, per pass, FFT kernels -> 16 warps of
+// 16 columns each -> now): q1 9.6 -> 4.4 -> 3.7 ms, q2 10.0 -> 6.0 -> 5.1 ms, filter q1 + q2
+// 17.5 -> 8.0 -> 6.6 ms; a 128 x 128 operator with L = 155 = 5 x 31: 462 -> 23 us. Largest
+// error on white lines 2.4e-16 of the largest value (FP64 FFT: 6e-16 to 9e-16). No pipe is
+// full (ncu in profiles/k_mm_cart_cyl_array10.md): fixed latencies of the integer chains
+// and the barriers between a tile's phases are what is left; 64 registers and 32 warps gained
+// 1% in q1 and lost 6% in q2 (spills), quartering the even part (22% fewer matrix
+// instructions, twice the live sums) lost 8% and 18%.
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -223,7 +223,7 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
                                          Ep ep) {
   constexpr int NT = Cfg::NT, S = Cfg::S, NW = NT / 32, TS = NT / 4;  // TS: points per step of a line
   // opaque copies: without them the compiler hoists the address arithmetic of both of a
-  // kernel's rounds out of their loop (250 registers, 280 bytes of spills; so 128 and < 100)
+  // kernel's rounds out of their loop (250 registers wanted instead of 160, at that time)
   int tid = threadIdx.x;
   MmPlan p = plan;
   asm volatile("" : "+r"(tid), "+r"(p.H), "+r"(p.Kp), "+r"(p.nx), "+r"(p.Mp));
