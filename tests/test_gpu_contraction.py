@@ -102,3 +102,24 @@ def test_curvilinear_patch_after_affine_ones(gpu_lib, wall_form):
     ctx.rhs(e, out, to_dev_scalar_field(mu))
     errs = rel_err(from_dev(out, w), sv.rhs(st, mu))
     assert max(errs) < 1e-11, errs
+
+
+@pytest.mark.parametrize("k", [-400, 400])
+def test_viscosity_of_a_scaled_state_has_the_same_bits(gpu_lib, k):
+    """Quotients from a shared reciprocal (exponents in the middle of the range) against
+    divisions (the state times 2^400 or 2^-400): velocity, Mach number and sound speed do not
+    depend on the scale, so neither do the classes and the viscosity, to the last bit."""
+    w = _box(301, 203)
+    ctx = gpu_lib.Context(w)
+    g = np.random.default_rng(7)
+    st = W.random_smooth_state(w, seed=5, amp=0.2)
+    st[0] = np.array(st[0])
+    st[0][:, :, 100:] *= 1.0 + 1e-3 * g.standard_normal(st[0][:, :, 100:].shape)  # all significands
+    st[0][2][:, :200] = 0.0  # no velocity across
+    e = to_dev(st)
+    mu, mu_s = torch.empty_like(e[0]), torch.empty_like(e[0])
+    tau, tau_s = (torch.empty(e.shape[1], dtype=torch.int32, device="cuda") for _ in range(2))
+    ctx.viscosity(e, mu, tau)
+    ctx.viscosity(e * 2.0**k, mu_s, tau_s)
+    assert int(tau.min()) < int(tau.max()) and float(mu.max()) > 0.0
+    assert torch.equal(tau, tau_s) and torch.equal(mu, mu_s)
