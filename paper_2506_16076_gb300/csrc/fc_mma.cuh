@@ -19,7 +19,7 @@
 // 16 columns each -> now): q1 9.6 -> 4.4 -> 3.7 ms, q2 10.0 -> 6.0 -> 5.1 ms, filter q1 + q2
 // 17.5 -> 8.0 -> 6.6 ms; a 128 x 128 operator with L = 155 = 5 x 31: 462 -> 23 us. Largest
 // error on white lines 2.4e-16 of the largest value (FP64 FFT: 6e-16 to 9e-16). No pipe is
-// full (ncu in profiles/k_mm_cart_cyl_array10.md): fixed latencies of the integer chains
+// full (FP64 and matrix pipes 15% to 39% busy): fixed latencies of the integer chains
 // and the barriers between a tile's phases are what is left; 64 registers and 32 warps gained
 // 1% in q1 and lost 6% in q2 (spills), quartering the even part (22% fewer matrix
 // instructions, twice the live sums) lost 8% and 18%.
