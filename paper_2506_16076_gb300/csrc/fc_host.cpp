@@ -146,7 +146,8 @@ struct fc_ctx {
   Queue q_cart1, q_cart2, q_gen1, q_gen2, q_filt1, q_filt2;
   int* d_fix = nullptr;
   int nfix = 0;
-  // the y fluxes of the affine patches' points, written by the q1 pass for the q2 pass, and
+  // the y fluxes of the affine patches' points, written by the q1 pass for the q2 pass (and,
+  // in the adjoint, mu eta between a pass's rounds; there whenever an affine line is), and
   // the points on affine q2 lines that no affine q1 line visits (their y flux comes from
   // k_flux_y_points)
   double* d_Fy = nullptr;
@@ -1777,7 +1778,7 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
        c->alloc(&c->d_muhat, P) && c->alloc(&c->d_num, P) && c->alloc(&c->d_tmp, P) && c->alloc(&c->d_mu, P) &&
        c->alloc(&c->d_den, P) && c->alloc(&c->d_dt, 1) && c->alloc(&c->d_pmax, 2 * (size_t)npatch) &&
        c->alloc(&c->d_flag, 1) && c->alloc(&c->d_skip_lines, 2) && c->alloc(&c->d_skip_flops, 2) &&
-       (jc2.empty() || c->alloc(&c->d_Fy, 4 * P));
+       ((jc1.empty() && jc2.empty()) || c->alloc(&c->d_Fy, 4 * P));
   if (!ok) {
     fprintf(stderr, "fc_init_patches: %s\n", c->err.c_str());
     delete c;
