@@ -1173,7 +1173,7 @@ __global__ void __launch_bounds__(DTB) k_dt_reduce(DevTables T, const double* __
   int patch[DTP];
   unsigned long long bm = 0;
   const bool whole = first == last;
-  const float g1 = (float)gam - 1.f;
+  const float g1 = (float)(gam - 1.0);  // one rounding, also where gamma is near 1
   float low = -1.f;
   int at = -1;
 #pragma unroll
@@ -1195,7 +1195,7 @@ __global__ void __launch_bounds__(DTB) k_dt_reduce(DevTables T, const double* __
   for (int k = 0; k < DTP; ++k) {
     // relative errors: truncated inputs 2^-23 and FP32 operations 2^-24 each leave 3.6e-7 in u,
     // v and 6e-7 in ke; the pressure loses what E and ke share, and a half of its error
-    // reaches a; sums and root 1.2e-7
+    // reaches a; gamma - 1, gamma, 1 / rho, three products and the root 3.3e-7 in a; sums 1.2e-7
     const float r = dt_float(q[k][0]), mx = dt_float(q[k][1]), my = dt_float(q[k][2]), E = dt_float(q[k][3]);
     const float ir = 1.f / r, u = fabsf(mx * ir), v = fabsf(my * ir);
     const float ke = 0.5f * (fabsf(mx) * u + fabsf(my) * v), p = g1 * (E - ke);
