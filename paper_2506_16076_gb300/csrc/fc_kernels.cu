@@ -1199,11 +1199,12 @@ __global__ void __launch_bounds__(DTB) k_dt_reduce(DevTables T, const double* __
     const float r = dt_float(q[k][0]), mx = dt_float(q[k][1]), my = dt_float(q[k][2]), E = dt_float(q[k][3]);
     const float ir = 1.f / r, u = fabsf(mx * ir), v = fabsf(my * ir);
     const float ke = 0.5f * (fabsf(mx) * u + fabsf(my) * v), p = g1 * (E - ke);
-    const float a = sqrtf((float)gam * p * ir);
+    const float a2 = (float)gam * p * ir, a = sqrtf(a2);
     const float dp = g1 * (1e-7f * fabsf(E) + 4e-7f * ke);  // a half of p's error
     const float S = u + v + a, dS = 8e-7f * (u + v) + a * (8e-7f + dp / p);
-    // false on NaN too; the pressure's sign and its root's expansion need dp well below p
-    const bool sure = p > 0.f && r > 0.f && dp < 0.25f * p && dS < 0.25f * S;
+    // false on NaN too; the pressure's sign and its root's expansion need dp well below p, and
+    // p and a^2 far from underflow (1e-30) make what underflows elsewhere too small to matter
+    const bool sure = p > 1e-30f && a2 > 1e-30f && r > 0.f && dp < 0.25f * p && dS < 0.25f * S;
     hi[k] = patch[k] < 0 ? -1.f : (sure ? S + dS : INFINITY);
     if (patch[k] >= 0 && sure && S - dS > low) {
       low = S - dS;

@@ -67,3 +67,12 @@ def test_time_step_is_that_of_the_largest_speed(gpu_lib, gamma):
     dt = torch.zeros(1, dtype=torch.float64, device="cuda")
     ctx.timestep(e, mu, dt)
     assert bool(torch.isnan(dt).all())
+
+
+@pytest.mark.parametrize("k", [60, 80, 100, -60, -100])
+def test_time_step_of_scaled_states(gpu_lib, k):
+    """Densities times 2^k and pressures times 2^-k (speeds times 2^-k): values that FP32 holds,
+    with squares of the sound speed that it does not."""
+    rng = np.random.default_rng(12)
+    scale = torch.tensor([2.0**k, 1.0, 1.0, 2.0**-k], dtype=torch.float64, device="cuda")[:, None]
+    _check(gpu_lib, [(64, 48)], 1.4, [_state(rng, 64 * 48, 1.4, 0.5, 0.3) * scale for _ in range(20)])
