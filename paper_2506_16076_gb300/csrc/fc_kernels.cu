@@ -1184,12 +1184,38 @@ __global__ void __launch_bounds__(DTB) k_dt_reduce(DevTables T, const double* __
 #pragma unroll
     for (int c = 0; c < 4; ++c) q[k][c] = e[pc + c * cs];
     const unsigned long long m = (unsigned long long)__double_as_longlong(mu[pc]);
-    if (patch[k] >= 0) {
-      if (whole)
-        bm = m > bm ? m : bm;
-      else
+    if (patch[k] >= 0) bm = m > bm ? m : bm;
+  }
+  if (!whole) {  // a patch boundary in the block: every point exactly, one pair of atomics per
+                 // warp of one patch (per point, they took as long as the speeds)
+#pragma unroll
+    for (int k = 0; k < DTP; ++k) {
+      const unsigned act = __ballot_sync(0xffffffffu, patch[k] >= 0);
+      if (act == 0) continue;
+      unsigned long long s = 0, m = 0;
+      if (patch[k] >= 0) {
+        s = dt_speed(q[k], gam);
+        m = (unsigned long long)__double_as_longlong(mu[p0 + tid + k * DTB]);
+      }
+      const int pw = __shfl_sync(0xffffffffu, patch[k], __ffs(act) - 1);
+      if (__all_sync(0xffffffffu, patch[k] < 0 || patch[k] == pw)) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const unsigned long long s2 = __shfl_down_sync(0xffffffffu, s, o);
+          const unsigned long long m2 = __shfl_down_sync(0xffffffffu, m, o);
+          s = s2 > s ? s2 : s;
+          m = m2 > m ? m2 : m;
+        }
+        if (lane == 0) {
+          atomicMax(pmax + 2 * pw, s);
+          atomicMax(pmax + 2 * pw + 1, m);
+        }
+      } else if (patch[k] >= 0) {
+        atomicMax(pmax + 2 * patch[k], s);
         atomicMax(pmax + 2 * patch[k] + 1, m);
+      }
     }
+    return;
   }
 #pragma unroll
   for (int k = 0; k < DTP; ++k) {
@@ -1210,12 +1236,6 @@ __global__ void __launch_bounds__(DTB) k_dt_reduce(DevTables T, const double* __
       low = S - dS;
       at = tid + k * DTB;
     }
-  }
-  if (!whole) {  // a patch boundary in the block: every point exactly
-#pragma unroll
-    for (int k = 0; k < DTP; ++k)
-      if (patch[k] >= 0) atomicMax(pmax + 2 * patch[k], dt_speed(q[k], gam));
-    return;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
