@@ -141,6 +141,7 @@ struct fc_ctx {
     Job* dmm = nullptr;                          // all tiles' jobs: per patch, then batched
     uint8_t* dvisc = nullptr;                    // their viscous flags (valid while ctx::flags_on)
     int ntiles = 0;                              // per order
+    bool filter = false;                         // the filter's lines (contracted with the filter's table)
     std::unique_ptr<Queue> rest;
   };
   Queue q_cart1, q_cart2, q_gen1, q_gen2, q_filt1, q_filt2;
@@ -931,7 +932,9 @@ struct Builder {
     }
     fma_tables(p, tg);
     plans.push_back(p);
-    mm.push_back(mm_length_ok(L) ? mm_plan(L, &sig, mmlo, mmhi) : MmPlan{});
+    // an odd p makes sigma(2k/L) uneven in k: not one circulant for the FFT engine's packed pairs
+    const bool even = prm.p_f % 2 == 0;
+    mm.push_back(mm_length_ok(L) ? mm_plan(L, even ? &sig : nullptr, mmlo, mmhi) : MmPlan{});
     std::vector<Plan> alt{p};
     for (size_t o = 1; o < orders.size(); ++o) {
       if ((int)orders[o].size() > MAXST) continue;
@@ -1016,7 +1019,7 @@ void make_tiles(fc_ctx* c, fc_ctx::Queue& q, const std::vector<Job>& pp, const s
   std::vector<Job> rest;
   for (const Job& J : pp) {
     const MmPlan& m = mm[J.plan];
-    if (m.H == 0 || J.C > MM_CMAX || c->d > 8) {
+    if (m.H == 0 || J.C > MM_CMAX || c->d > 8 || (q.filter ? m.ftab : m.dtab) < 0) {
       rest.push_back(J);
       continue;
     }
@@ -1707,6 +1710,7 @@ fc_status fc_init_patches(fc_ctx** out, const fc_patch_desc* patches, int npatch
 
   // ---- upload
   bool ok = true;
+  c->q_filt1.filter = c->q_filt2.filter = true;
   make_queue(c, c->q_cart1, jc1, B.plans, npatch, ok, &B.mm);
   make_queue(c, c->q_cart2, jc2, B.plans, npatch, ok, &B.mm);
   make_queue(c, c->q_gen1, jg1, B.plans, npatch, ok, &B.mm);

@@ -23,11 +23,10 @@
 
 namespace fcx {
 
-// whether lines of continued length L run as contractions: both parts' inner length,
-// padded to the instruction's 16, fits 256 (exact level sums, one CTA's pairs)
+// whether lines of continued length L run as contractions: the parts' inner length fits a CTA
 inline bool mm_length_ok(int L) { return L >= 16 && ((L % 2 == 0 && L / 2 <= MM_KMAX) || (L % 2 == 1 && L <= MM_KMAX)); }
 
-// FP16 bits of an integer in [-1024, 1024]
+// FP16 bits of an integer in [-2048, 2048]
 inline uint16_t mm_half(int v) {
   if (v == 0) return 0;
   const int a = v < 0 ? -v : v;
@@ -48,7 +47,10 @@ inline void mm_digits(long long q, int* dg) {
 
 // appends the tables of coefficients c (L values, c(m) = c[m mod L]) to lo / hi (entries
 // of digits 0..3 and 4..5) and returns the first entry; *te: the coefficients were scaled
-// by 2^te
+// by 2^te, which takes the largest to about 2^SP_COEF but leaves the joined sums, and U + V and
+// U - V, in 63 bits: with line values below 2^(SP_DATA + 1) each is at most
+// sum |c| 2^(te + SP_DATA + 2) units of 2^SP_UNIT. (A broad filter's coefficients are small and
+// many, sum |c| about 1: 2^64 or so then, four bits more than the largest of a narrow one gets.)
 inline int mm_table(const MmPlan& p, int L, const std::vector<long double>& c, std::vector<uint4>& lo,
                     std::vector<uint2>& hi, int* te) {
   const int H = p.H, S = p.S, nx = p.nx, off = p.Mp;
@@ -58,10 +60,14 @@ inline int mm_table(const MmPlan& p, int L, const std::vector<long double>& c, s
     const long double b = c[(size_t)((((m + H) % L) + L) % L)];
     return s ? a - b : a + b;
   };
-  long double top = 0;
+  long double top = 0, sum = 0;
   for (int s = 0; s < S; ++s)
     for (int m = 0; m < H; ++m) top = std::max(top, std::fabs(t(s, m)));
-  *te = top > 0 ? SP_COEF - (int)std::lround(std::log2((double)top)) : SP_COEF;
+  for (long double v : c) sum += std::fabs(v);
+  *te = SP_COEF;
+  if (top > 0)
+    *te = std::min(SP_COEF - (int)std::lround(std::log2((double)top)),
+                   63 + SP_UNIT - SP_DATA - 2 + (int)std::floor(-0.1 - std::log2((double)sum)));
   const int first = (int)lo.size();
   for (int s = 0; s < S; ++s) {
     std::vector<uint16_t> dg((size_t)SP_DIGITS * (nx + 1));
@@ -82,7 +88,7 @@ inline int mm_table(const MmPlan& p, int L, const std::vector<long double>& c, s
 }
 
 // MmPlan of length L (mm_length_ok) with its derivative table and, when sig is given
-// (sigma(2k/L) for k = 0..L/2), its filter table
+// (sigma(2k/L) >= 0 for k = 0..L/2) and its size is that of FP64 numbers, its filter table
 inline MmPlan mm_plan(int L, const std::vector<long double>* sig, std::vector<uint4>& lo, std::vector<uint2>& hi) {
   const long double PI_L = 3.14159265358979323846264338327950288L;
   MmPlan p{};
@@ -104,10 +110,21 @@ inline MmPlan mm_plan(int L, const std::vector<long double>* sig, std::vector<ui
   if (L % 2 == 0) c[L / 2] = 0.0L;
   p.dtab = mm_table(p, L, c, lo, hi, &p.dte);
   p.ftab = -1;
-  if (sig) {
-    // cosine sums in 128-bit integers (sigma and cosines in 2^-58)
+  // 2^(se - 1) < largest sigma <= 2^se
+  long double stop = 0;
+  bool usable = sig != nullptr;
+  if (sig)
+    for (long double v : *sig) {
+      usable = usable && std::isfinite(v);
+      stop = std::max(stop, v);
+    }
+  int se = 0;
+  if (usable && stop > 0 && std::frexp(stop, &se) == 0.5L) --se;
+  usable = usable && stop > 0 && std::abs(se) <= 900;
+  if (usable) {
+    // cosine sums in 128-bit integers (sigma in 2^(se - 58), cosines in 2^-58)
     std::vector<long long> sq((size_t)L / 2 + 1), cq((size_t)L);
-    for (int k = 0; 2 * k <= L; ++k) sq[k] = (long long)std::llround(std::ldexp((*sig)[k], 58));
+    for (int k = 0; 2 * k <= L; ++k) sq[k] = (long long)std::llround(std::ldexp((*sig)[k], 58 - se));
     for (int j = 0; 2 * j <= L; ++j) {
       cq[j] = (long long)std::llround(std::ldexp(cs[4 * j], 58));
       if (j) cq[L - j] = cq[j];
@@ -118,7 +135,7 @@ inline MmPlan mm_plan(int L, const std::vector<long double>* sig, std::vector<ui
       a *= 2;
       a += (__int128)sq[0] * cq[0];
       if (L % 2 == 0) a += (__int128)sq[L / 2] * cq[(size_t)((long long)(L / 2) * m % L)];
-      const long double v = std::ldexp((long double)a, -116) / L;
+      const long double v = std::ldexp((long double)a, se - 116) / L;
       c[m] = v;
       if (m) c[L - m] = v;
     }

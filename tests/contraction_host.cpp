@@ -1,11 +1,12 @@
 // Host build of the split-integer contraction (fc_split.cuh, fc_mmtab.h): the tables and
 // the arithmetic the GPU kernels use, with the matrix products formed in plain loops.
 //
-//   contraction_host L1 L2 ...
-//     for every continued length, the derivative and the filter of a white line, a nearly
+//   contraction_host [filter alpha p] L1 L2 ...
+//     for every continued length, the derivative and the filter (filter: only that one, with
+//     sigma(z) = exp(-alpha z^p); else alpha = 10, p = 14) of a white line, a nearly
 //     constant one and one with a spike against the same circulant in long double; prints
-//     "L op kind error/max|x| largest_level_sum" (op 0: derivative, 1: filter), or "L none"
-//     when lines of this length are left to the FFT kernels.
+//     "L op kind error/max|x| largest_level_sum" (op 0: derivative, 1: filter; the error also over
+//     the largest sigma), or "L none" when lines of this length are left to the FFT kernels.
 //
 //   contraction_host continuation C Q
 //     the continuation's digit products (mm_continuation, fragments read back as the matrix
@@ -113,7 +114,9 @@ int main(int argc, char** argv) {
   std::mt19937_64 g(1);
   std::uniform_real_distribution<double> U(-1.0, 1.0);
   const long double PI = 3.14159265358979323846264338327950288L;
-  for (int a = 1; a < argc; ++a) {
+  const bool filter = argc > 4 && !std::strcmp(argv[1], "filter");
+  const long double alpha = filter ? std::atof(argv[2]) : 10.0L, pw = filter ? std::atof(argv[3]) : 14.0L;
+  for (int a = filter ? 4 : 1; a < argc; ++a) {
     const int L = std::atoi(argv[a]);
     if (!mm_length_ok(L)) {
       printf("%d none\n", L);
@@ -122,9 +125,11 @@ int main(int argc, char** argv) {
     std::vector<uint4> lo;
     std::vector<uint2> hi;
     std::vector<long double> sig;
-    for (int k = 0; 2 * k <= L; ++k) sig.push_back(expl(-10.0L * powl(2.0L * k / L, 14)));
+    for (int k = 0; 2 * k <= L; ++k) sig.push_back(expl(-alpha * powl(2.0L * k / L, pw)));
+    const double stop = (double)*std::max_element(sig.begin(), sig.end());
     const MmPlan p = mm_plan(L, &sig, lo, hi);
-    for (int op = 0; op < 2; ++op) {
+    if (filter && p.ftab < 0) printf("%d none\n", L);
+    for (int op = filter; op < (p.ftab < 0 ? 1 : 2); ++op) {
       std::vector<long double> c(L, 0.0L);  // the circulant, by its definition
       for (int m = 0; m < L; ++m) {
         long double s = 0;
@@ -167,7 +172,7 @@ int main(int argc, char** argv) {
               si[l] = (int)lev[l];
               level = std::max(level, std::fabs(lev[l]));
             }
-            joined += sp_join(si);
+            joined = (long long)((unsigned long long)joined + (unsigned long long)sp_join(si));
             }
             W[s].push_back(joined);
           }
@@ -179,7 +184,7 @@ int main(int argc, char** argv) {
           for (int j = 0; j < L; ++j) ref += c[((i - j) % L + L) % L] * (long double)x[j];
           err = std::max(err, (double)fabsl((long double)(sp_double(v) * fac) - ref));
         }
-        printf("%d %d %d %.3e %.0f\n", L, op, kind, err / top, level);
+        printf("%d %d %d %.3e %.0f\n", L, op, kind, err / top / (op ? stop : 1.0), level);
       }
     }
   }

@@ -45,6 +45,26 @@ def test_contraction_matches_the_circulant(exe):
         assert float(level) < 2 ** 24, (L, op, kind, level)
 
 
+# broad kernels (many coefficients of one size), an amplifying one, small ones throughout; p = 0
+# scales all modes alike
+@pytest.mark.parametrize("alpha,p", [(2000, 2), (1700, 2), (50, 1), (1e6, 4), (0, 2), (-5, 2), (10, 0), (10, -1)])
+def test_filters_of_any_width(exe, alpha, p):
+    r = subprocess.run([exe, "filter", str(alpha), str(p), "17", "64", "255", "511", "512", "1024"],
+                       capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr
+    rows = [ln.split() for ln in r.stdout.splitlines()]
+    assert len(rows) == 18
+    for L, op, kind, err, level in rows:
+        assert float(err) < 9e-16, (L, op, kind, err)
+
+
+def test_filters_out_of_range_are_left_to_the_transforms(exe):
+    # sigma up to e^2000 and down to e^-2000: neither is an FP64 number
+    for alpha, p in (("-2000", "2"), ("2000", "0")):
+        r = subprocess.run([exe, "filter", alpha, p, "64", "512"], capture_output=True, text=True)
+        assert r.returncode == 0 and [ln.split()[1] for ln in r.stdout.splitlines()] == ["none"] * 2
+
+
 def test_other_lengths_are_left_to_the_transforms(exe):
     r = subprocess.run([exe, "15", "513", "1026", "2048"], capture_output=True, text=True)
     assert r.returncode == 0 and [ln.split()[1] for ln in r.stdout.splitlines()] == ["none"] * 4

@@ -13,7 +13,7 @@ import torch
 
 from oracle import solver as S
 from paper_2506_16076_gb300 import workloads as W
-from tests.gpu_helpers import fp64_floor, from_dev, rel_err, smooth_mu, to_dev, to_dev_scalar_field
+from tests.gpu_helpers import fp64_floor, from_dev, rel_err, smooth_mu, to_dev, to_dev_scalar_field, ulp_floor
 
 pytestmark = pytest.mark.gpu
 
@@ -49,6 +49,51 @@ def test_rhs_and_filter_at_the_length_edges(gpu_lib, n1, n2):
     tol = max(1e-11, 2 * max(rel_err(fp64_floor(sv, lambda: sv.filter(st)), ref)))
     errs = rel_err(from_dev(e, w), ref)
     assert max(errs) < tol, (errs, tol)
+
+
+@pytest.mark.parametrize("alpha,p", [(2000.0, 2), (-5.0, 2), (10.0, 0)])
+def test_filters_of_any_width(gpu_lib, alpha, p):
+    """Continued lengths 512 and 255; sigma from 1 over few modes to e^5, and e^-10 throughout. A
+    filter of few modes takes up the rounding of the end values that the continuation weighs by
+    thousands, so the bound includes twice the effect of one rounding of the input (ulp_floor)."""
+    w = _box(485, 228)
+    w = dataclasses.replace(w, params=dataclasses.replace(w.params, alpha_f=alpha, p_f=p))
+    ctx = gpu_lib.Context(w)
+    sv = S.Solver(w)
+    st = W.random_smooth_state(w, seed=9, amp=0.2)
+    e = to_dev(st)
+    ctx.filter(e)
+    ref = sv.filter(st)
+    tol = max([1e-11] + [2 * x for x in rel_err(fp64_floor(sv, lambda: sv.filter(st)), ref) + ulp_floor(sv.filter, st)])
+    errs = rel_err(from_dev(e, w), ref)
+    assert max(errs) < tol, (errs, tol)
+
+
+def test_odd_filter_power_runs_as_transforms(gpu_lib):
+    """With an odd p, sigma(2k/L) differs for k and -k: such a filter is a multiplier of the packed
+    transforms of (rho, rho u) and (rho v, theta), as on the lines that are too long for contractions."""
+    from oracle import euler, fc
+    w = _box(101, 37)
+    prm = w.params = dataclasses.replace(w.params, alpha_f=0.5, p_f=1)
+    st = W.random_smooth_state(w, seed=9, amp=0.2)[0]
+
+    def lines(f):
+        n = f.shape[-1]
+        c = fc.extend_ld(f, prm.d, fc.choose_C(n, prm.C0, prm.c_policy, prm.d))
+        L = c.shape[-1]
+        s = np.exp(-prm.alpha_f * (2.0 * np.fft.fftfreq(L, 1.0 / L).round() / L) ** prm.p_f)
+        if L % 2 == 0:
+            s[L // 2] = np.exp(-prm.alpha_f)
+        z = np.fft.ifft(s * np.fft.fft(c[0::2] + 1j * c[1::2], axis=-1), axis=-1)[..., :n]
+        return np.stack([z[0].real, z[0].imag, z[1].real, z[1].imag])
+
+    q = lines(np.stack([st[0], st[1], st[2], euler.temperature(st, prm.gamma)]))
+    q = np.swapaxes(lines(np.ascontiguousarray(np.swapaxes(q, 1, 2))), 1, 2)
+    ref = np.stack([q[0], q[1], q[2], euler.energy_from_theta(*q, prm.gamma)])
+    e = to_dev([st])
+    gpu_lib.Context(w).filter(e)
+    errs = rel_err(from_dev(e, w), [ref])
+    assert max(errs) < 1e-11, errs
 
 
 def test_uniform_gas_at_rest_stays_exactly_at_rest(gpu_lib):
