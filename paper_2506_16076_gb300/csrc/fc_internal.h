@@ -15,7 +15,7 @@ constexpr int SDNN_H = 16;      // hidden width of the stand-in classifier
 constexpr int MAX_GENERIC_RADIX = 128;  // largest prime factor of a continued length
 constexpr int CONT_TMP = 32;    // complex scratch per warp after the line buffer (detrended end data, d <= 8)
 constexpr int MM_KMAX = 512;     // largest inner length of a tensor-core line contraction (fc_mma.cu)
-constexpr int MM_KCHUNK = 256;   // columns whose digit products are summed in FP32 before they are joined
+constexpr int MM_KCHUNK = 256;   // columns after which the level sums are joined
 constexpr int MM_CMAX = 128;     // largest continuation length of a contracted line
 constexpr int MM_LINES = 4;      // lines per tile of the contraction kernels
 constexpr int NCLASS = 24;      // length classes of the line queues: ceil(log2 Lmax)

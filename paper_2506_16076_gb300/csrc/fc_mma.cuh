@@ -147,6 +147,7 @@ __device__ __forceinline__ void mm_part(const uint4* __restrict__ lo, const uint
     baddr += 32;
 #pragma unroll
     for (int i = 0; i < SP_DIGITS; ++i) Am[i] = Ap[i];
+    sp_carries(acc, k0, ke - kb);
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -448,8 +449,8 @@ __device__ __forceinline__ void mm_round(const DevTables& T, const MmPlan& plan,
       }
     }
   };
-  // joined sums of part s for 16 rows from i0 and the two lines from l0. FP32 sums are exact
-  // over MM_KCHUNK columns: longer ones (768 threads) in two pieces
+  // joined sums of part s for 16 rows from i0 and the two lines from l0, joined every MM_KCHUNK
+  // columns (768 threads)
   auto part = [&](int s, int i0, int l0, long long* w) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) w[q] = 0;

@@ -45,8 +45,31 @@ inline void mm_digits(long long q, int* dg) {
   dg[0] = (int)q;
 }
 
+// Whether the level sums of one part's digits D[digit][x] stay exact for any data: per level, the
+// largest sum over a window of columns between carries (fc_split.cuh; any window of x: a row's
+// columns are consecutive entries) of |coefficient digit| times the largest data digit (the first is
+// at most 128, 256 for sums of two values), with 2^16 for what carries bring and leave, below 2^24
+inline bool mm_sums_exact(const std::vector<int>* D, int S, int H) {
+  const int nx = (int)D[0].size();
+  const long long B[4] = {128 * S, 512, 512, 512};
+  for (int l = 0; l < 4; ++l) {
+    const int w = std::min(H, l == 0 ? MM_KCHUNK : (l == 1 ? SP_CARRY2 : SP_CARRY));
+    auto at = [&](int x) {
+      long long a = 0;
+      for (int i = 0; i <= l; ++i) a += std::abs(D[i][x]) * B[l - i];
+      return a;
+    };
+    long long s = 0;
+    for (int x = 0; x < nx; ++x) {
+      s += at(x) - (x >= w ? at(x - w) : 0);
+      if (s + (1 << 16) >= 1 << 24) return false;
+    }
+  }
+  return true;
+}
+
 // appends the tables of coefficients c (L values, c(m) = c[m mod L]) to lo / hi (entries
-// of digits 0..3 and 4..5) and returns the first entry; *te: the coefficients were scaled
+// of digits 0..3 and 4..5) and returns the first entry (-1: their level sums would not be exact); *te: the coefficients were scaled
 // by 2^te, which takes the largest to about 2^SP_COEF but leaves the joined sums, and U + V and
 // U - V, in 63 bits: with line values below 2^(SP_DATA + 1) each is at most
 // sum |c| 2^(te + SP_DATA + 2) units of 2^SP_UNIT. (A broad filter's coefficients are small and
@@ -68,16 +91,26 @@ inline int mm_table(const MmPlan& p, int L, const std::vector<long double>& c, s
   if (top > 0)
     *te = std::min(SP_COEF - (int)std::lround(std::log2((double)top)),
                    63 + SP_UNIT - SP_DATA - 2 + (int)std::floor(-0.1 - std::log2((double)sum)));
+  std::vector<int> D[2][SP_DIGITS];
+  bool exact = false;
+  for (int cut = 0; cut < 5 && !exact; ++cut) {  // (broad filters have bits to spare)
+    if (cut) --*te;
+    exact = true;
+    for (int s = 0; s < S; ++s) {
+      for (int k = 0; k < SP_DIGITS; ++k) D[s][k].resize(nx + 1);
+      for (int x = 0; x <= nx; ++x) {
+        int d[SP_DIGITS];
+        mm_digits((long long)std::llround(std::ldexp(t(s, off - x), *te)), d);
+        for (int k = 0; k < SP_DIGITS; ++k) D[s][k][x] = d[k];
+      }
+      exact = exact && mm_sums_exact(D[s], S, H);
+    }
+  }
+  if (!exact) return -1;
   const int first = (int)lo.size();
   for (int s = 0; s < S; ++s) {
-    std::vector<uint16_t> dg((size_t)SP_DIGITS * (nx + 1));
-    for (int x = 0; x <= nx; ++x) {
-      int d[SP_DIGITS];
-      mm_digits((long long)std::llround(std::ldexp(t(s, off - x), *te)), d);
-      for (int k = 0; k < SP_DIGITS; ++k) dg[(size_t)k * (nx + 1) + x] = mm_half(d[k]);
-    }
     auto pair = [&](int k, int x) {
-      return (uint32_t)dg[(size_t)k * (nx + 1) + x] | ((uint32_t)dg[(size_t)k * (nx + 1) + x + 1] << 16);
+      return (uint32_t)mm_half(D[s][k][x]) | ((uint32_t)mm_half(D[s][k][x + 1]) << 16);
     };
     for (int x = 0; x < nx; ++x) {
       lo.push_back(uint4{pair(0, x), pair(1, x), pair(2, x), pair(3, x)});
@@ -147,7 +180,8 @@ inline MmPlan mm_plan(int L, const std::vector<long double>* sig, std::vector<ui
 // The continuation's contraction: ext_k = sum_q M[k][q] e_q over the Q <= 16 detrended end
 // values of a line, as digit products of one 16-column step. The columns' coefficients differ
 // by four orders of magnitude (second differences 1e4, values 1), so column q carries 2^-sq
-// and its value 2^sq. Fragments of the matrix instruction, 16 rows (continuation points) each:
+// and its value 2^sq. Levels 0 to 3 are exact for any data, as in mm_sums_exact, in the end with
+// one bit less of the coefficients (digits up to 512: 16 columns of 3 x 2^18 + 2^16). Fragments of the matrix instruction, 16 rows (continuation points) each:
 // [block][digit][lane], a lane's four registers side by side.
 inline MmCont mm_continuation(int C, int Q, const std::vector<long double>& M, std::vector<uint4>& lo) {
   MmCont r{};
@@ -159,10 +193,26 @@ inline MmCont mm_continuation(int C, int Q, const std::vector<long double>& M, s
     if (top > 0) std::frexp(top, &e);
     r.sq[q] = e;
   }
+  auto digits = [&](int k, int q, int* d) {
+    mm_digits((long long)std::llround(std::ldexp(M[(size_t)k * Q + q], SP_COEF - r.sq[q])), d);
+  };
+  bool exact = true;
+  for (int k = 0; k < C; ++k) {
+    long long s[4] = {0, 0, 0, 0};
+    for (int q = 0; q < Q; ++q) {
+      int d[SP_DIGITS];
+      digits(k, q, d);
+      for (int l = 0; l < 4; ++l)
+        for (int i = 0; i <= l; ++i) s[l] += (long long)std::abs(d[i]) * (i == l ? 128 : 512);
+    }
+    for (int l = 0; l < 4; ++l) exact = exact && s[l] < 1 << 24;
+  }
+  if (!exact)
+    for (int q = 0; q < Q; ++q) ++r.sq[q];
   auto digit = [&](int k, int q, int j) -> uint32_t {
     if (k >= C || q >= Q) return 0;
     int d[SP_DIGITS];
-    mm_digits((long long)std::llround(std::ldexp(M[(size_t)k * Q + q], SP_COEF - r.sq[q])), d);
+    digits(k, q, d);
     return mm_half(d[j]);
   };
   for (int b = 0; b < (C + 15) / 16; ++b)

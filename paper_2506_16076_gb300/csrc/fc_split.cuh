@@ -3,14 +3,21 @@
 // An FC line operator (derivative or filter of the continued line, eqs. fc_der and
 // filtering) is a circulant of length L: y_i = sum_j c(i - j) x_j. Data and coefficients
 // are held as fixed-point integers of 60 bits, cut into six balanced base-1024 digits in
-// [-512, 511]. A digit is exact in FP16, a product of two is at most 2^18 and a sum of up
-// to 256 of them stays below 2^24 for the operators used here (fc_mmtab.h), so the FP16
-// matrix instruction with FP32 accumulation adds them without rounding. The digit products
-// of equal weight (levels i + j = 0..5, 21 of the 36 pairs) share an accumulator; the
-// levels are joined in 64-bit integers. The dropped levels and the truncation of the data
-// leave an error of a few 2^-57 of the line's largest value times the operator's largest
-// coefficient, below the rounding of an FP64 transform of the same line.
+// [-512, 511]. A digit is exact in FP16, and the FP16 matrix instruction with FP32
+// accumulation adds digit products without rounding while their sums stay below 2^24. The
+// products of equal weight (levels i + j = 0..5, 21 of the 36 pairs) share an accumulator.
+// Levels 0 to 3 are exact for any data: level 3 hands what exceeds a digit to level 2, and 2
+// to 1, every 32 columns, level 1 to 0 every 64 (sp_carries), and a table is used only if its
+// digits keep these levels below 2^24 between the carries (mm_sums_exact in fc_mmtab.h: at most
+// 2^23.95 for the derivative and the default filter). Levels 4 and 5, which weigh 2^-56 and 2^-66
+// of the result's scale, stay below 2^24 for typical data and can reach 2^25.2 and 2^27.4 for data
+// whose digits all carry the signs of one row's coefficients; rounding their sums then costs up
+// to 2^-48 of that scale (an FP64 transform: 2^-50). The levels are joined in 64-bit integers.
+// The dropped levels and the truncation of the data leave an error of a few 2^-57 of the line's
+// largest value times the operator's largest coefficient, below the rounding of an FP64
+// transform of the same line.
 #pragma once
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -64,7 +71,35 @@ FC_HD long long sp_fixed(double x, int ex) {
 // as two FP16 integers in one word
 FC_HD uint32_t sp_field(long long biased, int k) { return (uint32_t)(biased >> (SP_BITS * (SP_DIGITS - 1 - k))) & 1023u; }
 
-// joined sum of the six level sums (exact integers below 2^24) in units 2^SP_UNIT
+// the multiple of 2^SP_BITS nearest to lo goes over to hi, the next higher level (|lo| < 2^31;
+// four FP32 operations, on a pipe that the contraction does not use otherwise)
+FC_HD void sp_carry(float& hi, float& lo) {
+  const float c = fmaf(lo, 1.f / (1 << SP_BITS), 12582912.f) - 12582912.f;  // 1.5 2^23: rounds to an integer
+  lo = fmaf(c, -(float)(1 << SP_BITS), lo);
+  hi += c;
+}
+// columns between carries out of levels 2 and 3, and out of levels 1 and 4
+constexpr int SP_CARRY = 32, SP_CARRY2 = 64;
+// carries of the level sums s[level][0..N-1] after the 16 columns from k0 of n that are summed before the
+// join (which needs none), higher levels first: they do not wait for one another. Measured against
+// none: step of a 28M-point array 69.3 -> 70.0 ms, operator of a 128 x 128 box (L = 155) 22.8 -> 23.4 us,
+// of a 509 x 333 box 113.1 -> 110.6 us (level 4 every 32 columns as well: half a percent more).
+template <int N>
+FC_HD void sp_carries(float (&s)[SP_DIGITS][N], int k0, int n) {
+  if ((k0 & (SP_CARRY - 16)) == 0 || k0 + 16 >= n) return;
+  const bool both = (k0 & (SP_CARRY2 - 16)) == SP_CARRY2 - 16;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int q = 0; q < N; ++q) {
+    if (both) sp_carry(s[0][q], s[1][q]);
+    sp_carry(s[1][q], s[2][q]);
+    sp_carry(s[2][q], s[3][q]);
+    if (both) sp_carry(s[3][q], s[4][q]);
+  }
+}
+
+// joined sum of the six level sums (integers below 2^28) in units 2^SP_UNIT
 FC_HD long long sp_join(const int* s) {
   const long long hi = ((long long)s[0] << 20) + ((long long)s[1] << 10) + s[2];
   const long long lo = ((long long)s[3] << 20) + ((long long)s[4] << 10) + s[5];

@@ -8,6 +8,15 @@
 //     "L op kind error/max|x| largest_level_sum" (op 0: derivative, 1: filter; the error also over
 //     the largest sigma), or "L none" when lines of this length are left to the FFT kernels.
 //
+//   contraction_host aligned L1 L2 ...
+//     the derivative and the filter of lines whose digits carry the signs of one row's coefficients,
+//     so that one level's sum is as large as it can be, summed in FP32 as the matrix
+//     instruction does, with the carries between levels; prints "L op level part error/max|x|
+//     largest_sum_of_levels_0_to_3".
+//
+//   contraction_host tables L1 L2 ...
+//     prints "L derivative filter": whether the tables exist (alpha = 10, p = 14).
+//
 //   contraction_host continuation C Q
 //     the continuation's digit products (mm_continuation, fragments read back as the matrix
 //     instruction does) for a matrix whose columns differ in size, on end values that differ,
@@ -108,7 +117,120 @@ static int continuation(int C, int Q) {
   return 0;
 }
 
+static std::vector<long double> default_sigma(int L) {
+  std::vector<long double> sig;
+  for (int k = 0; 2 * k <= L; ++k) sig.push_back(expl(-10.0L * powl(2.0L * k / L, 14)));
+  return sig;
+}
+
+static int tables(int n, char** v) {
+  for (int a = 0; a < n; ++a) {
+    const int L = std::atoi(v[a]);
+    std::vector<uint4> lo;
+    std::vector<uint2> hi;
+    const std::vector<long double> sig = default_sigma(L);
+    const MmPlan p = mm_plan(L, &sig, lo, hi);
+    printf("%d %d %d\n", L, p.dtab >= 0, p.ftab >= 0);
+  }
+  return 0;
+}
+
+static int aligned(int n, char** v) {
+  std::mt19937_64 g(5);
+  const long double PI = 3.14159265358979323846264338327950288L;
+  for (int a = 0; a < n; ++a) {
+    const int L = std::atoi(v[a]);
+    std::vector<uint4> lo;
+    std::vector<uint2> hi;
+    const std::vector<long double> sig = default_sigma(L);
+    const MmPlan p = mm_plan(L, &sig, lo, hi);
+    for (int op = 0; op < 2; ++op) {
+      const int te = op ? p.fte : p.dte, tab = op ? p.ftab : p.dtab;
+      std::vector<long double> c(L);  // the circulant
+      for (int m = 0; m < L; ++m) {
+        long double s = op ? sig[0] : 0.0L;
+        for (int k = 1; 2 * k <= L; ++k) {
+          const long double an = 2.0L * PI * ((long long)k * m % L) / L;
+          if (op == 0)
+            s += 2 * k < L ? -2.0L * (2.0L * PI * k / L) * sinl(an) : 0.0L;
+          else
+            s += (2 * k < L ? 2.0L : 1.0L) * sig[k] * cosl(an);
+        }
+        c[m] = s / L;
+      }
+      auto coef = [&](int s, int at, int* d) {
+        const int e = tab + s * p.nx + at;
+        const unsigned w[SP_DIGITS] = {lo[e].x, lo[e].y, lo[e].z, lo[e].w, hi[e].x, hi[e].y};
+        for (int u = 0; u < SP_DIGITS; ++u) d[u] = (int)half_value(w[u] & 0xffff);
+      };
+      for (int level = 1; level < 4; ++level)
+        for (int part = 0; part < p.S; ++part) {
+          const int row = (int)(g() % p.H);
+          std::vector<double> x(L, 0.0);
+          for (int k = 0; k < p.H; ++k) {
+            int d[SP_DIGITS];
+            coef(part, k - row + p.Mp, d);
+            long long val = 0;
+            for (int j = 0; j < SP_DIGITS - 1; ++j) {
+              const int big = j ? 511 : 127 * p.S, any = (int)(g() % (2 * big + 1)) - big;
+              val += (long long)(j <= level ? (d[level - j] < 0 ? -big : big) : any) << (SP_BITS * (SP_DIGITS - 1 - j));
+            }
+            const long long h = p.S == 2 ? val / 2 : val;
+            x[k] = std::ldexp((double)h, -57);
+            if (p.S == 2) x[k + p.H] = std::ldexp((double)(part ? h - val : val - h), -57);
+          }
+          double top = 0;
+          for (double y : x) top = std::max(top, std::fabs(y));
+          const int ex = (int)((sp_hi(top) >> 20) & 0x7ff);
+          std::vector<long long> W[2];
+          double largest = 0;
+          for (int s = 0; s < p.S; ++s)
+            for (int i = 0; i < p.H; ++i) {
+              unsigned long long joined = 0;
+              for (int kb = 0; kb < p.Kp; kb += MM_KCHUNK) {
+                float acc[SP_DIGITS][1] = {};
+                const int nk = std::min(p.Kp - kb, MM_KCHUNK);
+                for (int k0 = 0; k0 < nk; k0 += 16) {
+                  double step[SP_DIGITS][SP_DIGITS] = {};
+                  for (int k = kb + k0; k < std::min(p.H, kb + k0 + 16); ++k) {
+                    const long long x0 = sp_fixed(x[k], ex), x1 = p.S == 2 ? sp_fixed(x[k + p.H], ex) : 0;
+                    const long long b = (s ? x0 - x1 : x0 + x1) + SP_BIAS;
+                    int d[SP_DIGITS];
+                    coef(s, k - i + p.Mp, d);
+                    for (int u = 0; u < SP_DIGITS; ++u)
+                      for (int w = 0; u + w < SP_DIGITS; ++w) step[u][w] += (double)d[u] * ((int)sp_field(b, w) - 512);
+                  }
+                  for (int w = 0; w < SP_DIGITS; ++w)
+                    for (int u = 0; u + w < SP_DIGITS; ++u) {
+                      acc[u + w][0] = (float)(acc[u + w][0] + step[u][w]);
+                      if (u + w < 4) largest = std::max(largest, (double)std::fabs(acc[u + w][0]));
+                    }
+                  sp_carries(acc, k0, nk);
+                }
+                int si[SP_DIGITS];
+                for (int l = 0; l < SP_DIGITS; ++l) si[l] = (int)acc[l][0];
+                joined += (unsigned long long)sp_join(si);
+              }
+              W[s].push_back((long long)joined);
+            }
+          const double fac = std::scalbn(1.0, ex - 1023 - SP_DATA + SP_UNIT - te - (p.S - 1));
+          double err = 0;
+          for (int i = 0; i < L; ++i) {
+            const long long y = p.S == 1 ? W[0][i] : (i < p.H ? W[0][i] + W[1][i] : W[0][i - p.H] - W[1][i - p.H]);
+            long double ref = 0;
+            for (int j = 0; j < L; ++j) ref += c[((i - j) % L + L) % L] * (long double)x[j];
+            err = std::max(err, (double)fabsl((long double)sp_double(y) * fac - ref));
+          }
+          printf("%d %d %d %d %.3e %.0f\n", L, op, level, part, err / top, largest);
+        }
+    }
+  }
+  return 0;
+}
+
 int main(int argc, char** argv) {
+  if (argc > 2 && !std::strcmp(argv[1], "aligned")) return aligned(argc - 2, argv + 2);
+  if (argc > 2 && !std::strcmp(argv[1], "tables")) return tables(argc - 2, argv + 2);
   if (argc == 4 && !std::strcmp(argv[1], "continuation")) return continuation(std::atoi(argv[2]), std::atoi(argv[3]));
   if (argc == 2 && !std::strcmp(argv[1], "quotient")) return quotients();
   std::mt19937_64 g(1);

@@ -45,6 +45,27 @@ def test_contraction_matches_the_circulant(exe):
         assert float(level) < 2 ** 24, (L, op, kind, level)
 
 
+def test_level_sums_are_exact_for_aligned_data(exe):
+    """Lines made so that one of the levels 1 to 3 is as large as it can be. The bound of the module's
+    head; results are up to 14 times the largest value here (the derivative's coefficients sum
+    to that), so their own FP64 rounding counts 8 times: 2^-50.5 + 2^-50 (levels 4 and 5, whose
+    digits are random here, stay exact)."""
+    r = subprocess.run([exe, "aligned", "17", "30", "64", "155", "256", "400", "509", "510", "512", "800", "1024"],
+                       capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0, r.stderr
+    rows = [ln.split() for ln in r.stdout.splitlines()]
+    assert len(rows) == 3 * 6 + 8 * 12
+    for L, op, level, part, err, largest in rows:
+        assert float(largest) < 2 ** 24, (L, op, level, part, largest)
+        assert float(err) < 2.0 ** -50.5 + 2.0 ** -50, (L, op, level, part, err)
+
+
+def test_every_length_has_exact_tables(exe):
+    lengths = [L for L in range(16, 1025) if L % 2 == 0 or L <= 512]
+    r = subprocess.run([exe, "tables", *map(str, lengths)], capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0 and [ln.split() for ln in r.stdout.splitlines()] == [[str(L), "1", "1"] for L in lengths]
+
+
 # broad kernels (many coefficients of one size), an amplifying one, small ones throughout; p = 0
 # scales all modes alike
 @pytest.mark.parametrize("alpha,p", [(2000, 2), (1700, 2), (50, 1), (1e6, 4), (0, 2), (-5, 2), (10, 0), (10, -1)])
