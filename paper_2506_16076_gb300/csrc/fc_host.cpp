@@ -142,6 +142,7 @@ struct fc_ctx {
     uint8_t* dvisc = nullptr;                    // their viscous flags (valid while ctx::flags_on)
     int ntiles = 0;                              // per order
     bool filter = false;                         // the filter's lines (contracted with the filter's table)
+    std::vector<uint8_t> fft;                    // per plan: long_lines_to_fft (of the whole workload's lines)
     std::unique_ptr<Queue> rest;
   };
   Queue q_cart1, q_cart2, q_gen1, q_gen2, q_filt1, q_filt2;
@@ -1004,6 +1005,50 @@ struct Builder {
 void make_queue(fc_ctx* c, fc_ctx::Queue& q, std::vector<Job>& jobs, const std::vector<Plan>& plans, int npatch,
                 bool& ok, const std::vector<MmPlan>* mm);
 
+// Long even lines (L > 736) on the FFT kernels where their contraction would fill less than half of
+// a second wave. Such a tile takes a whole SM, so 153 tiles (609 lines) take as long as 304, while the
+// FFT kernels hold a warp per line and 6 to 8 of them on an SM. Measured per pass, q1 lines, FFT / contraction
+// (us, two rounds): L = 1024: 600 lines 432/347, 613 464/678, 898 509/685, 1098 885/686; L = 896: 613
+// lines 446/557, 898 485/563, 1098 835/565; L = 768: 350/397, 389/401, 472/403; shorter and odd lines
+// are contracted at least as fast at any number (L = 720: 411/381). The estimates below are of one round:
+// a tile's time by its padded inner length, a transform's by lane_cost and the lines of an SM, both within
+// 6% of the measured times. Other tiles of the queue fill the second wave, so their time counts. The
+// choice looks at all lines of the workload once: sharded and per-patch runs make the same one.
+void long_lines_to_fft(fc_ctx::Queue& q, const std::vector<Job>& jobs, const std::vector<Plan>& plans,
+                       const std::vector<MmPlan>& mm) {
+  constexpr int SMS = 152, LONG = 368;
+  q.fft.assign(plans.size(), 0);
+  auto tile_us = [](const MmPlan& m) {
+    const double k = m.Kp;
+    const double t = k <= 256 ? 7.2e-4 * k * k : (k <= 384 ? 0.267 * k : 124.0 + 0.4286 * (k - 400.0));
+    return m.S == 2 ? t : 0.5 * t;
+  };
+  long long lines = 0;
+  double other = 0, tile = 0, cost = 0;  // SM time of the other tiles; the largest of the long lines
+  int Lmax = 0;
+  for (const Job& J : jobs) {
+    const MmPlan& m = mm[J.plan];
+    if (m.H == 0) continue;
+    if (m.S == 2 && m.Kp > LONG) {
+      const Plan& p = plans[J.plan];
+      ++lines;
+      Lmax = std::max(Lmax, p.L);
+      tile = std::max(tile, tile_us(m));
+      const std::vector<int> rad(p.rad, p.rad + p.nst);
+      if (*std::max_element(rad.begin(), rad.end()) > 8) return;  // a generic stage: slower by far
+      cost = std::max(cost, (double)lane_cost(p.L, rad));
+    } else {
+      other += tile_us(m) / (MM_LINES * SMS);
+    }
+  }
+  const long long per_sm = (lines + SMS - 1) / SMS, resident = 232448 / ((2 * Lmax + CONT_TMP) * 16 + 1024);
+  if (lines <= MM_LINES * SMS || per_sm > 6 || per_sm > resident) return;
+  const double mm_us = std::max(2 * tile, lines * tile / (MM_LINES * SMS) + other);
+  const double fft_us = cost * (per_sm <= 5 ? 3.9e-3 : 4.2e-3) + other;
+  if (fft_us < 0.94 * mm_us)
+    for (size_t k = 0; k < mm.size(); ++k) q.fft[k] = mm[k].S == 2 && mm[k].Kp > LONG;
+}
+
 // Tiles of the contraction kernels from a queue's per-patch order pp; the lines of other
 // lengths go to q.rest. Launch classes by padded inner length: the shared memory of a CTA
 // grows with it, so a class has the lengths that let the same number of CTAs share an SM.
@@ -1017,9 +1062,10 @@ void make_tiles(fc_ctx* c, fc_ctx::Queue& q, const std::vector<Job>& pp, const s
   constexpr int MM_FEW = 304;
   std::vector<Tile> tiles;
   std::vector<Job> rest;
+  if (q.fft.empty()) long_lines_to_fft(q, pp, plans, mm);
   for (const Job& J : pp) {
     const MmPlan& m = mm[J.plan];
-    if (m.H == 0 || J.C > MM_CMAX || c->d > 8 || (q.filter ? m.ftab : m.dtab) < 0) {
+    if (m.H == 0 || J.C > MM_CMAX || c->d > 8 || (q.filter ? m.ftab : m.dtab) < 0 || q.fft[J.plan]) {
       rest.push_back(J);
       continue;
     }
