@@ -203,12 +203,14 @@ fc_status fc_rk_step_host(fc_ctx *ctx, double *e_host, double *dt_dev, double *m
 /* fc_autotune flags */
 enum { FC_TUNE_PLANS = 1, FC_TUNE_WARPS = 2 };
 /* Measured schedule choice for this context's lines (no paper counterpart: the paper's
- * CPU code has no launch schedule). FC_TUNE_PLANS: for every continued length L, the
- * stage orders of the FFT with the smallest modelled cost (up to 4, power-of-two radices
- * first) are each timed on that length's own lines and the fastest kept (if at least 1%
- * faster than the model's choice and its output agrees with it to 1e-10 relative).
- * FC_TUNE_WARPS: for every power-of-two length class, 1, 2, 4 or 8 warps per CTA, timed
- * on the class's q1 and q2 lines. The choices change rounding only, never the method.
+ * CPU code has no launch schedule). FC_TUNE_PLANS: for every continued length L that runs
+ * as FFTs somewhere, the stage orders with the smallest modelled cost (up to 4, power-of-two
+ * radices first) are each timed on that length's own lines and the fastest kept (if at least 1%
+ * faster than the model's choice and its output agrees with it to 1e-10 relative); a length
+ * that runs as contractions only is examined and has nothing to choose. FC_TUNE_WARPS: for
+ * every power-of-two length class of the FFT lines, 1, 2, 4 or 8 warps per CTA, timed on the
+ * class's q1 and q2 lines; every launch class of contracted q1 and q2 lines is examined and
+ * timed as it runs. The choices change rounding only, never the method.
  * Synchronises `stream`, overwrites the context's scratch (stage buffers, R1, its
  * internal mu), invalidates a captured step graph (the next FC_STEP_GRAPH step captures
  * again) and allocates 1 MB of device memory on its first call. report (nullable, 6 host doubles):

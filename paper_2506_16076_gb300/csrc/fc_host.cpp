@@ -2436,12 +2436,12 @@ fc_status fc_autotune(fc_ctx* c, int flags, double* report, void* stream) {
   constexpr int MAXT = 16384, MINT = 2048, REPS = 3;
   if (!c->d_tune_jobs && !c->alloc(&c->d_tune_jobs, MAXT)) return fail(c, FC_ERR_OOM, c->err);
   Job* d_tj = c->d_tune_jobs;
-  auto time_q1 = [&](const Job* jobs, int n, int Lmax) {
-    launch_cart_q1(c->T, jobs, n, Lmax, e, c->d_mu, c->d_R1, c->d_Fy, st);  // warm-up
+  auto timed = [&](auto&& launch) {
+    launch();  // warm-up
     float best = 1e30f;
     for (int r = 0; r < REPS; ++r) {
       cudaEventRecord(ea, st);
-      launch_cart_q1(c->T, jobs, n, Lmax, e, c->d_mu, c->d_R1, c->d_Fy, st);
+      launch();
       cudaEventRecord(eb, st);
       cudaEventSynchronize(eb);
       float ms = 0.f;
@@ -2449,6 +2449,9 @@ fc_status fc_autotune(fc_ctx* c, int flags, double* report, void* stream) {
       best = std::min(best, ms);
     }
     return (double)best;
+  };
+  auto time_q1 = [&](const Job* jobs, int n, int Lmax) {
+    return timed([&] { launch_cart_q1(c->T, jobs, n, Lmax, e, c->d_mu, c->d_R1, c->d_Fy, st); });
   };
   // R1 of the first timed line, 4 components (strided copy)
   auto sample = [&](const Job& J, std::vector<double>& out) {
@@ -2459,19 +2462,27 @@ fc_status fc_autotune(fc_ctx* c, int flags, double* report, void* stream) {
     cudaStreamSynchronize(st);
   };
   fc_status status = FC_OK;
+  // the lines that the FFT kernels run: those the contraction kernels leave, and the lines of the
+  // product-rule wall form, whose adjoint pass B has the FFT form only
+  std::vector<std::vector<Job>> fft;
+  for (const fc_ctx::Queue* q : {&c->q_cart1, &c->q_cart2, &c->q_gen1, &c->q_gen2, &c->q_filt1, &c->q_filt2})
+    fft.push_back(q->rest->h);
+  if (c->T.any_pform) fft.push_back(c->q_gen2.h);
   // (1) stage order of each continued length, timed on that length's lines
   if (flags & FC_TUNE_PLANS) {
-    const fc_ctx::Queue* qs[6] = {&c->q_cart1, &c->q_cart2, &c->q_gen1, &c->q_gen2, &c->q_filt1, &c->q_filt2};
     for (size_t pi = 0; pi < c->plans_h.size() && status == FC_OK; ++pi) {
       const std::vector<Plan>& cand = c->plan_cands[pi];
-      if (cand.size() < 2) continue;
       std::vector<Job> base;
-      for (const fc_ctx::Queue* q : qs) {
-        for (const Job& J : q->h)
+      for (const std::vector<Job>& v : fft) {
+        for (const Job& J : v)
           if (J.plan == (int)pi) base.push_back(J);
         if (!base.empty()) break;  // the first pass with lines of this length
       }
-      if (base.empty()) continue;
+      if (base.empty()) {  // contracted throughout: nothing to choose
+        rep[0] += 1;
+        continue;
+      }
+      if (cand.size() < 2) continue;
       std::vector<Job> tj;
       while ((int)tj.size() < MINT)
         for (const Job& J : base) {
@@ -2512,10 +2523,28 @@ fc_status fc_autotune(fc_ctx* c, int flags, double* report, void* stream) {
       if (cudaGetLastError() != cudaSuccess) status = cuda_check(c, "fc_autotune (plans)");
     }
   }
-  // (2) warps per CTA of each length class, timed on the class's q1 and q2 lines
+  // (2) warps per CTA of each length class, timed on the class's q1 and q2 lines; the contraction
+  // kernels' launches, whose shape follows from their sizes, are timed as they are
   if ((flags & FC_TUNE_WARPS) && status == FC_OK) {
+    StageCoef sc{};
+    sc.Ucur = e;
+    sc.out = c->d_B2;
+    sc.rhs_only = 1;
+    for (int dir = 0; dir < 2; ++dir)
+      for (MmTiles m : (dir ? c->q_cart2 : c->q_cart1).mm) {
+        m.visc = nullptr;  // flags belong to another mu
+        const double t = timed([&] {
+          if (dir)
+            launch_mm_cart_q2(c->T, m, c->d_mu, c->d_R1, c->d_Fy, sc, st);
+          else
+            launch_mm_cart_q1(c->T, m, e, c->d_mu, c->d_R1, c->d_Fy, st);
+        });
+        rep[2] += 1;
+        rep[4] += t;
+        rep[5] += t;
+      }
     std::map<int, std::vector<std::pair<const fc_ctx::Queue*, int>>> byclass;  // class -> (queue, class slot)
-    for (const fc_ctx::Queue* q : {&c->q_cart1, &c->q_cart2})
+    for (const fc_ctx::Queue* q : {c->q_cart1.rest.get(), c->q_cart2.rest.get()})
       for (size_t k = 0; k < q->classes.size(); ++k) byclass[length_class(q->classes[k].second)].push_back({q, (int)k});
     for (auto& kv : byclass) {
       const int cls = kv.first;

@@ -107,3 +107,19 @@ def test_tuning_on_a_side_stream(gpu_lib):
     torch.cuda.synchronize()
     errs = rel_err(from_dev(out, w), ref)
     assert max(errs) < 1e-11, errs
+
+
+def _box(n1, n2):
+    fs = (1.4, 1.0, 0.3, 1.0)
+    p = W.PatchDesc(W.AFFINE, n1, n2, (0.0, 1.0, 0.0, 0.7), (W.DIRICHLET,) * 4, bc=(fs,) * 4)
+    return W.Workload(f"box_{n1}x{n2}", [p], W.Params(c_policy=0), fs, "freestream", 1)
+
+
+def test_report_covers_the_launches_of_a_step(gpu_lib):
+    # one continued length, contracted in both directions: one launch each, nothing to choose
+    rep = gpu_lib.Context(_box(101, 101)).autotune()
+    assert (rep["lengths"], rep["lengths_changed"], rep["classes"], rep["classes_changed"]) == (1, 0, 2, 0)
+    assert 0.0 < rep["ms_after"] == rep["ms_before"]
+    # q1 lines of 2025 + 27 = 2052 points stay on the FFT kernels, q2 lines are contracted
+    rep = gpu_lib.Context(_box(2025, 101)).autotune()
+    assert (rep["lengths"], rep["classes"]) == (2, 2)
