@@ -7,9 +7,9 @@ class), captured once as a CUDA graph and replayed. A point-update is one active
 (non-blanked) grid point receiving one RHS evaluation, so a step is 5 x active
 points point-updates.
 
-Before timing, fc_autotune times the candidate FFT stage orders of every continued
-length and the warps per CTA of every length class on the workload's own lines and
-keeps the fastest (--no-autotune: the cost model's choices).
+Before timing, fc_autotune times the candidate FFT stage orders and the warps per CTA of the
+lines that run as transforms and keeps the fastest (--no-autotune: the cost model's
+choices); on the default workload all lines are contracted and it has nothing to choose.
 
   python bench.py [--gpus N --steps K --warmup W --workload NAME --impl ours|reference]
 
@@ -241,7 +241,11 @@ def peaks():
 
 # the kernels and the host code that chooses their plans and launch shapes
 KERNEL_SOURCES = ["fc_kernels.cu", "fc_line.cuh", "fc_internal.h", "fc_host.cpp", "fc_tables.h", "fc_mma.cuh", "fc_mma.cu",
-                  "fc_point.cuh", "fc_split.cuh", "fc_mmtab.h"]
+                  "fc_mma_gen.cu", "fc_mma_adj.cu", "fc_mma_adj_gen.cu", "fc_point.cuh", "fc_split.cuh", "fc_mmtab.h"]
+
+# operations that a line pass leaves to the FP64 pipe, per point and per point of a gradient round (fluxes
+# or stage combination, the filter's pointwise maps, the lines' scale; a reciprocal counts as six)
+FP64_OPS = {"cart_q1": (22, 8), "cart_q2": (22, 8), "filter_q1": (17, 0), "filter_q2": (17, 0)}
 
 
 def kernel_sources_sha():
@@ -473,43 +477,43 @@ def main_ours(args):
             dist.destroy_process_group()
         return
 
-    # roofline of the dominant kernel (work by the FP64 FFT count, against the FP64 pipe)
+    # roofline of the dominant line pass: what its kernels do on the three pipes that could bound it
     pk = peaks()
-    dom = max((k for k in prof if k in ("cart_q1", "cart_q2", "filter_q1", "filter_q2")),
-              key=lambda k: prof[k][0], default=None)
+    dom = max((k for k in prof if k in FP64_OPS), key=lambda k: prof[k][0], default=None)
     roof = None
     if dom:
-        flops, nbytes, nl, npts = ctx.pass_stats(dom)
+        _, nbytes, nl, npts = ctx.pass_stats(dom)
+        products, transformed = ctx.pass_products(dom)
         tot_ms, cnt = prof[dom]
-        passes_prof = 2 * (5 if dom.startswith("cart") else 1)
-        # gradient rounds skipped on lines with mu == 0 everywhere are not counted as work done
-        skipped = {"cart_q1": skip[2], "cart_q2": skip[3]}.get(dom, 0.0) / passes_prof
-        skipped_lines = {"cart_q1": skip[0], "cart_q2": skip[1]}.get(dom, 0) / passes_prof
-        flops_full = flops
-        flops = flops - skipped
-        avg_s = tot_ms / 1e3 / max(cnt, 1)
-        # one pass launch group covers all its length classes; flops above are per full pass
-        groups = cnt
+        # one pass launch group covers all its length classes
         passes = 2 * (5 if dom.startswith("cart") else 1)  # profiled 2 steps
-        avg_pass_s = tot_ms / 1e3 / passes
+        avg_s = tot_ms / 1e3 / passes
+        # the gradient round is skipped on lines whose tile has mu == 0 everywhere
+        skipped = {"cart_q1": skip[0], "cart_q2": skip[1]}.get(dom, 0) / passes
+        viscous = 1.0 - skipped / max(nl, 1)
+        rounds = (1.0 + viscous) / 2.0 if dom.startswith("cart") else 1.0
+        ops, grad_ops = FP64_OPS[dom]
+        fp64_ops = npts * (ops + grad_ops * viscous)
         sm_max = pk.get("sm_max_mhz", 2070.0)
         n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
-        fp64_peak = n_sm * sm_max * 1e6 * 4 / 1e12  # 2 FP64 FMA lanes / clk / SM on GB300, TFLOP/s
-        ach = flops / avg_pass_s / 1e12
+        pipes = {  # name: (work per pass, peak per second, unit, scale of the unit)
+            "alu": (fp64_ops, n_sm * sm_max * 1e6 * 2, "T FP64 operations/s", 1e12),
+            "tensor": (products * rounds, pk.get("bf16_tflops", 1900.0) * 1e12, "TFLOP/s", 1e12),
+            "hbm": (nbytes, pk.get("hbm_gbs", 6787.9) * 1e9, "GB/s", 1e9)}
+        rates = {k: {"work_per_pass": wk, "achieved": round(wk / avg_s / sc, 4), "peak": round(top / sc, 4), "unit": u,
+                     "frac": round(wk / avg_s / top, 4)} for k, (wk, top, u, sc) in pipes.items()}
+        bound = max(rates, key=lambda k: rates[k]["frac"])
         kname = f"k_mm_{dom}"  # the kernel that takes the pass's lines of contracted lengths
-        roof = {"bound": "alu", "achieved": round(ach, 4), "peak": round(fp64_peak, 4), "unit": "TFLOP/s",
-                "frac": round(ach / fp64_peak, 4), "traffic": measured_traffic(kname, args.workload),
+        roof = {"bound": bound, **{k: rates[bound][k] for k in ("achieved", "peak", "unit", "frac")}, "pipes": rates,
+                "traffic": measured_traffic(kname, args.workload),
                 "traffic_unit": "DRAM bytes per pass (all length-class launches), ncu", "kernel": kname,
-                "algorithmic_bytes_per_pass": nbytes,
-                "lines_per_pass": nl, "inviscid_lines_per_pass": skipped_lines,
-                "flops_per_pass_executed": flops, "flops_per_pass_all_rounds": flops_full,
-                "pass_ms": round(avg_pass_s * 1e3, 3), "launches_per_pass": groups // passes,
-                "hbm_GBps": round(nbytes / avg_pass_s / 1e9, 1),
-                "hbm_frac_of_measured": round(nbytes / avg_pass_s / 1e9 / pk.get("hbm_gbs", 6787.9), 4),
-                "peak_note": f"FP64 unit count: {n_sm} SMs (device query) x 2 FMA lanes/clk x 2 flops x max SM "
-                             f"clock {sm_max:.0f} MHz",
-                "flops_note": "flops counted as the lines' FFTs in FP64 (5 L log2 L); the kernel forms them as exact "
-                              "digit products on the FP16 matrix pipe and FP64 pointwise work",
+                "algorithmic_bytes_per_pass": nbytes, "lines_per_pass": nl, "lines_as_transforms": transformed,
+                "inviscid_lines_per_pass": skipped, "pass_ms": round(avg_s * 1e3, 3),
+                "launches_per_pass": cnt // passes,
+                "note": f"alu: FP64 pipe, {n_sm} SMs (device query) x 2 operations/clk x max SM clock {sm_max:.0f} MHz; "
+                        "tensor: digit products at the measured bf16 rate (FP16 has the same; mma.sync does not reach it); "
+                        "hbm: compulsory bytes at the measured copy rate. No pipe is full: latencies between a tile's "
+                        "phases set the pace",
                 "probe_TFLOPs": None if probe is None else {"dfma": round(probe[0] / 1e3, 4),
                                                             "dmma": round(probe[1] / 1e3, 4),
                                                             "source": "fc_probe_fp64, this run"}}

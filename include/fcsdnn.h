@@ -294,6 +294,12 @@ fc_status fc_line_stats(fc_ctx *ctx, long long *lines_q1, long long *lines_q2, d
 fc_status fc_pass_stats(const fc_ctx *ctx, const char *pass, double *flops, double *bytes, long long *lines,
                         long long *points);
 
+/* The matrix work of one launch of such a pass: FP16 flops of the digit products of its contracted
+ * lines (2 per product, 21 digit pairs per coefficient and value, both derivative rounds), and the
+ * number of its lines that run as transforms instead. Used to place a measured duration on the
+ * matrix pipe's roofline. */
+fc_status fc_pass_products(const fc_ctx *ctx, const char *pass, double *flops, long long *transformed);
+
 /* ---- Sharded execution over several ranks (one GPU per rank) ----
  * The patches are the unit of work: a rank advances only the patches it owns, and the
  * operator couples patches only through the inter-patch exchange of every projection

@@ -141,6 +141,7 @@ struct fc_ctx {
     Job* dmm = nullptr;                          // all tiles' jobs: per patch, then batched
     uint8_t* dvisc = nullptr;                    // their viscous flags (valid while ctx::flags_on)
     int ntiles = 0;                              // per order
+    double products = 0;                         // FP16 flops of a round's digit products, all tiles
     bool filter = false;                         // the filter's lines (contracted with the filter's table)
     std::vector<uint8_t> fft;                    // per plan: long_lines_to_fft (of the whole workload's lines)
     std::unique_ptr<Queue> rest;
@@ -1087,6 +1088,12 @@ void make_tiles(fc_ctx* c, fc_ctx::Queue& q, const std::vector<Job>& pp, const s
     while (top[t.cls] < t.kp) ++t.cls;
     tiles.push_back(t);
   }
+  q.products = 0;
+  for (const Tile& t : tiles)
+    for (const Job& J : t.j) {
+      const MmPlan& m = mm[t.j[0].plan];
+      if (J.n > 0) q.products += 2.0 * 21 * 4 * ((double)m.S * m.H * m.H + (J.fcm >= 0 ? 16.0 * J.C : 0.0));
+    }
   for (Tile& t : tiles)  // absent lines: the first one's addresses (read, never written) and no points
     for (int l = 1; l < MM_LINES; ++l)
       if (t.j[l].n == 0) {
@@ -2727,6 +2734,20 @@ fc_status fc_pass_stats(const fc_ctx* c, const char* pass, double* flops, double
   *bytes = Bt;
   *lines = nl;
   *points = np;
+  return FC_OK;
+}
+
+fc_status fc_pass_products(const fc_ctx* c, const char* pass, double* flops, long long* transformed) {
+  if (!c || !pass || !flops || !transformed) return FC_ERR_INVALID;
+  const std::string n(pass);
+  const fc_ctx::Queue* q = n == "cart_q1"     ? &c->q_cart1
+                           : n == "cart_q2"   ? &c->q_cart2
+                           : n == "filter_q1" ? &c->q_filt1
+                           : n == "filter_q2" ? &c->q_filt2
+                                              : nullptr;
+  if (!q) return FC_ERR_INVALID;
+  *flops = (q->filter ? 1 : 2) * q->products;
+  *transformed = (long long)q->rest->h.size();
   return FC_OK;
 }
 

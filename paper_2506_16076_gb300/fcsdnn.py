@@ -29,7 +29,7 @@ EXPORTS = ["fc_init_patches", "fc_state_size", "fc_patch_offset", "fc_active_poi
            "fc_filter", "fc_project", "fc_timestep", "fc_rk_step", "fc_rk_step_host", "fc_autotune", "fc_adjoint_step",
            "fc_initial_sensitivity", "fc_drag", "fc_sync_status", "fc_partition", "fc_shard", "fc_shard_counts",
            "fc_launch_count", "fc_profile_enable", "fc_profile_read", "fc_profile_get", "fc_profile_reset",
-           "fc_pass_stats", "fc_line_stats", "fc_probe_fp64", "fc_rhs_patch_noalloc", "fc_last_error", "fc_destroy"]
+           "fc_pass_stats", "fc_pass_products", "fc_line_stats", "fc_probe_fp64", "fc_rhs_patch_noalloc", "fc_last_error", "fc_destroy"]
 
 
 class FcError(RuntimeError):
@@ -95,6 +95,7 @@ def load():
         "fc_profile_read": (C.c_int, [vp]),
         "fc_profile_get": (C.c_int, [vp, ip, C.POINTER(C.c_char_p), C.POINTER(C.c_double), C.POINTER(C.c_int)]),
         "fc_profile_reset": (C.c_int, [vp]),
+        "fc_pass_products": (C.c_int, [vp, C.c_char_p, C.POINTER(C.c_double), C.POINTER(C.c_longlong)]),
         "fc_pass_stats": (C.c_int, [vp, C.c_char_p, C.POINTER(C.c_double), C.POINTER(C.c_double),
                                     C.POINTER(C.c_longlong), C.POINTER(C.c_longlong)]),
         "fc_line_stats": (C.c_int, [vp, C.POINTER(C.c_longlong), C.POINTER(C.c_longlong), C.POINTER(C.c_double),
@@ -392,6 +393,12 @@ class Context:
         a, b, f, g = C.c_longlong(), C.c_longlong(), C.c_double(), C.c_double()
         self._check(self.lib.fc_line_stats(self.ctx, C.byref(a), C.byref(b), C.byref(f), C.byref(g), 1 if reset else 0))
         return a.value, b.value, f.value, g.value
+
+    def pass_products(self, name):
+        """(FP16 matrix flops of the digit products, lines that run as transforms) of one launch of a line pass."""
+        f, nl = C.c_double(), C.c_longlong()
+        self._check(self.lib.fc_pass_products(self.ctx, name.encode(), C.byref(f), C.byref(nl)))
+        return f.value, nl.value
 
     def profile_reset(self):
         self._check(self.lib.fc_profile_reset(self.ctx))

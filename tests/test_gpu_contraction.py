@@ -168,3 +168,15 @@ def test_viscosity_of_a_scaled_state_has_the_same_bits(gpu_lib, k):
     ctx.viscosity(e * 2.0**k, mu_s, tau_s)
     assert int(tau.min()) < int(tau.max()) and float(mu.max()) > 0.0
     assert torch.equal(tau, tau_s) and torch.equal(mu, mu_s)
+
+
+def test_pass_products_count_the_contracted_lines(gpu_lib):
+    # L = 128 = 2 x 64 along both directions: 21 digit pairs, 2 parts of 64 x 64 and 16 columns of 27
+    # continuation points, 4 components
+    per_line = 2 * 21 * 4 * (2 * 64 * 64 + 16 * 27)
+    ctx = gpu_lib.Context(_box(101, 101))
+    assert ctx.pass_products("cart_q2") == (2 * 101 * per_line, 0)
+    assert ctx.pass_products("filter_q1") == (101 * per_line, 0)
+    # 2025 + 27 points: transforms
+    ctx = gpu_lib.Context(_box(2025, 101))
+    assert ctx.pass_products("cart_q1") == (0.0, 101) and ctx.pass_products("cart_q2") == (2 * 2025 * per_line, 0)
