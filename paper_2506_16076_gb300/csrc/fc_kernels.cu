@@ -3,8 +3,9 @@
 // Line kernels: one warp per grid-line segment, shared-memory mixed-radix Stockham
 // FFTs of the FC-Gram continued line (Sec. 2.2), fused with the Euler flux, the
 // artificial-viscosity flux and the SSPRK stage combination (Sec. 2.1, 2.3, 4.1). They
-// take the lines whose continued length the contraction kernels (fc_mma.cuh) do not: these
-// are twice as fast up to 1024 points. The FFT form is bound by the FP64 pipe (2 FP64
+// take the lines that the contraction kernels (fc_mma.cuh), about twice as fast up to 700 points, do
+// not: longer ones than 1024, odd ones above 512, and long ones whose tiles would leave half of a
+// wave empty (long_lines_to_fft in fc_host.cpp). The FFT form is bound by the FP64 pipe (2 FP64
 // lanes/clk/SM on GB300), so it minimises FP64 instructions: packed real pairs per complex
 // FFT, radix 2/3/4/5/7/8 butterflies with table twiddles, continuation as a 2d-term matvec.
 #include <cuda_runtime.h>

@@ -1,10 +1,10 @@
 // FC line operators as exact tensor-core contractions (fc_split.cuh, fc_mmtab.h).
 //
-// GB300 executes 2 FP64 FMAs per clock and SM but 1024 FP16 ones through mma.sync (measured
-// 600 TFLOP/s), so the circulant of a continued line (21 FP16 digit products per entry,
-// L^2/2 entries per line) costs less time than the FP64 butterflies of its two FFTs up to
-// lengths of a few hundred. What a line still needs from the FP64 pipe is its pointwise
-// work: fluxes and stage combination.
+// GB300 executes 2 FP64 FMAs per clock and SM but about 1000 FP16 ones through mma.sync
+// (profiles/mma_sync_probe.md), so the circulant of a continued line (21 FP16 digit products per
+// entry, L^2/2 entries per line) costs less time than the FP64 butterflies of its two FFTs, by a
+// factor of 2 at a few hundred points and about as much as them at 1024. What a line still needs
+// from the FP64 pipe is its pointwise work: fluxes and stage combination.
 //
 // A CTA takes MM_LINES lines of one length (16 columns: 4 lines x 4 components): their values
 // go to shared memory with lanes along the points, are continued there, and are replaced by
@@ -15,9 +15,9 @@
 // table of 24 bytes per entry). Digits need 12 bytes per point, component and part; 24
 // accumulators per lane leave room for 24 warps per SM at 80 registers.
 //
-// Measured (28M points, affine lines of 48 to 384 points, per pass, FFT kernels -> 16 warps of
-// 16 columns each -> now): q1 9.6 -> 4.4 -> 3.7 ms, q2 10.0 -> 6.0 -> 5.1 ms, filter q1 + q2
-// 17.5 -> 8.0 -> 6.6 ms; a 128 x 128 operator with L = 155 = 5 x 31: 462 -> 23 us. Largest
+// Measured (28M points, affine lines of 48 to 384 points, per pass, FFT kernels -> these): q1 9.6
+// -> 3.5 ms, q2 10.0 -> 5.0 ms, filter q1 + q2 17.5 -> 6.4 ms; a 128 x 128 operator with
+// L = 155 = 5 x 31: 462 -> 23 us. Largest
 // error on white lines 2.4e-16 of the largest value (FP64 FFT: 6e-16 to 9e-16). No pipe is
 // full (FP64 and matrix pipes 15% to 39% busy): fixed latencies of the integer chains
 // and the barriers between a tile's phases are what is left; 64 registers and 32 warps gained
@@ -73,7 +73,7 @@ __device__ __forceinline__ void ldsm4(uint32_t* r, uint32_t addr) {
                : "r"(addr));
 }
 
-// table entries stay in L1 (every warp of the SM reads them), the lines' data pass by it
+// table entries stay in L1 (every warp of the SM reads them)
 __device__ __forceinline__ uint4 ldg_keep(const uint4* p) {
   uint4 v;
   asm volatile("ld.global.nc.L1::evict_last.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -84,11 +84,6 @@ __device__ __forceinline__ uint4 ldg_keep(const uint4* p) {
 __device__ __forceinline__ uint2 ldg_keep(const uint2* p) {
   uint2 v;
   asm volatile("ld.global.nc.L1::evict_last.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ double ld_pass(const double* p) {
-  double v;
-  asm volatile("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
   return v;
 }
 

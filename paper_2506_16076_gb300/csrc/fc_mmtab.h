@@ -26,7 +26,7 @@ namespace fcx {
 // whether lines of continued length L run as contractions: the parts' inner length fits a CTA
 inline bool mm_length_ok(int L) { return L >= 16 && ((L % 2 == 0 && L / 2 <= MM_KMAX) || (L % 2 == 1 && L <= MM_KMAX)); }
 
-// FP16 bits of an integer in [-2048, 2048]
+// FP16 bits of an integer of magnitude below 2048
 inline uint16_t mm_half(int v) {
   if (v == 0) return 0;
   const int a = v < 0 ? -v : v;

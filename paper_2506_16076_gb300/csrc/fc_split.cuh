@@ -32,7 +32,7 @@ namespace fcx {
 constexpr int SP_DIGITS = 6;     // digits per value = accumulation levels
 constexpr int SP_BITS = 10;      // bits per digit
 constexpr int SP_DATA = 56;      // a line's data are scaled so that its largest value lies in [2^56, 2^57)
-constexpr int SP_COEF = 60;      // coefficients are scaled so that the largest lies in [2^59.5, 2^60.5]
+constexpr int SP_COEF = 60;      // coefficients: the largest is scaled into [2^59.5, 2^60.5], or lower (mm_table)
 constexpr int SP_UNIT = 60;      // unit of the joined sums: 2^60 of data x coefficient units
 // 512 in every digit position: turns balanced digits into plain bit fields
 constexpr long long SP_BIAS = (512ll << 50) | (512ll << 40) | (512ll << 30) | (512ll << 20) | (512ll << 10) | 512ll;
